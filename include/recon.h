@@ -11,6 +11,17 @@
  * first, then queue-driven propagation. R is unique, so every schedule returns
  * the same bytes.
  *
+ * Two engines compute it. The wavefront engine is the hybrid above: one
+ * persistent launch whose scan / queue schedule the RECON_P_* settings, the
+ * autotuner, the cost model and recon_batch_ex control. The merging engine
+ * finds the same R as widest-path values, by merging regions of the mask along
+ * their best passes; its depth is logarithmic in the region count instead of
+ * the length of the propagation path, and it has no schedule. recon_run*,
+ * recon_batch* and the host-buffer calls use the merging engine while all of
+ * the context's wavefront settings (BLOCK_H, SWEEPS, GRID, BANDS, TMA,
+ * REVISIT_SCANS, SCAN_GAIN, TEST_STALL, TRACE) hold their defaults, and the
+ * wavefront engine otherwise, as recon_batch_ex with a variant or an order does.
+ *
  * Two more operations run on the same engine (recon_tile.op):
  *   reconstruction by erosion, the dual: R = lim_n eps_I^n(J),
  *     eps_I(X)(p) = max( min_{q in N(p)} X(q), I(p) ), for J >= I;
@@ -62,7 +73,7 @@ enum {
 /* Flags for recon_init. */
 #define RECON_FLAG_SYNC      0x1u  /* each call waits for the device and returns its status */
 #define RECON_FLAG_NO_CHECK  0x2u  /* skip the J <= I check (caller guarantees it) */
-#define RECON_FLAG_LEARNED   0x4u  /* recon_batch: the cost model picks variant and order */
+#define RECON_FLAG_LEARNED   0x4u  /* recon_batch on the wavefront engine: the cost model picks variant and order */
 #define RECON_FLAG_NO_GRAPH  0x8u  /* recon_batch: never capture / replay a CUDA graph */
 
 /* Operations (recon_tile.op). */
@@ -85,7 +96,9 @@ typedef struct {
 /* Creates a context on CUDA device `device`: the library's scratch for the
  * state Algorithm 1 (Sec. II-B) keeps beside the image D it updates in place --
  * the wavefront queues' overflow areas, per-block state and work list, tile
- * descriptors and status words -- plus the cost model. It owns no image data.
+ * descriptors and status words -- plus the merging engine's (about 2.7 bytes
+ * per pixel of up to 268 Mpx, or of the largest tile) and the cost model. It
+ * owns no image data.
  * `cuda_stream` is a cudaStream_t
  * (NULL: the context creates its own non-blocking stream). flags: RECON_FLAG_*.
  * The environment variables RECON_BLOCK_H, RECON_SWEEPS, RECON_BANDS,
@@ -108,7 +121,8 @@ int recon_run_op(recon_ctx *ctx, const uint8_t *I, uint8_t *J, int H, int W, int
  * (tiles are processed concurrently, as the 4K x 4K tiles of Sec. V are).
  * `tiles` is a HOST array of n descriptors with device image pointers.
  * Tiles must not overlap in memory. With RECON_FLAG_LEARNED the cost model
- * chooses each tile's variant and the packing order (never the pixel values).
+ * chooses each tile's variant and the packing order when the wavefront engine
+ * runs (never the pixel values).
  * 1 <= n <= 2^28 (RECON_EINVAL otherwise).
  * On a device error, recon_last_error_tile names the first failing tile. */
 int recon_batch(recon_ctx *ctx, const recon_tile *tiles, int n);
@@ -131,7 +145,7 @@ int recon_run_host(recon_ctx *ctx, const uint8_t *I, uint8_t *J, int H, int W, i
  * a FillHoles tile is only written. A batch of 256 Mpx or more is cut into
  * four runs of consecutive tiles with about equal pixel counts, processed as
  * a pipeline: a run's inputs are copied in one run ahead of its use, each run
- * is planned (RECON_FLAG_LEARNED) while the run before it is reconstructed
+ * is planned (RECON_FLAG_LEARNED, wavefront engine) while the run before it is reconstructed
  * and then queued behind it, and a run's results are copied back while the
  * next run is reconstructed (copies from pinned host memory overlap the
  * reconstruction). Each run's device status is checked before its results are
@@ -176,7 +190,8 @@ enum {
                                 host memory (read with recon_trace, even while running) */
     RECON_P_LAST_ABORT = 10, /* read-only: which device-side bound ran out in the last call
                                 (0 = none; 1 rerun, 2 overflow, 3 levels, 4 scans, 5 unused,
-                                6 notify, 7 unused, 8 idle wait, 9 ring push, 10 TMA) */
+                                6 notify, 7 unused, 8 idle wait, 9 ring push, 10 TMA,
+                                11 a walk of the merging engine) */
     RECON_P_REVISIT_SCANS = 11, /* scan pairs a block runs when revisited (after a neighbour
                                    raised its halo) before its queue phase; default 0 */
     RECON_P_SCAN_GAIN = 12,     /* default adaptive scan-to-queue switch: after its fixed scan
@@ -189,7 +204,10 @@ int recon_set_param(recon_ctx *ctx, int key, int64_t value);
 int64_t recon_get_param(recon_ctx *ctx, int key);
 
 /* Work counters of one tile in the last call (propagation work measured by
- * the method itself: what the cost model learns from). */
+ * the method itself: what the cost model learns from). The merging engine
+ * reports visits (blocks of 64 x 64 pixels), seeds (basins of the mask), levels
+ * (merging rounds, summed over the blocks), busy_ns and, in phase_ns: load,
+ * basins, passes, rounds, results, 0. */
 typedef struct {
     uint64_t visits;      /* block visits (first visits + revisits after a halo change) */
     uint64_t scan_rows;   /* rows processed by raster / anti-raster scans */

@@ -230,8 +230,10 @@ def init_params(rng) -> np.ndarray:
 
 
 def evaluate(ctx, model_path, workload="eval1000", reps=3):
-    """Learned vs plain schedule on one batch: device time of the persistent
-    launch, and byte equality of the two outputs."""
+    """Learned vs plain schedule of the wavefront engine on one batch: device
+    time of the persistent launch, and byte equality of the two outputs. Both
+    schedules are passed explicitly (a call without one runs on the
+    region-merging engine, which has no schedule to choose)."""
     import torch
     import synth
     w = synth.workload(workload)
@@ -253,6 +255,10 @@ def evaluate(ctx, model_path, workload="eval1000", reps=3):
     st, var, order, pred = rc.recon_sched_plan_batch(ctx, tiles)
     rc.check(st, "plan")
 
+    k, gain = rc.recon_get_param(ctx, rc.RECON_P_SWEEPS), rc.recon_get_param(ctx, rc.RECON_P_SCAN_GAIN)
+    plain_var = [k + 256 * (gain // 64) if k >= 0 else -1] * len(specs)
+    plain_order = sorted(range(len(specs)), key=lambda i: -specs[i].H * specs[i].W)
+
     def timed(fn):
         out = []
         for r in range(reps + 1):
@@ -264,7 +270,7 @@ def evaluate(ctx, model_path, workload="eval1000", reps=3):
                 out.append(rc.recon_last_kernel_ms(ctx))
         return float(np.median(out))
 
-    ms_plain = timed(lambda: rc.check(rc.recon_batch(ctx, tiles), "plain"))
+    ms_plain = timed(lambda: rc.check(rc.recon_batch_ex(ctx, tiles, plain_var, plain_order), "plain"))
     R_plain = dJ.clone()
     ms_learned = timed(lambda: rc.check(rc.recon_batch_ex(ctx, tiles, var, order), "learned"))
     same = bool(torch.equal(R_plain, dJ))

@@ -19,6 +19,7 @@
 #include "recon_sched.h"
 #include "recon_learn.h"
 #include "recon_dt.h"
+#include "recon_forest.h"
 
 extern "C" size_t rk_smem_bytes(int bh);
 extern "C" cudaError_t rk_configure(int bh, int *ctas_per_sm);
@@ -46,6 +47,11 @@ struct recon_ctx {
     rk::Ctl *d_ctl = nullptr;
     int *d_tile_err = nullptr; rk::Work *d_work = nullptr; size_t cap_tiles = 0;
     uint16_t *d_spill = nullptr; size_t cap_spill_ctas = 0;
+    // region-merging engine: status + work + tile lists (one upload), block scratch
+    unsigned char *d_fmeta = nullptr; size_t cap_fmeta = 0;
+    unsigned char *d_forest = nullptr; size_t cap_forest = 0;
+    // status and work counters of the last call (either engine's)
+    rk::Ctl *last_ctl = nullptr; rk::Work *last_work = nullptr;
     // host staging (pinned)
     unsigned char *h_meta = nullptr; size_t cap_hmeta = 0;
     cudaEvent_t meta_free = nullptr, ev0 = nullptr, ev1 = nullptr;
@@ -136,6 +142,7 @@ extern "C" int recon_init(recon_ctx **out, int device, void *cuda_stream, unsign
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev1);
     if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_ctl, sizeof(rk::Ctl));
+    if (e == cudaSuccess) e = rf_configure();
     if (e == cudaSuccess) {
         int occ = 0;
         for (int bh : {32, 64, 128, 256})
@@ -180,6 +187,8 @@ extern "C" int recon_free(recon_ctx *c)
     cudaFree(c->d_tile_err);
     cudaFree(c->d_work);
     cudaFree(c->d_spill);
+    cudaFree(c->d_fmeta);
+    cudaFree(c->d_forest);
     cudaFree(c->d_img);
     cudaFree(c->d_dt);
     cudaFree(c->d_dt_site);
@@ -351,15 +360,10 @@ static MetaLayout meta_layout(int n)
     return L;
 }
 
-// Builds the descriptor table + packing tables in the pinned staging buffer.
-// Returns bytes used, or 0 on failure.
-static int stage_meta(recon_ctx *c, const recon_tile *tiles, int n, const int *variant,
-                      const int *order, size_t *bytes, unsigned *nblocks, int *nfill)
+// Grows the pinned staging buffer to `total` bytes once the previous call's
+// copy out of it is done (its event is recorded right after that copy).
+static int ensure_stage(recon_ctx *c, size_t total)
 {
-    const MetaLayout L = meta_layout(n);
-    const size_t off_order = L.off_order, off_base = L.off_base, total = L.total;
-    // the previous call's copy out of the staging buffer must be done (its
-    // event is recorded right after that copy, not after the kernels)
     CK(cudaEventSynchronize(c->meta_free));
     if (c->cap_hmeta < total) {
         if (c->h_meta) cudaFreeHost(c->h_meta);
@@ -368,6 +372,18 @@ static int stage_meta(recon_ctx *c, const recon_tile *tiles, int n, const int *v
         CK(cudaMallocHost((void **)&c->h_meta, total));
         c->cap_hmeta = total;
     }
+    return RECON_OK;
+}
+
+// Builds the descriptor table + packing tables in the pinned staging buffer.
+// Returns bytes used, or 0 on failure.
+static int stage_meta(recon_ctx *c, const recon_tile *tiles, int n, const int *variant,
+                      const int *order, size_t *bytes, unsigned *nblocks, int *nfill)
+{
+    const MetaLayout L = meta_layout(n);
+    const size_t off_order = L.off_order, off_base = L.off_base, total = L.total;
+    int rc = ensure_stage(c, total);
+    if (rc) return rc;
     rk::TileDesc *D = (rk::TileDesc *)c->h_meta;
     int *ord = (int *)(c->h_meta + off_order);
     unsigned *base = (unsigned *)(c->h_meta + off_base);
@@ -430,6 +446,128 @@ static int stage_meta(recon_ctx *c, const recon_tile *tiles, int n, const int *v
     return RECON_OK;
 }
 
+// Whether a call without an explicit schedule runs on the region-merging
+// engine: when the context's wavefront settings are all at their defaults.
+// Setting any of them (recon_set_param, RECON_*, recon_autotune) or passing
+// variants or an order asks for the wavefront engine. The merging engine was
+// faster at every size, marker, connectivity and operation measured, by 1.03
+// (4096^2, h-dome: 405 -> 394 us) to 12 times (3000^2, border-seeded: 4.18 ->
+// 0.34 ms), so there is no size below or above which the other is chosen.
+static bool use_forest(const recon_ctx *c)
+{
+    return c->bh == 128 && c->k == 1 && c->grid == 0 && c->bands == 4 && c->use_tma == 1 && c->revisit_scans == 0 &&
+           c->scan_gain == 2048 && !c->phantom && !c->trace_on;
+}
+
+// Runs the batch on the region-merging engine: one upload (status, counters,
+// tile lists), then up to three launches per group of tiles. *done = 0 when the
+// batch does not fit that engine (nothing was launched). Launched directly, not
+// as a graph: a graph would be rebuilt whenever a call brings other buffers.
+static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, int *done)
+{
+    *done = 0;
+    struct Group { int conn, first, count; unsigned nblocks; int flat; size_t off_base; };
+    std::vector<Group> groups;
+    std::vector<int> seq;
+    seq.reserve(n);
+    int nfill = 0;
+    for (int conn : {8, 4})
+        for (int t = 0; t < n; ++t)
+            if (tiles[t].conn == conn) seq.push_back(t);
+    for (int t = 0; t < n; ++t) nfill += tiles[t].op == RECON_OP_FILL_HOLES;
+    if (nfill > 65535) return RECON_EINVAL;
+    unsigned most = 0;
+    for (int i = 0; i < n; ++i) {
+        const recon_tile &T = tiles[seq[i]];
+        const unsigned long long nbx = ((unsigned long long)T.W + rf::BS - 1) / rf::BS;
+        const unsigned long long nby = ((unsigned long long)T.H + rf::BS - 1) / rf::BS;
+        if (nbx * nby > rf::MAX_BLOCKS) return RECON_OK;
+        const unsigned nb = (unsigned)(nbx * nby);
+        if (groups.empty() || groups.back().conn != T.conn || groups.back().nblocks + nb > rf::MAX_GROUP_BLOCKS)
+            groups.push_back(Group{T.conn, i, 0, 0u, 1, 0});
+        Group &g = groups.back();
+        g.count += 1;
+        g.nblocks += nb;
+        g.flat &= nb == 1;
+        most = std::max(most, g.nblocks);
+    }
+    // one buffer, uploaded whole: status | tile status | counters | tiles | block counts
+    const size_t off_err = align_up(sizeof(rk::Ctl), 16);
+    const size_t off_work = align_up(off_err + sizeof(int) * (size_t)n, 16);
+    const size_t off_tiles = align_up(off_work + sizeof(rk::Work) * (size_t)n, 16);
+    size_t total = align_up(off_tiles + sizeof(rf::Tile) * (size_t)n, 16);
+    for (Group &g : groups) {
+        g.off_base = total;
+        total += align_up(sizeof(unsigned) * ((size_t)g.count + 1), 16);
+    }
+    const size_t need = rf::scratch_bytes(most);
+    int rc;
+    if (c->cap_fmeta < total || c->cap_forest < need) {
+        CK(cudaStreamSynchronize(c->stream));
+        if (c->last_ctl == (rk::Ctl *)c->d_fmeta) c->launched = 0;   // that call's status goes with the buffer
+        if ((rc = grow(&c->d_fmeta, &c->cap_fmeta, total))) return rc;
+        rc = grow(&c->d_forest, &c->cap_forest, need);
+        if (rc == RECON_ENOMEM) return RECON_OK;   // the wavefront engine needs far less scratch
+        if (rc) return rc;
+    }
+    if ((rc = ensure_stage(c, total))) return rc;
+    unsigned char *h = c->h_meta;
+    memset(h, 0, off_tiles);
+    ((rk::Ctl *)h)->err_tile = INT_MAX;
+    rf::Tile *ft = (rf::Tile *)(h + off_tiles);
+    for (const Group &g : groups) {
+        unsigned *base = (unsigned *)(h + g.off_base), acc = 0;
+        for (int i = 0; i < g.count; ++i) {
+            const int t = seq[g.first + i];
+            const recon_tile &T = tiles[t];
+            rf::Tile d;
+            memset(&d, 0, sizeof(d));
+            d.I = T.I; d.J = T.J; d.H = T.H; d.W = T.W; d.pitch = T.pitch;
+            d.nbx = (T.W - 1) / rf::BS + 1;
+            d.nby = (T.H - 1) / rf::BS + 1;
+            d.dual = T.op != RECON_OP_DILATE ? 1 : 0;
+            d.fill = T.op == RECON_OP_FILL_HOLES ? 1 : 0;
+            d.index = t;
+            ft[g.first + i] = d;
+            base[i] = acc;
+            acc += (unsigned)(d.nbx * d.nby);
+        }
+        base[g.count] = acc;
+    }
+    *done = 1;
+    c->last_n = n;
+    c->last_err_tile = -1;
+    c->host_status = 0;
+    c->last_ctl = (rk::Ctl *)c->d_fmeta;
+    c->last_work = (rk::Work *)(c->d_fmeta + off_work);
+    CK(cudaMemcpyAsync(c->d_fmeta, h, total, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaEventRecord(c->meta_free, c->stream));
+    CK(cudaEventRecord(c->ev0, c->stream));
+    for (const Group &g : groups) {
+        rf::Params P;
+        memset(&P, 0, sizeof(P));
+        P.tiles = (const rf::Tile *)(c->d_fmeta + off_tiles) + g.first;
+        P.base = (const unsigned *)(c->d_fmeta + g.off_base);
+        P.ntiles = g.count;
+        P.nblocks = g.nblocks;
+        const size_t nb = g.nblocks;
+        P.px = (uint16_t *)c->d_forest;
+        P.link = (unsigned long long *)(P.px + nb * rf::BPX);
+        P.rim = (uint16_t *)(P.link + nb * rf::MAX_TERM);
+        P.nterm = (unsigned *)(P.rim + nb * 4 * rf::BS);
+        P.ctl = c->last_ctl;
+        P.tile_err = (int *)(c->d_fmeta + off_err);
+        P.work = c->last_work;
+        P.check = (c->flags & RECON_FLAG_NO_CHECK) ? 0 : 1;
+        P.flat = g.flat;
+        CK(rf_launch(g.conn, &P, c->stream));
+    }
+    CK(cudaEventRecord(c->ev1, c->stream));
+    c->launched = 1;
+    if (c->flags & RECON_FLAG_SYNC) return recon_sync(c);
+    return RECON_OK;
+}
+
 static int batch_impl(recon_ctx *c, const recon_tile *tiles, int n, const int *variant, const int *order)
 {
     if (!c || !tiles || n < 1 || n > rk::MAX_TILES) return RECON_EINVAL;
@@ -440,6 +578,18 @@ static int batch_impl(recon_ctx *c, const recon_tile *tiles, int n, const int *v
             if (variant[t] < -1 || (variant[t] >= 0 && ((variant[t] & 0xFF) > 64 || (variant[t] >> 8) > 4096)))
                 return RECON_EINVAL;
     CK(cudaSetDevice(c->device));
+
+    if (!variant && !order && use_forest(c)) {
+        if (!(c->flags & RECON_FLAG_NO_GRAPH)) {
+            // a stream the caller is capturing is refused, as the graph path below refuses it
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            CK(cudaStreamIsCapturing(c->stream, &cap));
+            if (cap != cudaStreamCaptureStatusNone) return RECON_ECUDA;
+        }
+        int done = 0;
+        const int frc = forest_batch(c, tiles, n, &done);
+        if (done || frc != RECON_OK) return frc;
+    }
 
     std::vector<int> lv, lo;
     if ((c->flags & RECON_FLAG_LEARNED) && !variant && !order && c->sched) {
@@ -546,6 +696,8 @@ static int batch_impl(recon_ctx *c, const recon_tile *tiles, int n, const int *v
     c->last_n = n;
     c->last_err_tile = -1;
     c->host_status = 0;
+    c->last_ctl = c->d_ctl;
+    c->last_work = c->d_work;
     const bool use_graph = !(c->flags & RECON_FLAG_NO_GRAPH);
     if (use_graph && c->gexec && sig == c->gsig) {
         // the graph records meta_free itself, right after its descriptor copy
@@ -614,7 +766,7 @@ extern "C" int recon_sync(recon_ctx *c)
     if (!c->launched) return RECON_OK;
     if (!c->host_status) {   // a host batch records its own status (its segments share the control word)
         rk::Ctl h;
-        CK(cudaMemcpy(&h, c->d_ctl, sizeof(h), cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(&h, c->last_ctl, sizeof(h), cudaMemcpyDeviceToHost));
         c->last_err_tile = (h.err_tile == INT_MAX) ? -1 : h.err_tile;
         c->last_abort = h.abort;
     }
@@ -637,7 +789,7 @@ extern "C" int recon_get_work(recon_ctx *c, recon_work *out, int n)
     CK(cudaStreamSynchronize(c->stream));
     if (n == 0) return RECON_OK;
     std::vector<rk::Work> w(n);
-    CK(cudaMemcpy(w.data(), c->d_work, sizeof(rk::Work) * n, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(w.data(), c->last_work, sizeof(rk::Work) * n, cudaMemcpyDeviceToHost));
     for (int i = 0; i < n; ++i) {
         out[i].visits = w[i].visits;
         out[i].scan_rows = w[i].scan_rows;
@@ -750,7 +902,7 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
         const int t0 = first(s), ns = seg_end[s] - t0;
         std::vector<int> lv, lo;
         const int *var = nullptr, *ord = nullptr;
-        if ((fl & RECON_FLAG_LEARNED) && c->sched && recon_sched_has_model(c->sched)) {
+        if ((fl & RECON_FLAG_LEARNED) && !use_forest(c) && c->sched && recon_sched_has_model(c->sched)) {
             CK(cudaStreamWaitEvent(c->s_plan, c->ev_in[s], 0));
             const int prc = recon_sched_plan(c->sched, dt.data() + t0, ns, c->sms, c->s_plan, &lv, &lo);
             if (prc != RECON_OK) return prc;
@@ -760,7 +912,7 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
         CK(cudaStreamWaitEvent(c->stream, c->ev_in[s], 0));
         const int brc = batch_impl(c, dt.data() + t0, ns, var, ord);
         if (brc != RECON_OK) return brc;
-        CK(cudaMemcpyAsync(&c->h_seg_ctl[s], c->d_ctl, sizeof(rk::Ctl), cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaMemcpyAsync(&c->h_seg_ctl[s], c->last_ctl, sizeof(rk::Ctl), cudaMemcpyDeviceToHost, c->stream));
         CK(cudaEventRecord(c->ev_out[s], c->stream));
         return RECON_OK;
     };

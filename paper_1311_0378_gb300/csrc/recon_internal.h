@@ -83,7 +83,7 @@ struct Params {
 // where-codes recorded in Ctl::abort when a bound runs out
 enum {
     AB_RERUN = 1, AB_OVERFLOW = 2, AB_LEVELS = 3, AB_SCANS = 4, /* 5: unused */ AB_NOTIFY = 6,
-    /* 7: unused */ AB_IDLE = 8, AB_PUSH = 9, AB_TMA = 10
+    /* 7: unused */ AB_IDLE = 8, AB_PUSH = 9, AB_TMA = 10, AB_MERGE = 11
 };
 
 }  // namespace rk
