@@ -29,10 +29,15 @@
 // every link goes to a node of higher (hashed) priority: no cycles in any
 // interleaving, and walks of logarithmic expected length.
 //
-// Measured on GB300 (whole call, the wavefront engine before -> this one): a
-// 4096^2 tile seeded from its border, 4-connected, 5.61 -> 0.61 ms; with an
-// h-dome marker, 8-connected, 0.405 -> 0.394 ms; 200 tiles of 256 .. 4096
-// pixels a side (910 Mpx, both markers) 60.4 -> 19.4 ms; 512^2 0.230 -> 0.121 ms.
+// Measured on GB300 (whole call, the wavefront engine -> this one): a 4096^2
+// tile seeded from its border, 4-connected, 5.74 -> 0.457 ms; with an h-dome
+// marker, 8-connected, 0.402 -> 0.323 ms; 200 tiles of 256 .. 4096 pixels a
+// side (910 Mpx, both markers) 54.4 -> 15.3 ms; 512^2 0.235 -> 0.098 ms.
+// block_kernel takes most of it (0.33 of 0.40 ms of kernel time on the
+// border-seeded tile) and is bound by instruction issue (66% of the issue slots,
+// 49% of the shared-memory pipe; DRAM below 10%), so what counts is instructions
+// per pixel: saddles instead of all pixel pairs cut its time from 0.71 to 0.46 ms,
+// and code small enough for the instruction cache (rolled loops) to 0.33.
 #include <climits>
 #include "recon_forest.h"
 
@@ -40,15 +45,17 @@ namespace rf {
 
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int NT = 256;            // threads per CTA: one 16-pixel run each
-// Shared-memory image: row stride ST, pixel (x, y) at (y + 1) * ST + X0 + x.
+// Shared-memory label image: row stride ST, pixel (x, y) at (y + 1) * ST + X0 + x.
 // The cell right of a row's last pixel is the first cell of the next row.
-constexpr int ST = BS + 4, X0 = 4;
-constexpr int NCELL = (BS + 2) * ST + 4;
+constexpr int ST = BS + 8, X0 = 8;
+constexpr int NCELL = (BS + 2) * ST + 8;
 constexpr int IST = 20;            // row stride of the byte image in words (interior at word 4)
-constexpr int TAB = 2560;          // passes a block can list
+constexpr int JOFF = (BS + 2) * IST + 4, IMG = JOFF + BPX / 4;   // where J's bytes start, words in all
+constexpr int TAB = 2048;          // passes a block can list (noise has about 1150)
 constexpr unsigned ROOT = 0x8000u; // label flag: a basin number, not a pointer to a cell
-constexpr unsigned DONE = 0xFFFFFFFFu;
-constexpr unsigned K_SOURCE = 2u << 22, K_EDGE = 1u << 22;   // edge kinds, heavier wins a tie
+constexpr unsigned FINAL = 0xFFFFFFFEu, NODE = 0xFFFFFFFFu;   // best[] of a region that stopped
+// edge kinds of a region's heaviest edge (weight << 24 | kind | number): the larger wins a tie
+constexpr unsigned K_SOURCE = 2u << 22, K_EDGE = 1u << 22, K_OUT = 0u;
 constexpr unsigned SRC = 0xFFFFFFFFu;   // parent number of the source
 constexpr unsigned RES = 255u;          // node slot of a pixel whose value is final
 constexpr int MAX_STEPS = 1 << 20;      // bound of every walk
@@ -58,16 +65,16 @@ constexpr int MAX_STEPS = 1 << 20;      // bound of every walk
 template <int CONN>
 struct Smem {
     static constexpr int NB = (CONN == 8 ? BPX / 4 : BPX / 2) + 32;
-    alignas(16) uint32_t W[NCELL];    // I << 24 | label
-    alignas(16) uint32_t tab[TAB];    // passes: basin << 20 | basin << 8 | weight; before that the byte images
-    uint32_t best[NB];                // heaviest edge of a region this round; then cap << 8 | node slot
-    uint32_t sj[NB], cb[NB];          // heaviest edge to the source / out of the block
-    uint16_t comp[NB], up[NB];        // region's root, link to the region merged into
-    uint8_t capw[NB], st[NB];         // weight of that link; 1 = node, 2 = final (then the node slot)
+    alignas(16) uint16_t L[NCELL];    // labels: a cell number, or ROOT | basin
+    alignas(16) uint32_t img[IMG];    // byte image of I, then the bytes of J
+    uint32_t tab[TAB];                // saddles, then passes: region << 20 | region << 8 | weight, 0 = none
+    uint32_t best[NB];                // heaviest edge of a live region to a region or out of the block; FINAL, NODE
+    uint32_t sv[NB];                  // its heaviest source edge
+    uint16_t comp[NB], up[NB];        // region's root (at the end cap << 8 | node slot), link to the region merged into
+    uint8_t capw[NB];                 // weight of the up link; a final root's value; a node root's slot
     uint32_t link[MAX_TERM];          // node links: weight << 8 | parent slot (RES = source)
-    uint32_t ss[MAX_TERM];
     uint8_t hT[BS + 2], hB[BS + 2], hL[BS], hR[BS];   // mask of the pixels around the block
-    unsigned nb, nt, ne;              // basins, nodes, passes
+    unsigned nb, nt, nsad, nmore;     // basins, nodes, saddles, passes beyond one per saddle
     int tile;
     unsigned local;
 };
@@ -104,18 +111,15 @@ __device__ __forceinline__ int find_tile(const Params &P, unsigned b)
     return lo;
 }
 
-// 16 pixels of an image row from column x on, zero right of column W. Any
-// alignment: aligned words around the run, shifted; a word is only read when
-// it holds a pixel of the run.
-__device__ __forceinline__ uint4 load16(const uint8_t *row, int x, int W, bool vec)
+// 16 pixels of an image row from column x on, zero right of column W (n = W - x
+// pixels are inside). Any alignment: aligned words around the run, shifted; a
+// word is only read when it holds a pixel of the run.
+__device__ __noinline__ uint4 load16_any(const uint8_t *at, int n)
 {
-    const int n = W - x;
-    if (vec && n >= 16) return *(const uint4 *)(row + x);
     uint32_t w[5] = {0u, 0u, 0u, 0u, 0u};
     if (n > 0) {
-        const uintptr_t a = (uintptr_t)(row + x);
-        const int s = (int)(a & 3);
-        const uint32_t *q = (const uint32_t *)(a - s);
+        const int s = (int)((uintptr_t)at & 3);
+        const uint32_t *q = (const uint32_t *)(at - s);
 #pragma unroll
         for (int j = 0; j < 5; ++j)
             if (4 * j - s < min(n, 16)) w[j] = q[j];
@@ -129,33 +133,41 @@ __device__ __forceinline__ uint4 load16(const uint8_t *row, int x, int W, bool v
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+__device__ __forceinline__ uint4 load16(const uint8_t *at, int n, bool vec)
+{
+    if (vec && n >= 16) return *(const uint4 *)at;
+    return load16_any(at, n);
+}
+
 __device__ __forceinline__ uint32_t inside(int n)   // byte mask of the first n pixels of a word
 {
     return n >= 4 ? 0xFFFFFFFFu : (n > 0 ? 0xFFFFFFFFu >> (8 * (4 - n)) : 0u);
 }
 
-__device__ __forceinline__ void store16(uint8_t *row, int x, int W, uint4 v, bool vec)
+// The first n of 16 pixels to any address: whole words inside, bytes at the ends.
+__device__ __noinline__ void store16_any(uint8_t *at, int n, uint4 v)
 {
-    const int n = min(W - x, 16);
-    if (vec && n == 16) {
-        *(uint4 *)(row + x) = v;
-        return;
-    }
-    if (n <= 0) return;
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    if ((((uintptr_t)(row + x)) & 3) == 0) {
+    n = min(n, 16);
+    const int lead = (int)(-(intptr_t)at & 3);   // bytes before the first aligned word
+    const uint32_t w[5] = {v.x, v.y, v.z, v.w, 0u};
+    if (lead < n)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (4 * j + 3 < n) *(uint32_t *)(row + x + 4 * j) = w[j];
-            else
-                for (int b = 0; b < 4; ++b)
-                    if (4 * j + b < n) row[x + 4 * j + b] = (uint8_t)(w[j] >> (8 * b));
-        }
-        return;
+        for (int j = 0; j < 4; ++j)
+            if (lead + 4 * j + 4 <= n) *(uint32_t *)(at + lead + 4 * j) = __funnelshift_r(w[j], w[j + 1], 8 * lead);
+    const int done = lead < n ? lead + (n - lead) / 4 * 4 : 0;   // words cover lead .. done - 1
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+        if (lead < n && i == lead) i = done;
+        if (i >= n) break;
+        const uint32_t q = i < 8 ? (i < 4 ? v.x : v.y) : (i < 12 ? v.z : v.w);
+        at[i] = (uint8_t)(q >> (8 * (i & 3)));
     }
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-        if (j < n) row[x + j] = (uint8_t)(w[j >> 2] >> (8 * (j & 3)));
+}
+
+__device__ __forceinline__ void store16(uint8_t *at, int n, uint4 v, bool vec)
+{
+    if (vec && n >= 16) *(uint4 *)at = v;
+    else if (n > 0) store16_any(at, n, v);
 }
 
 // Cell offset of direction d (0..7: NW, N, NE, W, E, SW, S, SE, in the order
@@ -299,49 +311,29 @@ struct GlobalLinks {
     __device__ bool before(unsigned a, unsigned b) const { return priority(a) < priority(b); }
 };
 
-// Every pass between two basins, f(a, b, w, number): the list's entries, or
-// (when there are too many for it) every pair of neighbouring pixels.
+// A block with more passes than its list holds works on every pair of
+// neighbouring pixels instead: pair i is pixel i / 4 and its E, SW, S or SE
+// neighbour.
 template <int CONN, class F>
-__device__ __forceinline__ void each_pass(Smem<CONN> &S, F f)
+__device__ __noinline__ void each_pair(Smem<CONN> &S, F f)
 {
-    if (S.ne <= TAB) {
-        for (unsigned i = threadIdx.x; i < S.ne; i += NT) {
-            const uint32_t e = S.tab[i];
-            f(e >> 20, (e >> 8) & 0xFFFu, e & 255u, i);
-        }
-    } else {
-        for (unsigned i = threadIdx.x; i < BPX * 4; i += NT) {
-            const unsigned px = i >> 2, d = i & 3u;
-            if (CONN == 4 && (d & 1u)) continue;
-            const unsigned p = (px / BS + 1) * ST + X0 + px % BS;
-            const uint32_t a = S.W[p], b = S.W[p + dir_off(4u + d)];
-            const unsigned w = min(a >> 24, b >> 24);
-            if (w && ((a ^ b) & 0xFFFFu)) f(a & 0x7FFFu, b & 0x7FFFu, w, i);
-        }
-    }
-}
-
-// The two basins of pass number i.
-template <int CONN>
-__device__ __forceinline__ void pass_ends(const Smem<CONN> &S, unsigned i, unsigned &a, unsigned &b)
-{
-    if (S.ne <= TAB) {
-        const uint32_t e = S.tab[i];
-        a = e >> 20;
-        b = (e >> 8) & 0xFFFu;
-    } else {
-        const unsigned px = i >> 2, p = (px / BS + 1) * ST + X0 + px % BS;
-        a = S.W[p] & 0x7FFFu;
-        b = S.W[p + dir_off(4u + (i & 3u))] & 0x7FFFu;
+    const uint8_t *img = (const uint8_t *)S.img;
+    for (unsigned i = threadIdx.x; i < BPX * 4; i += NT) {
+        const unsigned px = i >> 2, d = i & 3u;
+        if (CONN == 4 && (d & 1u)) continue;
+        const int py = (int)(px / BS), qx = (int)(px % BS);
+        const int dx = d == 0 ? 1 : (int)d - 2, dy = d != 0;
+        const unsigned a = S.L[(py + 1) * ST + X0 + qx], b = S.L[(py + dy + 1) * ST + X0 + qx + dx];
+        const unsigned w = min(img[(py + 1) * IST * 4 + 16 + qx], img[(py + dy + 1) * IST * 4 + 16 + qx + dx]);
+        if (w && a != b) f(a & 0x7FFFu, b & 0x7FFFu, w, i);
     }
 }
 
 template <int CONN>
-__global__ void __launch_bounds__(NT, CONN == 8 ? 4 : 3) block_kernel(Params P)
+__global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Smem<CONN> &S = *reinterpret_cast<Smem<CONN> *>(smem_raw);
-    constexpr int NB = Smem<CONN>::NB;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned blk = blockIdx.x;
     unsigned long long tick[6];   // thread 0: start and end of the phases (recon_work.phase_ns)
@@ -353,7 +345,8 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 4 : 3) block_kernel(Params P)
             S.local = blk - P.base[t];
             S.nb = 1;
             S.nt = 0;
-            S.ne = 0;
+            S.nsad = 0;
+            S.nmore = 0;
         }
     }
     __syncthreads();
@@ -363,15 +356,16 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 4 : 3) block_kernel(Params P)
     const bool vec = (D.pitch % 16) == 0 && ((uintptr_t)D.I % 16) == 0 && ((uintptr_t)D.J % 16) == 0;
     const int r = tid >> 2, c = tid & 3;         // this thread's run: row r, columns 16c .. 16c + 15
     const int y = y0 + r, x = x0 + 16 * c;
-    uint32_t *const bi = S.tab;                  // byte image of I: rows -1 .. 64, IST words each
-    uint32_t *const bj = S.tab + (BS + 2) * IST + 4;   // bytes of J: 64 rows of 16 words
-    uint4 vi = make_uint4(0, 0, 0, 0), vj = vi;
+    uint32_t *const bi = S.img;                  // I: rows -1 .. 64, IST words each, 0 around the block
+    uint32_t *const bj = S.img + JOFF;           // J: 64 rows of 16 words
     {
+        uint4 vi = make_uint4(0, 0, 0, 0), vj = vi;
         if (y < D.H) {
-            vi = load16(D.I + (size_t)y * D.pitch, x, D.W, vec);
-            if (!D.fill) vj = load16(D.J + (size_t)y * D.pitch, x, D.W, vec);
+            vi = load16(D.I + (size_t)y * D.pitch + x, D.W - x, vec);
+            if (!D.fill) vj = load16(D.J + (size_t)y * D.pitch + x, D.W - x, vec);
         }
         // the mask around the block: 66 pixels above, 66 below, 64 left, 64 right
+        #pragma unroll 1
         for (int i = tid; i < 2 * (BS + 2) + 2 * BS; i += NT) {
             int yy, xx;
             uint8_t *h;
@@ -409,7 +403,6 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 4 : 3) block_kernel(Params P)
             }
         }
         *(uint4 *)&bi[(r + 1) * IST + 4 + 4 * c] = vi;
-        *(uint4 *)&bj[r * (BS / 4) + 4 * c] = vj;
         if (tid < IST) bi[tid] = 0u;                                   // row above
         else if (tid < 2 * IST) bi[(BS + 1) * IST + tid - IST] = 0u;   // row below
         else if (tid >= 64 && tid < 64 + BS + 3) {                     // words left of row q and right of row q - 1
@@ -417,14 +410,14 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 4 : 3) block_kernel(Params P)
             if (q < BS + 2) bi[q * IST + 3] = 0u;
             if (q) bi[q * IST] = 0u;
         }
-        if (tid < ST + 4) S.W[tid] = ROOT;                             // cells around the block: basin 0
-        else if (tid < 2 * (ST + 4)) S.W[(BS + 1) * ST + tid - (ST + 4)] = ROOT;
+        *(uint4 *)&bj[r * (BS / 4) + 4 * c] = vj;
+        if (tid < ST + 8) S.L[tid] = ROOT;                             // cells around the block: basin 0
+        else if (tid < 2 * (ST + 8)) S.L[(BS + 1) * ST + tid - (ST + 8)] = ROOT;
         if (tid < BS) {
-            S.W[(tid + 1) * ST + X0 - 1] = ROOT;
-            S.W[(tid + 2) * ST] = ROOT;
+            S.L[(tid + 1) * ST + X0 - 1] = ROOT;
+            S.L[(tid + 2) * ST] = ROOT;
         }
-        for (int i = tid; i < NB; i += NT) S.cb[i] = 0u;
-        if (tid == 0) S.sj[0] = 0u;
+        if (tid == 0) { S.sv[0] = 0u; S.best[0] = 0u; }
         bool bad = false;
         if (P.check && !D.fill)
             bad = (__vcmpgtu4(vj.x, vi.x) | __vcmpgtu4(vj.y, vi.y) | __vcmpgtu4(vj.z, vi.z) | __vcmpgtu4(vj.w, vi.w)) != 0;
@@ -441,221 +434,301 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 4 : 3) block_kernel(Params P)
     if (tid == 0) tick[1] = now_ns();
     // Basins: every pixel points to its highest neighbour (the later one of
     // equals), if that one is higher or equal and later; the others are tops.
-    uint32_t saddle[4];   // this thread's saddles: a byte per pixel
-    {
-        uint32_t rows[3][6];
+    // A warp takes two rows at a time, a lane one word of four pixels (a loop,
+    // not unrolled: this kernel is bound by instruction fetch before anything else).
+#pragma unroll 1
+    for (int it = 0; it < BS / 2; it += NT / 32) {
+        const int row = 2 * (it + warp) + (lane >> 4), cw = lane & 15;
+        const uint32_t *at = &bi[(row + 1) * IST + 4 + cw];
+        const uint32_t l[3] = {at[-IST - 1], at[-1], at[IST - 1]};
+        const uint32_t m[3] = {at[-IST], at[0], at[IST]};
+        const uint32_t q[3] = {at[-IST + 1], at[1], at[IST + 1]};
+        uint32_t kE, kO;
+        const uint32_t saddle = classify<CONN>(l, m, q, kE, kO);
+        const uint32_t k4[4] = {kE & 0xFFFFu, kO & 0xFFFFu, kE >> 16, kO >> 16};
+        const int cell = (row + 1) * ST + X0 + 4 * cw;
+        uint32_t f[4], arcs[4];
+        unsigned top[4], mine = 0;   // tops in the low half, saddles in the high half
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const uint32_t *row = &bi[(r + a) * IST + 4 + 4 * c];
-            const uint4 v = *(const uint4 *)row;
-            rows[a][0] = row[-1];
-            rows[a][1] = v.x; rows[a][2] = v.y; rows[a][3] = v.z; rows[a][4] = v.w;
-            rows[a][5] = row[4];
+        for (int b = 0; b < 4; ++b) {
+            const uint32_t v = (m[1] >> (8 * b)) & 255u;
+            // height 0 has value 0, like the outside (basin 0)
+            f[b] = v ? (uint32_t)(cell + b + dir_off(k4[b] & 7u)) : ROOT;
+            top[b] = v && k4[b] < (v << 3 | 4u);
+            arcs[b] = v ? (saddle >> (8 * b)) & 255u : 0u;
+            mine += top[b] | (arcs[b] ? 0x10000u : 0u);
         }
-        uint32_t lab[16];
-        unsigned tops = 0;
-        const int cell = (r + 1) * ST + X0 + 16 * c;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t l[3] = {rows[0][j], rows[1][j], rows[2][j]};
-            const uint32_t m[3] = {rows[0][j + 1], rows[1][j + 1], rows[2][j + 1]};
-            const uint32_t q[3] = {rows[0][j + 2], rows[1][j + 2], rows[2][j + 2]};
-            uint32_t kE, kO;
-            saddle[j] = classify<CONN>(l, m, q, kE, kO);
-            const uint32_t k4[4] = {kE & 0xFFFFu, kO & 0xFFFFu, kE >> 16, kO >> 16};
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const uint32_t v = (m[1] >> (8 * b)) & 255u;
-                const bool top = k4[b] < (v << 3 | 4u);
-                lab[4 * j + b] = v << 24 | (uint32_t)(cell + 4 * j + b + dir_off(k4[b] & 7u));
-                tops |= (top ? 1u : 0u) << (4 * j + b);
-            }
-        }
-        const unsigned mine = __popc(tops);
         unsigned incl = mine;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const unsigned o = __shfl_up_sync(FULL, incl, d);
             if (lane >= d) incl += o;
         }
-        unsigned at = 0;
-        if (lane == 31) at = atomicAdd(&S.nb, incl);
-        at = __shfl_sync(FULL, at, 31) + incl - mine;
-        const uint32_t jw[4] = {vj.x, vj.y, vj.z, vj.w};
+        unsigned id = 0, slot = 0;
+        if (lane == 31) {
+            id = atomicAdd(&S.nb, incl & 0xFFFFu);
+            slot = atomicAdd(&S.nsad, incl >> 16);
+        }
+        id = __shfl_sync(FULL, id, 31) + ((incl - mine) & 0xFFFFu);
+        slot = __shfl_sync(FULL, slot, 31) + ((incl - mine) >> 16);
+        const uint32_t jw = bj[row * (BS / 4) + cw];
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-            if ((tops >> j) & 1u) {
-                S.sj[at] = (jw[j >> 2] >> (8 * (j & 3))) & 255u;   // the top's own source edge
-                lab[j] = (lab[j] & 0xFF000000u) | ROOT | at++;
+        for (int b = 0; b < 4; ++b) {
+            if (top[b]) {
+                S.sv[id] = (jw >> (8 * b)) & 255u;   // the top's own source edge
+                S.best[id] = 0u;
+                f[b] = ROOT | id++;
             }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            *(uint4 *)&S.W[cell + 4 * j] = make_uint4(lab[4 * j], lab[4 * j + 1], lab[4 * j + 2], lab[4 * j + 3]);
+            // a saddle: weight << 24 | cell << 11 | direction of the highest neighbour << 8 | arc starts
+            if (arcs[b]) {
+                if (slot < TAB) S.tab[slot] = (m[1] >> (8 * b)) << 24 | (uint32_t)(cell + b) << 11 | (k4[b] & 7u) << 8 | arcs[b];
+                ++slot;
+            }
+        }
+        *(uint2 *)&S.L[cell] = make_uint2(f[0] | f[1] << 16, f[2] | f[3] << 16);
     }
     __syncthreads();
     const unsigned nb = S.nb;
-    // Every pixel's basin, and the heaviest source edge of each basin.
-    const int col = (warp & 1) * 32 + lane, row0 = (warp >> 1) * 16;   // pixel passes: 32 columns x 16 rows a warp
+    // Every pixel's basin, and the heaviest source edge of each basin. A pixel
+    // takes its target's label until that is a basin; all warps do so at once,
+    // so paths halve as they are walked (each step goes to a higher (value,
+    // number), so they end). 16 pixels a thread, their loads in flight together.
     {
-        volatile uint32_t *W = S.W;
-        const uint8_t *jb = (const uint8_t *)bj;
-        for (int i = 0; i < 16; ++i) {
-            const int p = (row0 + i + 1) * ST + X0 + col;
-            const uint32_t w = W[p];
-            unsigned l = w & 0xFFFFu;
-            if (!(l & ROOT)) {
-                do l = W[l] & 0xFFFFu; while (!(l & ROOT));   // ends: each step goes to a higher (value, number)
-                W[p] = (w & 0xFF000000u) | l;
-            }
-            const unsigned j = jb[(row0 + i) * BS + col], b = l & 0x7FFFu;
-            if (j > *(volatile uint32_t *)&S.sj[b]) atomicMax(&S.sj[b], j);
-        }
-    }
-    __syncthreads();
-    // the heaviest edge out of the block of each basin; the passes take the byte images' place
-    for (int i = tid; i < 4 * BS; i += NT) {
-        const int side = i / BS, k = i % BS;
-        int p;
-        unsigned m;
-        if (side < 2) {
-            p = (side ? BS : 1) * ST + X0 + k;
-            const uint8_t *h = side ? S.hB : S.hT;
-            m = h[k + 1];
-            if (CONN == 8) m = max(m, max((unsigned)h[k], (unsigned)h[k + 2]));
-        } else {
-            p = (k + 1) * ST + X0 + (side == 2 ? 0 : BS - 1);
-            const uint8_t *h = side == 2 ? S.hL : S.hR;
-            m = h[k];
-            if (CONN == 8) {   // (the corners' diagonal pixels belong to the top and bottom lines)
-                if (k > 0) m = max(m, (unsigned)h[k - 1]);
-                if (k < BS - 1) m = max(m, (unsigned)h[k + 1]);
+        const int p0 = ((warp >> 1) * 16 + 1) * ST + X0 + (warp & 1) * 32 + lane;   // 32 columns x 16 rows a warp
+        volatile uint16_t *L = S.L;
+        const uint8_t *jb = (const uint8_t *)bj + (warp >> 1) * 16 * BS + (warp & 1) * 32 + lane;
+        unsigned l[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) l[i] = L[p0 + i * ST];
+        bool more = true;
+        while (more) {
+            unsigned n[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) n[i] = (l[i] & ROOT) ? l[i] : L[l[i]];
+            more = false;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                if (n[i] != l[i]) L[p0 + i * ST] = (uint16_t)n[i];
+                l[i] = n[i];
+                more |= !(n[i] & ROOT);
             }
         }
-        const uint32_t w = S.W[p];
-        m = min(m, w >> 24);
-        if (m) atomicMax(&S.cb[w & 0x7FFFu], m);
-    }
-    for (unsigned b = tid; b < nb; b += NT) {
-        S.comp[b] = (uint16_t)b;
-        S.up[b] = (uint16_t)b;
-        S.capw[b] = 255;
-        S.st[b] = 0;
+        unsigned over = 0;   // pixels with a heavier source edge than their basin has so far
+#pragma unroll
+        for (int i = 0; i < 16; ++i) over |= (jb[i * BS] > S.sv[l[i] & 0x7FFFu] ? 1u : 0u) << i;
+#pragma unroll 1
+        for (; over; over &= over - 1) {
+            const int i = __ffs(over) - 1;
+            atomicMax(&S.sv[S.L[p0 + i * ST] & 0x7FFFu], (uint32_t)jb[i * BS]);
+        }
     }
     __syncthreads();
     if (tid == 0) tick[2] = now_ns();
-    // Passes: a saddle joins its own basin to the one each arc starts in, at
-    // its own height (weight 0 never beats a source edge and is left out).
-    {
-        const int cell = (r + 1) * ST + X0 + 16 * c;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            for (uint32_t bits = saddle[j]; bits; bits &= bits - 1) {
-                const unsigned b = __ffs(bits) - 1;
-                const int p = cell + 4 * j + (int)(b >> 3);
-                const uint32_t w = S.W[p], q = S.W[p + ring_off(b & 7u)];
-                if (((w ^ q) & 0xFFFFu) && w >> 24) {
-                    const unsigned at = atomicAdd(&S.ne, 1u);
-                    if (at < TAB) S.tab[at] = (w & 0x7FFFu) << 20 | (q & 0x7FFFu) << 8 | w >> 24;
+    auto offer = [&](unsigned a, uint32_t key) {
+        if (key > *(volatile uint32_t *)&S.best[a]) atomicMax(&S.best[a], key);
+    };
+    // Passes: a saddle joins its own basin to the one each arc starts in. The
+    // arc of its highest neighbour needs none (that is its own basin): with the
+    // ring turned so that this neighbour comes last, its arc's start is the
+    // last one set. A pass no heavier than the source edges of both ends is
+    // never taken. A saddle's first pass takes the saddle's place in the list,
+    // further ones follow behind. The first round's maxima are taken here too.
+    const unsigned nsad = S.nsad;
+    if (nsad <= TAB) {
+#pragma unroll 1
+        for (unsigned i = tid; i < nsad; i += NT) {
+            const uint32_t e = S.tab[i], p = (e >> 11) & 0x1FFFu, w = e >> 24;
+            const unsigned turn = ((0x34526107u >> (4 * ((e >> 8) & 7u))) & 7u) + 1u;   // that neighbour's ring position + 1
+            uint32_t arcs = e & 255u, first = 0u;
+            arcs &= ~(1u << ((31 - __clz((arcs * 0x101u >> turn) & 255u) + turn) & 7u));
+            const unsigned a = S.L[p] & 0x7FFFu;
+            const bool above = w > S.sv[a];
+#pragma unroll 1
+            for (; arcs; arcs &= arcs - 1) {
+                const unsigned b = S.L[(int)p + ring_off(__ffs(arcs) - 1)] & 0x7FFFu;
+                if (a == b || !(above || w > S.sv[b])) continue;
+                const uint32_t n = a << 20 | b << 8 | w;
+                unsigned at = i;
+                if (first == 0u) {
+                    first = n;
+                } else {
+                    at = atomicAdd(&S.nmore, 1u) + nsad;
+                    if (at >= TAB) break;
+                    S.tab[at] = n;
                 }
+                offer(a, w << 24 | K_EDGE | at);
+                offer(b, w << 24 | K_EDGE | at);
             }
+            S.tab[i] = first;
+        }
+    }
+    // this thread's edge out of the block: pixel tid & 63 of side tid >> 6 (top, bottom, left, right)
+    unsigned ob, ow;
+    {
+        const int side = tid >> 6, k = tid & 63;
+        const int px = side < 2 ? k : (side == 2 ? 0 : BS - 1), py = side < 2 ? (side ? BS - 1 : 0) : k;
+        const uint8_t *h = side < 2 ? (side ? S.hB : S.hT) + 1 : (side == 2 ? S.hL : S.hR);
+        ow = h[k];
+        if (CONN == 8) {   // (the corners' diagonal pixels belong to the top and bottom lines)
+            if (side < 2 || k > 0) ow = max(ow, (unsigned)h[k - 1]);
+            if (side < 2 || k < BS - 1) ow = max(ow, (unsigned)h[k + 1]);
+        }
+        ow = min(ow, (unsigned)((const uint8_t *)bi)[(py + 1) * IST * 4 + 16 + px]);
+        ob = S.L[(py + 1) * ST + X0 + px] & 0x7FFFu;
+        if (ow) offer(ob, ow << 24 | K_OUT);
+    }
+#pragma unroll 1
+    for (unsigned b = tid; b < nb; b += NT) {
+        S.comp[b] = (uint16_t)b;
+        S.up[b] = (uint16_t)b;
     }
     __syncthreads();
+    const unsigned ne = nsad + S.nmore;
+    const bool listed = ne <= TAB;   // else: pairs of pixels instead of passes
+    if (!listed) {
+#pragma unroll 1
+        for (unsigned b = tid; b < nb; b += NT) S.best[b] = 0u;
+        __syncthreads();
+    }
 
     if (tid == 0) tick[3] = now_ns();
-    // Boruvka's rounds. A live region takes the heaviest of its edges to the
-    // source and to other regions (numbers break ties, the same for both
-    // ends, so only the two ends of one edge can choose each other); if an
-    // edge out of the block is heavier still, it stops as a node.
+    // Boruvka's rounds. A live region takes the heaviest of its edges: to the
+    // source, to another region (numbers break ties, the same for both ends,
+    // so only the two ends of one edge can choose each other) or out of the
+    // block, where it stops as a node.
     int rounds = 0;
-    for (bool live = true; live; ++rounds) {
-        for (unsigned b = tid; b < nb; b += NT)
-            if (S.up[b] == b && S.st[b] == 0) S.best[b] = S.sj[b] << 24 | K_SOURCE;
-        __syncthreads();
-        each_pass<CONN>(S, [&](unsigned a, unsigned b, unsigned w, unsigned i) {
-            const unsigned ca = S.comp[a], cb = S.comp[b];
-            if (ca == cb) return;
-            const uint32_t key = w << 24 | K_EDGE | i;
-            if (key > *(volatile uint32_t *)&S.best[ca]) atomicMax(&S.best[ca], key);
-            if (key > *(volatile uint32_t *)&S.best[cb]) atomicMax(&S.best[cb], key);
-        });
-        __syncthreads();
+    for (;; ++rounds) {
+        // edges: to their present ends; one inside a region is dropped
+        if (rounds || !listed) {
+            if (ow) offer(S.comp[ob], ow << 24 | K_OUT);
+            if (listed) {
+#pragma unroll 1
+                for (unsigned i = tid; i < ne; i += NT) {
+                    uint32_t e = S.tab[i];
+                    if (e == 0u) continue;
+                    const unsigned a = S.comp[e >> 20], b = S.comp[(e >> 8) & 0xFFFu];
+                    const uint32_t n = a == b ? 0u : (a << 20 | b << 8 | (e & 255u));
+                    if (n != e) S.tab[i] = n;
+                    if (n == 0u) continue;
+                    offer(a, e << 24 | K_EDGE | i);
+                    offer(b, e << 24 | K_EDGE | i);
+                }
+            } else {
+                each_pair(S, [&](unsigned a, unsigned b, unsigned w, unsigned i) {
+                    a = S.comp[a];
+                    b = S.comp[b];
+                    if (a == b) return;
+                    offer(a, w << 24 | K_EDGE | i);
+                    offer(b, w << 24 | K_EDGE | i);
+                });
+            }
+            __syncthreads();
+        }
+#pragma unroll 1
         for (unsigned b = tid; b < nb; b += NT) {
-            if (S.up[b] != b || S.st[b] != 0) continue;
-            const uint32_t key = S.best[b];
-            const unsigned w = key >> 24;
-            if (S.cb[b] > w || (key & K_SOURCE)) {
-                S.st[b] = S.cb[b] > w ? 1 : 2;
-                *(volatile uint32_t *)&S.best[b] = DONE;
+            if (S.up[b] != b) continue;
+            const uint32_t key = S.best[b], src = S.sv[b] << 24 | K_SOURCE;
+            if (key >= FINAL) continue;
+            if (src > key) {
+                S.capw[b] = (uint8_t)(src >> 24);
+                *(volatile uint32_t *)&S.best[b] = FINAL;
                 continue;
             }
-            unsigned a1, a2;
-            pass_ends<CONN>(S, key & 0x3FFFFFu, a1, a2);
-            unsigned t = S.comp[a1];
-            if (t == b) t = S.comp[a2];
-            // the other end chose this edge too and will not stop: the lower number stays
-            if (b < t && *(volatile uint32_t *)&S.best[t] == key && S.cb[t] <= w) continue;
+            if (!(key & K_EDGE)) {
+                S.capw[b] = (uint8_t)atomicAdd(&S.nt, 1u);
+                *(volatile uint32_t *)&S.best[b] = NODE;
+                continue;
+            }
+            const unsigned i = key & 0x3FFFFFu;
+            unsigned t, t2;
+            if (listed) {
+                const uint32_t e = S.tab[i];
+                t = e >> 20;
+                t2 = (e >> 8) & 0xFFFu;
+            } else {
+                const unsigned px = i >> 2, p = (px / BS + 1) * ST + X0 + px % BS;
+                t = S.comp[S.L[p] & 0x7FFFu];
+                t2 = S.comp[S.L[p + dir_off(4u + (i & 3u))] & 0x7FFFu];
+            }
+            if (t == b) t = t2;
+            // both ends chose this edge: the lower number stays
+            if (b < t && *(volatile uint32_t *)&S.best[t] == key && (S.sv[t] << 24 | K_SOURCE) < key) continue;
             S.up[b] = (uint16_t)t;
-            S.capw[b] = (uint8_t)w;
+            S.capw[b] = (uint8_t)(key >> 24);
         }
         __syncthreads();
-        live = false;
+        bool live = false;
+#pragma unroll 1
         for (unsigned b = tid; b < nb; b += NT) {
             const unsigned was = S.comp[b];
             unsigned t = was;
+#pragma unroll 1
             while (S.up[t] != t) t = S.up[t];
-            S.comp[b] = (uint16_t)t;
-            if (was == b) {
-                if (t != b) {   // merged this round
-                    atomicMax(&S.sj[t], S.sj[b]);
-                    atomicMax(&S.cb[t], S.cb[b]);
-                } else if (S.best[b] != DONE) {
-                    live = true;
-                }
+            if (t != was) {
+                S.comp[b] = (uint16_t)t;
+                if (was == b && S.sv[b] > *(volatile uint32_t *)&S.sv[t]) atomicMax(&S.sv[t], S.sv[b]);   // merged this round
+            } else if (t == b && S.best[b] < FINAL) {
+                live = true;
+                S.best[b] = 0u;
             }
         }
-        live = __syncthreads_or(live);
+        if (!__syncthreads_or(live)) break;
     }
 
-    // Nodes and, per basin, its cap (or final value) and node
-    for (unsigned b = tid; b < nb; b += NT)
-        if (S.st[b] == 1) {
-            const unsigned k = atomicAdd(&S.nt, 1u);
-            S.ss[k] = S.sj[b];
-            S.cb[b] = k;
-        }
-    __syncthreads();
+    // Per basin its cap (or final value) and node, cap << 8 | node slot, in comp.
     const unsigned nt = S.nt;
+#pragma unroll 1
     for (unsigned b = tid; b < nb; b += NT) {
-        unsigned v = 255, t = b;
-        while (S.up[t] != t) {
-            v = min(v, (unsigned)S.capw[t]);
-            t = S.up[t];
-        }
-        S.best[b] = S.st[t] == 1 ? (v << 8 | S.cb[t]) : (min(v, S.sj[t]) << 8 | RES);
+        const unsigned root = S.comp[b];
+        const bool node = S.best[root] == NODE;
+        unsigned v = node ? 255u : S.capw[root];
+#pragma unroll 1
+        for (unsigned t = b; t != root; t = S.up[t]) v = min(v, (unsigned)S.capw[t]);
+        S.comp[b] = (uint16_t)(v << 8 | (node ? S.capw[root] : RES));
+        if (node && b == root) S.link[S.capw[b]] = S.sv[b] << 8 | RES;
     }
     __syncthreads();
     if (nt) {
-        // node links inside the block: to the source, then to each other
-        each_pass<CONN>(S, [&](unsigned a, unsigned b, unsigned w, unsigned) {
-            const uint32_t fa = S.best[a], fb = S.best[b];
-            const unsigned na = fa & 255u, nb2 = fb & 255u;
-            if (na == nb2 || (na != RES && nb2 != RES)) return;
-            atomicMax(&S.ss[na == RES ? nb2 : na], min(w, min(fa >> 8, fb >> 8)));
-        });
-        __syncthreads();
-        for (unsigned k = tid; k < nt; k += NT) S.link[k] = S.ss[k] << 8 | RES;
+        // Node links inside the block: to the source, then to each other. (An
+        // edge left between two regions is no heavier than the caps inside them.)
+        auto ends = [&](unsigned a, unsigned b, unsigned w) -> uint32_t {
+            const unsigned fa = S.comp[a], fb = S.comp[b], na = fa & 255u, nb2 = fb & 255u;
+            w = min(w, min(fa >> 8, fb >> 8));
+            if (na == nb2 || w == 0) return 0u;
+            if (na != RES && nb2 != RES) return na << 16 | nb2 << 8 | w;   // between two nodes
+            uint32_t *l = &S.link[na == RES ? nb2 : na];
+            if ((w << 8 | RES) > *(volatile uint32_t *)l) atomicMax(l, w << 8 | RES);
+            return 0u;
+        };
+        if (listed) {
+#pragma unroll 1
+            for (unsigned i = tid; i < ne; i += NT) {
+                const uint32_t e = S.tab[i];
+                if (e) S.tab[i] = ends(e >> 20, (e >> 8) & 0xFFFu, e & 255u);
+            }
+        } else {
+            each_pair(S, [&](unsigned a, unsigned b, unsigned w, unsigned) { ends(a, b, w); });
+        }
         __syncthreads();
         SharedLinks F{S.link, blk * MAX_TERM};
         bool ok = true;
-        each_pass<CONN>(S, [&](unsigned a, unsigned b, unsigned w, unsigned) {
-            const uint32_t fa = S.best[a], fb = S.best[b];
-            const unsigned na = fa & 255u, nb2 = fb & 255u;
-            if (na == nb2 || na == RES || nb2 == RES) return;
-            w = min(w, min(fa >> 8, fb >> 8));
-            if (w) ok &= join(F, na, nb2, w);
-        });
+        if (listed) {
+#pragma unroll 1
+            for (unsigned i = tid; i < ne; i += NT) {
+                const uint32_t e = S.tab[i];
+                if (e) ok &= join(F, e >> 16, (e >> 8) & 255u, e & 255u);
+            }
+        } else {
+            // (the sources' part was done above; links may now point to nodes)
+            each_pair(S, [&](unsigned a, unsigned b, unsigned w, unsigned) {
+                const unsigned fa = S.comp[a], fb = S.comp[b], na = fa & 255u, nb2 = fb & 255u;
+                w = min(w, min(fa >> 8, fb >> 8));
+                if (na != nb2 && na != RES && nb2 != RES && w) ok &= join(F, na, nb2, w);
+            });
+        }
         if (!ok) atomicCAS(&P.ctl->abort, 0, (int)rk::AB_MERGE);
         __syncthreads();
+#pragma unroll 1
         for (unsigned k = tid; k < nt; k += NT) {
             const uint32_t l = S.link[k];
             const unsigned par = l & 255u;
@@ -669,25 +742,26 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 4 : 3) block_kernel(Params P)
     // Results: the pixels themselves when everything is final, else (cap, node)
     {
         const int cell = (r + 1) * ST + X0 + 16 * c;
+        const uint4 iv = *(const uint4 *)&bi[(r + 1) * IST + 4 + 4 * c];
+        const uint32_t iw[4] = {iv.x, iv.y, iv.z, iv.w};
         uint32_t o[8];   // 16 x (value << 8 | node slot)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint4 q = *(const uint4 *)&S.W[cell + 4 * j];
+        for (int h = 0; h < 2; ++h) {
+            const uint4 q = *(const uint4 *)&S.L[cell + 8 * h];
             const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-            uint32_t f[4];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const uint32_t e = S.best[w[b] & 0x7FFFu];
-                f[b] = min(e >> 8, w[b] >> 24) << 8 | (e & 255u);
+            for (int j = 0; j < 4; ++j) {   // pixels 8h + 2j, 8h + 2j + 1
+                const uint32_t i2 = iw[2 * h + (j >> 1)] >> (16 * (j & 1));
+                const uint32_t e0 = S.comp[w[j] & 0x7FFFu], e1 = S.comp[(w[j] >> 16) & 0x7FFFu];
+                o[4 * h + j] = (min(e0 >> 8, i2 & 255u) << 8 | (e0 & 255u)) |
+                               (min(e1 >> 8, (i2 >> 8) & 255u) << 8 | (e1 & 255u)) << 16;
             }
-            o[2 * j] = f[0] | f[1] << 16;
-            o[2 * j + 1] = f[2] | f[3] << 16;
         }
         if (nt == 0) {
             uint32_t w[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) w[j] = __byte_perm(o[2 * j], o[2 * j + 1], 0x7531) ^ (D.dual ? FULL : 0u);
-            if (y < D.H) store16(D.J + (size_t)y * D.pitch, x, D.W, make_uint4(w[0], w[1], w[2], w[3]), vec);
+            if (y < D.H) store16(D.J + (size_t)y * D.pitch + x, D.W - x, make_uint4(w[0], w[1], w[2], w[3]), vec);
         } else {
             uint4 *dst = (uint4 *)(P.px + (size_t)blk * BPX + r * BS + 16 * c);
             dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
@@ -709,7 +783,8 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 4 : 3) block_kernel(Params P)
         rk::Work &wk = P.work[D.index];
         atomicAdd(&wk.visits, 1ull);
         atomicAdd(&wk.seeds, (unsigned long long)(nb - 1));
-        atomicAdd(&wk.levels, (unsigned long long)rounds);
+        atomicAdd(&wk.pops, (unsigned long long)ne);
+        atomicAdd(&wk.levels, (unsigned long long)rounds + 1);
         atomicAdd(&wk.busy_ns, tick[5] - tick[0]);
 #pragma unroll
         for (int k = 0; k < 5; ++k) atomicAdd(&wk.phase_ns[k], tick[k + 1] - tick[k]);
@@ -826,7 +901,7 @@ __global__ void __launch_bounds__(NT) value_kernel(Params P)
         w[j] = v ^ (D.dual ? FULL : 0u);
     }
     const bool vec = (D.pitch % 16) == 0 && ((uintptr_t)D.J % 16) == 0;
-    store16(D.J + (size_t)y * D.pitch, x, D.W, make_uint4(w[0], w[1], w[2], w[3]), vec);
+    store16(D.J + (size_t)y * D.pitch + x, D.W - x, make_uint4(w[0], w[1], w[2], w[3]), vec);
 }
 
 }  // namespace rf
