@@ -78,6 +78,8 @@ struct recon_ctx {
     int *d_dt_site = nullptr; size_t cap_dt_site = 0;
     unsigned *h_dt_cnt = nullptr;
     int dt_levels = 0;
+    // training scratch (moments, epoch losses, two epochs' sample orders)
+    unsigned char *d_train = nullptr; size_t cap_train = 0;
     // autotuner results: (size bucket, connectivities, marker class) -> {bh, bands, k, gain}
     std::map<std::tuple<int, int, int>, std::vector<int>> tune_cache;
     int tune_from_cache = 0;
@@ -192,6 +194,7 @@ extern "C" int recon_free(recon_ctx *c)
     cudaFree(c->d_img);
     cudaFree(c->d_dt);
     cudaFree(c->d_dt_site);
+    cudaFree(c->d_train);
     if (c->h_dt_cnt) cudaFreeHost(c->h_dt_cnt);
     if (c->h_meta) cudaFreeHost(c->h_meta);
     if (c->h_trace) cudaFreeHost(c->h_trace);
@@ -1018,25 +1021,27 @@ static uint64_t sm64(uint64_t z)
     return z ^ (z >> 31);
 }
 
-extern "C" int recon_mlp_train_resume(recon_ctx *c, float *theta, float *adam_mv, int *step, int epoch0,
-                                      const float *X, const float *T, int n, int epochs, int batch, float lr,
-                                      uint64_t seed, float *epoch_loss)
+// Epochs epoch0 .. epoch0 + epochs - 1 of mini-batch Adam, one launch each. The
+// host shuffles the next epoch while one runs; the two index buffers alternate.
+// adam_mv NULL: moments in the context's scratch, starting at zero.
+static int train_epochs(recon_ctx *c, float *theta, float *adam_mv, int *step, int epoch0, const float *X, const float *T,
+                        int n, int epochs, int batch, float lr, uint64_t seed, float *epoch_loss)
 {
-    if (!c || !theta || !adam_mv || !step || *step < 0 || epoch0 < 0 || !X || !T || n < 1 || epochs < 1 ||
-        batch < 1 || !(lr > 0.0f))
-        return RECON_EINVAL;
     CK(cudaSetDevice(c->device));
     CK(cudaStreamSynchronize(c->stream));
-    float *m = adam_mv, *v = adam_mv + MLP_NPARAMS, *g = nullptr, *dl = nullptr;
-    int *didx = nullptr;
-    cudaError_t e = cudaMalloc((void **)&g, sizeof(float) * MLP_NPARAMS);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g, 0, sizeof(float) * MLP_NPARAMS, c->stream);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&didx, sizeof(int) * (size_t)n * 2);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&dl, sizeof(float) * epochs);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dl, 0, sizeof(float) * epochs, c->stream);
+    const size_t off_loss = align_up(sizeof(float) * 2 * MLP_NPARAMS, 16);
+    const size_t off_idx = align_up(off_loss + sizeof(float) * (size_t)epochs, 16);
+    int rc = grow(&c->d_train, &c->cap_train, off_idx + sizeof(int) * 2 * (size_t)n);
+    if (rc) return rc;
+    float *mv = adam_mv ? adam_mv : (float *)c->d_train, *dl = (float *)(c->d_train + off_loss);
+    int *didx = (int *)(c->d_train + off_idx);
+    // the scratch moments and the epoch losses lie next to each other
+    cudaError_t e = adam_mv ? cudaMemsetAsync(dl, 0, sizeof(float) * (size_t)epochs, c->stream)
+                            : cudaMemsetAsync(c->d_train, 0, off_idx, c->stream);
+    batch = std::min(batch, n);
     std::vector<int> perm(n);
     int t = *step;
-    const int nbatches = (n + batch - 1) / batch;
+    const int nbatches = (n - 1) / batch + 1;
     for (int k = 0; k < epochs && e == cudaSuccess; ++k) {
         const int ep = epoch0 + k;   // the shuffle depends on the absolute epoch, so a resumed run repeats it
         // Fisher-Yates shuffle driven by SplitMix64 outputs of (seed, epoch)
@@ -1047,14 +1052,12 @@ extern "C" int recon_mlp_train_resume(recon_ctx *c, float *theta, float *adam_mv
             const int j = (int)(st % (uint64_t)(i + 1));
             std::swap(perm[i], perm[j]);
         }
-        int *buf = didx + (size_t)(k & 1) * n;  // double-buffered: the copy of epoch e+1 cannot race epoch e
+        int *buf = didx + (size_t)(k & 1) * n;
+        // returns once the pageable source is staged, so perm may be refilled
         e = cudaMemcpyAsync(buf, perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // perm is pageable and reused
-        for (int s = 0; s < n && e == cudaSuccess; s += batch) {
-            const int nb = std::min(batch, n - s);
-            e = rl_grad(theta, X, T, buf + s, nb, g, dl + k, c->stream);
-            if (e == cudaSuccess) e = rl_adam(theta, g, m, v, ++t, lr, c->stream);
-        }
+        if (e == cudaSuccess)
+            e = rl_train_epoch(theta, mv, mv + MLP_NPARAMS, X, T, buf, n, batch, t, lr, dl + k, c->stream);
+        t += nbatches;
     }
     if (e == cudaSuccess && epoch_loss) {
         e = cudaMemcpyAsync(epoch_loss, dl, sizeof(float) * epochs, cudaMemcpyDeviceToHost, c->stream);
@@ -1063,26 +1066,25 @@ extern "C" int recon_mlp_train_resume(recon_ctx *c, float *theta, float *adam_mv
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e == cudaSuccess) *step = t;
-    cudaFree(g);
-    cudaFree(didx);
-    cudaFree(dl);
     return cuda_status(e);
+}
+
+extern "C" int recon_mlp_train_resume(recon_ctx *c, float *theta, float *adam_mv, int *step, int epoch0,
+                                      const float *X, const float *T, int n, int epochs, int batch, float lr,
+                                      uint64_t seed, float *epoch_loss)
+{
+    if (!c || !theta || !adam_mv || !step || *step < 0 || epoch0 < 0 || !X || !T || n < 1 || epochs < 1 ||
+        batch < 1 || !(lr > 0.0f))
+        return RECON_EINVAL;
+    return train_epochs(c, theta, adam_mv, step, epoch0, X, T, n, epochs, batch, lr, seed, epoch_loss);
 }
 
 extern "C" int recon_mlp_train(recon_ctx *c, float *theta, const float *X, const float *T, int n, int epochs,
                                int batch, float lr, uint64_t seed, float *epoch_loss)
 {
-    if (!c) return RECON_EINVAL;
-    CK(cudaSetDevice(c->device));
-    float *mv = nullptr;
-    CK(cudaMalloc((void **)&mv, sizeof(float) * MLP_NPARAMS * 2));
     int step = 0;
-    cudaError_t e = cudaMemsetAsync(mv, 0, sizeof(float) * MLP_NPARAMS * 2, c->stream);
-    int rc = e == cudaSuccess ? recon_mlp_train_resume(c, theta, mv, &step, 0, X, T, n, epochs, batch, lr, seed,
-                                                       epoch_loss)
-                              : cuda_status(e);
-    cudaFree(mv);
-    return rc;
+    if (!c || !theta || !X || !T || n < 1 || epochs < 1 || batch < 1 || !(lr > 0.0f)) return RECON_EINVAL;
+    return train_epochs(c, theta, nullptr, &step, 0, X, T, n, epochs, batch, lr, seed, epoch_loss);
 }
 
 extern "C" int recon_sched_set_model(recon_ctx *c, const float *theta, const float *norm, int variant_a,
