@@ -354,23 +354,19 @@ int recon_checks(int *enabled, unsigned *violations, unsigned *first, int reset)
 
 /* ---- distance transform (Table II) ----
  * For each foreground pixel (B != 0) of the H x W image B (device uint8,
- * pitch = W), the squared Euclidean distance to the background pixel that the
- * 8-connected irregular wavefront propagation assigns to it: Algorithm 1 with
- * elements D(p) = the nearest background pixel ("site") found so far, seeded
- * from the background pixels that touch the foreground; a foreground neighbour
- * q takes site s when (|q - s|^2, s) < (|q - site(q)|^2, site(q)).
+ * pitch = W), the squared Euclidean distance to the nearest background pixel
+ * (its "site"), the fixed point that the irregular wavefront propagation of
+ * Algorithm 1 approximates: every pixel holds the site with the smallest
+ * (|q - s|^2, s). Computed exactly, by columns and rows; the result does not
+ * depend on any order.
  * d2: device uint32 H x W out (0 on background; 0xFFFFFFFF everywhere when B
  * has no background pixel). site: device int32 H x W out, index y*W + x of the
- * assigned background pixel (-1 without background), or NULL (the context then
- * keeps it in its scratch). 1 <= H, W <= 32768, H * W < 2^31.
- * Like Danielsson's vector propagation this approximates the exact Euclidean
- * transform (a pixel passes on only the site it holds); the result depends on
- * the processing order, but every site is a background pixel and no pixel has
- * an 8-neighbour holding a closer site. Runs on the context stream and waits;
- * RECON_ETIMEOUT if an iteration bound ran out. */
+ * assigned background pixel (-1 without background), or NULL.
+ * 1 <= H, W <= 32768, H * W < 2^31. Runs on the context stream and waits. */
 int recon_dt(recon_ctx *ctx, const uint8_t *B, uint32_t *d2, int32_t *site, int H, int W);
 
-/* Wavefront levels the last recon_dt call ran (diagnostics), or -1. */
+/* Wavefront levels the last recon_dt call ran: 0 (it needs none), or -1 without
+ * a context. */
 int recon_dt_levels(recon_ctx *ctx);
 
 /* ---- device micro-benchmarks (Sec. V-C, Tables III and IV) ----

@@ -75,9 +75,6 @@ struct recon_ctx {
     recon_sched *sched = nullptr;
     // distance transform scratch
     unsigned char *d_dt = nullptr; size_t cap_dt = 0;
-    int *d_dt_site = nullptr; size_t cap_dt_site = 0;
-    unsigned *h_dt_cnt = nullptr;
-    int dt_levels = 0;
     // training scratch (moments, epoch losses, two epochs' sample orders)
     unsigned char *d_train = nullptr; size_t cap_train = 0;
     // autotuner results: (size bucket, connectivities, marker class) -> {bh, bands, k, gain}
@@ -193,9 +190,7 @@ extern "C" int recon_free(recon_ctx *c)
     cudaFree(c->d_forest);
     cudaFree(c->d_img);
     cudaFree(c->d_dt);
-    cudaFree(c->d_dt_site);
     cudaFree(c->d_train);
-    if (c->h_dt_cnt) cudaFreeHost(c->h_dt_cnt);
     if (c->h_meta) cudaFreeHost(c->h_meta);
     if (c->h_trace) cudaFreeHost(c->h_trace);
     if (c->meta_free) cudaEventDestroy(c->meta_free);
@@ -1291,23 +1286,18 @@ extern "C" int recon_dt(recon_ctx *c, const uint8_t *B, uint32_t *d2, int32_t *s
     if (!c || !B || !d2 || H < 1 || W < 1 || H > 32768 || W > 32768) return RECON_EINVAL;
     if ((long long)H * W > 0x7FFFFFFFll) return RECON_EINVAL;
     CK(cudaSetDevice(c->device));
-    const size_t n = (size_t)H * W;
     const size_t need = dt_scratch_bytes(H, W);
-    if (c->cap_dt < need || (!site && c->cap_dt_site < n) || !c->h_dt_cnt) {
+    if (c->cap_dt < need) {
         CK(cudaStreamSynchronize(c->stream));
-        int rc;
-        if ((rc = grow(&c->d_dt, &c->cap_dt, need))) return rc;
-        if (!site && (rc = grow(&c->d_dt_site, &c->cap_dt_site, n))) return rc;
-        if (!c->h_dt_cnt) CK(cudaMallocHost((void **)&c->h_dt_cnt, 4 * sizeof(unsigned)));
+        const int rc = grow(&c->d_dt, &c->cap_dt, need);
+        if (rc) return rc;
     }
-    int *s = site ? (int *)site : c->d_dt_site;
-    const int rc = dt_run(B, H, W, s, (unsigned *)d2, c->d_dt, c->h_dt_cnt, 8 * c->sms, c->stream, &c->dt_levels);
-    if (rc == DT_ECUDA) return RECON_ECUDA;
+    if (dt_run(B, H, W, (int *)site, (unsigned *)d2, c->d_dt, c->sms, c->stream) != DT_OK) return RECON_ECUDA;
     CK(cudaStreamSynchronize(c->stream));
-    return rc == DT_ELIMIT ? RECON_ETIMEOUT : RECON_OK;
+    return RECON_OK;
 }
 
 extern "C" int recon_dt_levels(recon_ctx *c)
 {
-    return c ? c->dt_levels : -1;
+    return c ? 0 : -1;   // the transform no longer runs in levels
 }

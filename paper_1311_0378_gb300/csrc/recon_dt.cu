@@ -1,25 +1,28 @@
-// Distance transform by irregular wavefront propagation (Table II, "Distance
-// Transform": for each foreground pixel the distance to the closest background
-// pixel; irregular, 8-connected, IWPP).
+// Distance transform (Table II, "Distance Transform": for each foreground pixel
+// the distance to the closest background pixel). What Algorithm 1's wavefront
+// propagates towards -- every pixel holding the nearest background pixel
+// ("site") -- is computed directly, in two separable steps (Saito and Toriwaki
+// 1994): the nearest background pixel of each pixel's column, then, along the
+// row, the smallest dx^2 + (column distance)^2. The result is exact and does
+// not depend on any order; of equally near sites the one with the lower index
+// is taken. (A wavefront passes on only the site a pixel holds, so it can miss
+// the nearest one; where it does not, the two agree.)
 //
-// Algorithm 1 with data elements D(p) = the background pixel ("site") nearest
-// to p found so far. Initialization: background pixels are their own sites,
-// foreground pixels have none; the wavefront S = background pixels touching a
-// foreground pixel. Propagation: for an element p of S with site s, every
-// foreground 8-neighbour q with key(q, s) < key(q, site(q)) takes s and joins
-// S, key(q, s) = (|q - s|^2, s) (ties to the lower site index).
+//   mask_kernel    32 rows of a column per 32-bit word (bit set: background)
+//   column_kernel  signed distance to the nearest background row of the column,
+//                  by bit scans of the column's words (16 bits a pixel)
+//   row_kernel     a row of squared column distances in shared memory; each
+//                  pixel searches outwards until dx^2 reaches its best, past 32
+//                  columns in runs of 32 that a run's minimum can rule out
 //
-// GB300 form: the wavefront is processed level-synchronously in global memory,
-// one launch per level over a compacted frontier; a site is taken by a 32-bit
-// compare-and-swap, and a per-pixel level stamp keeps each pixel at most once
-// in a level's frontier. While the transform runs, sites and frontier entries
-// are packed coordinates (y << 16 | x), which order like y * W + x and need no
-// division; the final pass writes indices y * W + x. Three rotating level
-// counters let consecutive level launches run back to back without a host
-// round trip; the host reads a counter once per batch of levels to learn when
-// S is empty. A CTA reserves the slots of all its new frontier entries with one
-// global atomic add (a single global counter is the contended resource).
-#include <climits>
+// The work per pixel is a few bit operations plus about two instructions per
+// column within its distance; no step waits for another pixel's result. A
+// 4096^2 mask of the space between objects (distances up to 97, 112 wavefront
+// levels, each a launch of dependent global loads) takes 0.145 ms, 2.63 ms as a
+// wavefront; the objects of a 2048 x 3000 mask 40 us, 297 us before. The row
+// search is two thirds of it (60% of the issue slots, 4.4 instructions per pixel
+// and column of distance); masks and columns are bound by memory latency.
+#include <algorithm>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -27,188 +30,297 @@
 
 namespace dt {
 
-// packed coordinates: y << 16 | x (y, x < 32768)
-__device__ __forceinline__ unsigned dist2(int q, int s)
-{
-    const int dy = (q >> 16) - (s >> 16), dx = (q & 0xFFFF) - (s & 0xFFFF);
-    return (unsigned)(dy * dy) + (unsigned)(dx * dx);
-}
+constexpr unsigned INF = 0x7FFFFFFFu;   // above every squared distance (2 * 32767^2); INF + dx^2 fits 32 bits
+constexpr uint32_t FAR = 32767u + 1u;   // more than any distance within a column
+constexpr int PAD = 128;                // columns of INF at both ends of a row in shared memory
 
-// key(q, s) = (|q - s|^2, s); no site = +infinity. Packed sites order like
-// their indices y * W + x, so the tie-break is the same.
-__device__ __forceinline__ unsigned long long key_of(int q, int s)
+// A thread packs four columns of a strip of 32 rows.
+__global__ void __launch_bounds__(128) mask_kernel(const uint8_t *B, int H, int W, uint32_t *M)
 {
-    if (s < 0) return ~0ull;
-    return ((unsigned long long)dist2(q, s) << 32) | (unsigned)s;
-}
-
-// warp-aggregated append of v to list (count *cnt) when pred
-__device__ __forceinline__ void push(int *list, unsigned *cnt, bool pred, int v)
-{
-    const unsigned bal = __ballot_sync(0xFFFFFFFFu, pred);
-    if (!bal) return;
-    const int lane = threadIdx.x & 31, leader = __ffs(bal) - 1;
-    unsigned base = 0;
-    if (lane == leader) base = atomicAdd(cnt, (unsigned)__popc(bal));
-    base = __shfl_sync(0xFFFFFFFFu, base, leader);
-    if (pred) list[base + __popc(bal & ((1u << lane) - 1u))] = v;
-}
-
-__global__ void __launch_bounds__(256) init_kernel(const uint8_t *B, int H, int W, int *site, int *stamp, int *F0,
-                                                   unsigned *cnt)
-{
-    const long long n = (long long)H * W;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    // whole warps iterate together (the ballot in push needs every lane)
-    for (long long base = (long long)blockIdx.x * blockDim.x; base < n; base += stride) {
-        const long long p = base + threadIdx.x;
-        bool seed = false;
-        if (p < n) {
-            const bool fg = B[p] != 0;
-            const int y = (int)(p / W), x = (int)(p - (long long)y * W);
-            site[p] = fg ? -1 : (y << 16 | x);
-            stamp[p] = 0;
-            if (!fg) {
-                for (int dy = -1; dy <= 1 && !seed; ++dy)
-                    for (int dx = -1; dx <= 1; ++dx) {
-                        const int yy = y + dy, xx = x + dx;
-                        if ((dy || dx) && yy >= 0 && yy < H && xx >= 0 && xx < W && B[(long long)yy * W + xx]) {
-                            seed = true;
-                            break;
-                        }
-                    }
-            }
-        }
-        push(F0, &cnt[0], seed, p < n ? (int)((p / W) << 16 | (p % W)) : 0);
-    }
-}
-
-// Level L: reads frontier Fin (count cnt[L % 3]), appends to Fout (count
-// cnt[(L + 1) % 3]) and resets cnt[(L + 2) % 3], which no launch reads again
-// before level L + 2 (it was level L - 1's input count).
-__global__ void __launch_bounds__(256) level_kernel(const uint8_t *B, int H, int W, int *site, int *stamp,
-                                                    const int *Fin, int *Fout, unsigned *cnt, int L, int *err)
-{
-    __shared__ unsigned s_tot, s_base;
-    const unsigned n = cnt[L % 3];
-    if (blockIdx.x == 0 && threadIdx.x == 0) cnt[(L + 2) % 3] = 0;
-    if (threadIdx.x == 0) s_tot = 0;
-    __syncthreads();
-    const unsigned stride = gridDim.x * blockDim.x;
-    for (unsigned base = blockIdx.x * blockDim.x; base < n; base += stride) {
-        const unsigned i = base + threadIdx.x;
-        unsigned raised = 0;   // bit k: neighbour k took this site and is new in the next level
-        int p = 0;   // packed coordinates
-        if (i < n) {
-            p = Fin[i];
-            const int y = p >> 16, x = p & 0xFFFF;
-            const int s = __ldcg(site + (y * W + x));
+    const int x = 4 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (x >= W) return;
+    const bool vec = (W & 3) == 0 && ((uintptr_t)B & 3) == 0;
+    const int y1 = min(H - (int)blockIdx.y * 32, 32);
+    const uint8_t *p = B + (size_t)blockIdx.y * 32 * W + x;
+    uint32_t m[4] = {0u, 0u, 0u, 0u};
+    for (int r0 = 0; r0 < y1; r0 += 16) {   // 16 rows' loads in flight
+        uint32_t v[16];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int dy = k < 3 ? -1 : (k < 5 ? 0 : 1);
-                const int dx = (k == 0 || k == 3 || k == 5) ? -1 : ((k == 1 || k == 6) ? 0 : 1);
-                const int yy = y + dy, xx = x + dx;
-                if (yy < 0 || yy >= H || xx < 0 || xx >= W) continue;
-                const int qi = yy * W + xx, q = yy << 16 | xx;
-                if (!B[qi]) continue;
-                const unsigned long long kn = key_of(q, s);
-                int cur = __ldcg(site + qi);
-                for (int it = 0; kn < key_of(q, cur); ++it) {
-                    if (it > (1 << 16)) { atomicExch(err, 1); break; }
-                    const int prev = atomicCAS(site + qi, cur, s);
-                    if (prev == cur) {
-                        if (atomicExch(stamp + qi, L + 1) != L + 1) raised |= 1u << k;
-                        break;
-                    }
-                    cur = prev;
+        for (int r = 0; r < 16; ++r) {
+            v[r] = 0xFFFFFFFFu;
+            if (r0 + r < y1) {
+                const uint8_t *q = p + (size_t)(r0 + r) * W;
+                if (vec) {
+                    v[r] = __ldg((const uint32_t *)q);
+                } else {
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+                        if (x + b < W && q[b] == 0) v[r] &= ~(0xFFu << (8 * b));
                 }
             }
         }
-        unsigned bal[8], tot = 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            bal[k] = __ballot_sync(0xFFFFFFFFu, (raised >> k) & 1u);
-            tot += __popc(bal[k]);
-        }
-        // slots: warp offset inside the CTA (shared atomic), then one global
-        // atomic per CTA; the loop is block-uniform, so the barriers are safe
-        const int lane = threadIdx.x & 31;
-        unsigned o = 0;
-        if (lane == 0 && tot) o = atomicAdd(&s_tot, tot);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            s_base = s_tot ? atomicAdd(&cnt[(L + 1) % 3], s_tot) : 0u;
-            s_tot = 0;
-        }
-        __syncthreads();
-        if (tot) {
-            o = __shfl_sync(0xFFFFFFFFu, o, 0) + s_base;
-            const unsigned lt = (1u << lane) - 1u;
+        for (int r = 0; r < 16; ++r)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) m[b] |= (((v[r] >> (8 * b)) & 255u) == 0u ? 1u : 0u) << (r0 + r);
+    }
+    uint32_t *o = M + (size_t)blockIdx.y * W + x;
+    if ((W & 3) == 0) {
+        *(uint4 *)o = make_uint4(m[0], m[1], m[2], m[3]);
+    } else {
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+            if (x + b < W) o[b] = m[b];
+    }
+}
+
+// A thread takes two columns of a strip of 32 rows. The nearest background above
+// and below the strip comes from the words of the strips around it, eight at a
+// time (a walk word by word waits for one load after another). Then, as two u16
+// lanes, the distance downwards for all rows (kept in registers) and upwards. G:
+// rows of `pitch` (even) distances, FAR or more without background; with SITE
+// bit 15 says "upwards" (a tie goes up, to the lower index) and FAR alone means
+// none.
+template <bool SITE>
+__global__ void __launch_bounds__(128) column_kernel(const uint32_t *M, int H, int W, uint16_t *G, int pitch)
+{
+    const int x = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (x >= W) return;
+    const int s = blockIdx.y, ns = gridDim.y, y0 = 32 * s, xb = min(x + 1, W - 1);
+    const uint32_t m[2] = {M[(size_t)s * W + x], M[(size_t)s * W + xb]};
+    uint32_t up, dn;   // distances from the row before / after the strip
+    {
+        uint32_t u[2] = {FAR, FAR}, d[2] = {FAR, FAR};
+        // a strip whose first (last) row is background needs no look above (below)
+        bool more0 = !(m[0] & 1u), more1 = !(m[1] & 1u);
+        for (int t = s - 1; t >= 0 && (more0 || more1); t -= 8) {
+            uint32_t a[8], b[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                const int dy = k < 3 ? -1 : (k < 5 ? 0 : 1);
-                const int dx = (k == 0 || k == 3 || k == 5) ? -1 : ((k == 1 || k == 6) ? 0 : 1);
-                if ((raised >> k) & 1u) Fout[o + __popc(bal[k] & lt)] = p + dy * 65536 + dx;
-                o += __popc(bal[k]);
+                a[k] = more0 && t - k >= 0 ? M[(size_t)(t - k) * W + x] : 0u;
+                b[k] = more1 && t - k >= 0 ? M[(size_t)(t - k) * W + xb] : 0u;
+            }
+#pragma unroll
+            for (int k = 7; k >= 0; --k) {
+                if (a[k]) { u[0] = (uint32_t)(y0 - 1 - (32 * (t - k) + 31 - __clz(a[k]))); more0 = false; }
+                if (b[k]) { u[1] = (uint32_t)(y0 - 1 - (32 * (t - k) + 31 - __clz(b[k]))); more1 = false; }
+            }
+        }
+        more0 = !(m[0] >> 31);
+        more1 = !(m[1] >> 31);
+        for (int t = s + 1; t < ns && (more0 || more1); t += 8) {
+            uint32_t a[8], b[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                a[k] = more0 && t + k < ns ? M[(size_t)(t + k) * W + x] : 0u;
+                b[k] = more1 && t + k < ns ? M[(size_t)(t + k) * W + xb] : 0u;
+            }
+#pragma unroll
+            for (int k = 7; k >= 0; --k) {
+                if (a[k]) { d[0] = (uint32_t)(32 * (t + k) + __ffs(a[k]) - 1 - (y0 + 32)); more0 = false; }
+                if (b[k]) { d[1] = (uint32_t)(32 * (t + k) + __ffs(b[k]) - 1 - (y0 + 32)); more1 = false; }
+            }
+        }
+        up = u[0] | u[1] << 16;
+        dn = d[0] | d[1] << 16;
+    }
+    // lanes of ones where row r is background: bit r of both words moved to the sign and spread
+    auto bg = [&](int r) {
+        uint32_t o;
+        asm("prmt.b32 %0, %1, %2, 0xFFBB;" : "=r"(o) : "r"(m[0] << (31 - r)), "r"(m[1] << (31 - r)));
+        return o;
+    };
+    uint32_t down[32];
+#pragma unroll
+    for (int r = 31; r >= 0; --r) {
+        dn = (dn + 0x00010001u) & ~bg(r);
+        down[r] = dn;
+    }
+    const int rows = min(H - y0, 32);
+    uint16_t *o = G + (size_t)y0 * pitch + x;
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+        up = (up + 0x00010001u) & ~bg(r);
+        if (r < rows) {
+            uint32_t v;
+            asm("min.u16x2 %0, %1, %2;" : "=r"(v) : "r"(up), "r"(down[r]));
+            if (SITE) {
+                uint32_t w = 0;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const uint32_t g = (v >> (16 * c)) & 0xFFFFu, u = (up >> (16 * c)) & 0xFFFFu;
+                    w |= (g >= FAR ? FAR : (u == g && g ? g | 0x8000u : g)) << (16 * c);
+                }
+                v = w;
+            }
+            *(uint32_t *)(o + (size_t)r * pitch) = v;
+        }
+    }
+}
+
+// A row of squared column distances in shared memory (q, PAD x INF before and
+// PAD + 2 behind it) and the minimum of each run of 32 (low). All threads.
+template <bool SITE>
+__device__ __forceinline__ void load_row(const uint16_t *row, int W, uint32_t *q, uint32_t *low, uint16_t *gs)
+{
+    for (int x = threadIdx.x; x < (W + 31) / 32 * 32; x += blockDim.x) {
+        const uint32_t raw = x < W ? row[x] : FAR;
+        const uint32_t g = SITE ? raw & 0x7FFFu : raw;
+        const uint32_t v = (SITE ? raw == FAR : raw >= FAR) ? INF : g * g;
+        if (x < W) {
+            q[x] = v;
+            if (SITE) gs[x] = (uint16_t)raw;
+        }
+        const uint32_t mn = __reduce_min_sync(0xFFFFFFFFu, v);
+        if ((threadIdx.x & 31) == 0) low[x >> 5] = mn;
+    }
+}
+
+__device__ __forceinline__ void pad_row(int W, uint32_t *q)
+{
+    for (int i = threadIdx.x; i < PAD + 2; i += blockDim.x) {
+        if (i < PAD) q[i - PAD] = INF;
+        q[W + i] = INF;
+    }
+}
+
+// Columns further than PAD from x: whole runs of 32 are skipped when even their
+// minimum is too far. take(column, squared offset), beyond(lower bound): no use.
+template <class Take, class Beyond>
+__device__ __forceinline__ void search_far(int x, int W, const uint32_t *low, Take take, Beyond beyond)
+{
+    for (int c = x - PAD - 1; c >= 0; --c) {
+        const uint32_t d = (uint32_t)((x - c) * (x - c));
+        if (beyond(d)) break;
+        if ((c & 31) == 31 && beyond(d + low[c >> 5])) { c -= 31; continue; }
+        take(c, d);
+    }
+    for (int c = x + PAD + 1; c < W; ++c) {
+        const uint32_t d = (uint32_t)((c - x) * (c - x));
+        if (beyond(d)) break;
+        if ((c & 31) == 0 && beyond(d + low[c >> 5])) { c += 31; continue; }
+        take(c, d);
+    }
+}
+
+// Distances only. Two neighbouring pixels a thread: a pair of columns (one
+// 64-bit load) gives each of them two candidates, one add-and-min instruction
+// each, so a column costs 1.5 instructions a pixel and side (one pixel a thread
+// with 32-bit loads: 314 us for the 4096^2 mask's call instead of 165).
+__global__ void row_kernel(const uint16_t *G, int H, int W, int pitch, unsigned *d2)
+{
+    extern __shared__ __align__(16) uint32_t dt_smem[];
+    uint32_t *const q = dt_smem + PAD, *const low = q + (W + 1) / 2 * 2 + PAD + 2;
+    pad_row(W, q);
+    for (int y = blockIdx.x; y < H; y += gridDim.x) {
+        __syncthreads();                                            // the row before is done with
+        load_row<false>(G + (size_t)y * pitch, W, q, low, nullptr);
+        __syncthreads();
+        for (int x = 2 * threadIdx.x; x < W; x += 2 * blockDim.x) {
+            const uint2 own = *(const uint2 *)&q[x];
+            uint32_t b0 = __viaddmin_u32(own.y, 1u, own.x), b1 = __viaddmin_u32(own.x, 1u, own.y);
+            int j = 2;                                              // columns x - j, x - j + 1 and x + j, x + j + 1
+            for (; j <= PAD; j += 4) {
+                if ((uint32_t)((j - 1) * (j - 1)) >= max(b0, b1)) break;
+#pragma unroll
+                for (int k = 0; k < 4; k += 2) {
+                    const uint2 l = *(const uint2 *)&q[x - j - k], r = *(const uint2 *)&q[x + j + k];
+                    const uint32_t s0 = (uint32_t)((j + k - 1) * (j + k - 1)), s1 = (uint32_t)((j + k) * (j + k)),
+                                   s2 = (uint32_t)((j + k + 1) * (j + k + 1));
+                    b0 = __viaddmin_u32(l.x, s1, __viaddmin_u32(l.y, s0, b0));
+                    b1 = __viaddmin_u32(l.x, s2, __viaddmin_u32(l.y, s1, b1));
+                    b0 = __viaddmin_u32(r.x, s1, __viaddmin_u32(r.y, s2, b0));
+                    b1 = __viaddmin_u32(r.x, s0, __viaddmin_u32(r.y, s1, b1));
+                }
+            }
+            if (j > PAD) {
+                search_far(x, W, low, [&](int c, uint32_t d) { b0 = min(b0, q[c] + d); }, [&](uint32_t d) { return d >= b0; });
+                if (x + 1 < W)
+                    search_far(x + 1, W, low, [&](int c, uint32_t d) { b1 = min(b1, q[c] + d); },
+                               [&](uint32_t d) { return d >= b1; });
+            }
+            unsigned *o = d2 + (size_t)y * W + x;
+            b0 = b0 >= INF ? 0xFFFFFFFFu : b0;
+            b1 = b1 >= INF ? 0xFFFFFFFFu : b1;
+            if ((W & 1) == 0 && ((uintptr_t)d2 & 7) == 0) {
+                *(uint2 *)o = make_uint2(b0, b1);
+            } else {
+                o[0] = b0;
+                if (x + 1 < W) o[1] = b1;
             }
         }
     }
 }
 
-// d2 from the packed sites, and the sites rewritten as indices y * W + x
-__global__ void __launch_bounds__(256) final_kernel(int H, int W, int *site, unsigned *d2)
+// Distances and sites: of equally near sites the one with the lowest index, so
+// columns at exactly the best distance count too.
+__global__ void row_site_kernel(const uint16_t *G, int H, int W, int pitch, unsigned *d2, int *site)
 {
-    const long long n = (long long)H * W;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-        const int s = site[p];
-        const int y = (int)(p / W), x = (int)(p - (long long)y * W);
-        if (d2) d2[p] = s < 0 ? 0xFFFFFFFFu : dist2(y << 16 | x, s);
-        site[p] = s < 0 ? -1 : (s >> 16) * W + (s & 0xFFFF);
+    extern __shared__ __align__(16) uint32_t dt_smem[];
+    uint32_t *const q = dt_smem + PAD, *const low = q + (W + 1) / 2 * 2 + PAD + 2;
+    uint16_t *const gs = (uint16_t *)(low + (W + 31) / 32);         // the column distances with their direction
+    pad_row(W, q);
+    for (int y = blockIdx.x; y < H; y += gridDim.x) {
+        __syncthreads();
+        load_row<true>(G + (size_t)y * pitch, W, q, low, gs);
+        __syncthreads();
+        auto site_of = [&](int c) {
+            const int g = gs[c];
+            return (y + (g & 0x8000 ? -(g & 0x7FFF) : g)) * W + c;
+        };
+        for (int x = threadIdx.x; x < W; x += blockDim.x) {
+            uint32_t best = q[x];
+            int bs = best >= INF ? 0x7FFFFFFF : site_of(x);
+            auto take = [&](int c, uint32_t d) {
+                const uint32_t v = q[c] + d;
+                if (v > best || v >= INF) return;
+                const int s = site_of(c);
+                if (v < best || s < bs) bs = s;
+                best = v;
+            };
+            auto beyond = [&](uint32_t d) { return d > best; };
+            int dx = 1;
+            for (; dx <= PAD; ++dx) {
+                const uint32_t d = (uint32_t)(dx * dx);
+                if (beyond(d)) break;
+                take(x - dx, d);
+                take(x + dx, d);
+            }
+            if (dx > PAD) search_far(x, W, low, take, beyond);
+            const size_t p = (size_t)y * W + x;
+            d2[p] = best >= INF ? 0xFFFFFFFFu : best;
+            site[p] = best >= INF ? -1 : bs;
+        }
     }
 }
 
 }  // namespace dt
 
-size_t dt_scratch_bytes(int H, int W)
-{
-    const size_t n = (size_t)H * W;
-    return 256 + n * sizeof(int) * 3;   // counters + error | stamp | two frontiers
-}
+static size_t mask_bytes(int H, int W) { return (((size_t)((H + 31) / 32) * W * sizeof(uint32_t)) + 255) / 256 * 256; }
+static int g_pitch(int W) { return (W + 1) / 2 * 2; }
 
-int dt_run(const uint8_t *B, int H, int W, int *site, unsigned *d2, void *scratch, unsigned *h_cnt,
-           int grid, cudaStream_t st, int *levels_out)
+size_t dt_scratch_bytes(int H, int W) { return mask_bytes(H, W) + (size_t)H * g_pitch(W) * sizeof(uint16_t); }
+
+int dt_run(const uint8_t *B, int H, int W, int *site, unsigned *d2, void *scratch, int sms, cudaStream_t st)
 {
-    const size_t n = (size_t)H * W;
-    unsigned char *base = (unsigned char *)scratch;
-    unsigned *cnt = (unsigned *)base;      // cnt[0..2]
-    int *err = (int *)(base + 64);
-    int *stamp = (int *)(base + 256);
-    int *F[2] = {stamp + n, stamp + 2 * n};
-    if (cudaMemsetAsync(base, 0, 256, st) != cudaSuccess) return DT_ECUDA;   // counters, error word
-    dt::init_kernel<<<grid, 256, 0, st>>>(B, H, W, site, stamp, F[0], cnt);
-    if (cudaGetLastError() != cudaSuccess) return DT_ECUDA;
-    // every level improves some pixel's key; keys only decrease and each
-    // pixel's key has at most H*W + 1 values, but in practice a level count
-    // of a few times the largest distance suffices: bound it generously
-    const long long max_levels = 8ll * (H + W) + 1024;
-    constexpr int BATCH = 16;
-    int L = 0;
-    for (;;) {
-        for (int b = 0; b < BATCH; ++b, ++L) {
-            dt::level_kernel<<<grid, 256, 0, st>>>(B, H, W, site, stamp, F[L & 1], F[(L + 1) & 1], cnt, L, err);
-        }
-        if (cudaGetLastError() != cudaSuccess) return DT_ECUDA;
-        if (cudaMemcpyAsync(h_cnt, cnt, 4 * sizeof(unsigned), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return DT_ECUDA;
-        if (h_cnt[L % 3] == 0) break;   // level L has nothing to do: S is empty
-        if (L > max_levels) return DT_ELIMIT;
-    }
-    int herr = 0;
-    if (cudaMemcpy(&herr, err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return DT_ECUDA;
-    if (herr) return DT_ELIMIT;
-    dt::final_kernel<<<grid, 256, 0, st>>>(H, W, site, d2);
-    if (cudaGetLastError() != cudaSuccess) return DT_ECUDA;
-    if (levels_out) *levels_out = L;
-    return DT_OK;
+    uint32_t *M = (uint32_t *)scratch;
+    uint16_t *G = (uint16_t *)((unsigned char *)scratch + mask_bytes(H, W));
+    const int ns = (H + 31) / 32, pitch = g_pitch(W);
+    dt::mask_kernel<<<dim3((W + 511) / 512, ns), 128, 0, st>>>(B, H, W, M);
+    const dim3 cg((W + 255) / 256, ns);
+    if (site) dt::column_kernel<true><<<cg, 128, 0, st>>>(M, H, W, G, pitch);
+    else dt::column_kernel<false><<<cg, 128, 0, st>>>(M, H, W, G, pitch);
+    // a CTA per row; more threads where a wide row's shared memory leaves room for few CTAs
+    const int px = site ? W : (W + 1) / 2;
+    const int T = W > 8192 ? 1024 : std::min(256, (px + 31) / 32 * 32);
+    const size_t smem = sizeof(uint32_t) * ((size_t)(W + 1) / 2 * 2 + 2 * dt::PAD + 2 + (W + 31) / 32) +
+                        (site ? sizeof(uint16_t) * (size_t)W : 0);
+    const void *fn = site ? (const void *)dt::row_site_kernel : (const void *)dt::row_kernel;
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return DT_ECUDA;
+    const int grid = std::min(H, 64 * std::max(1, sms));
+    if (site) dt::row_site_kernel<<<grid, T, smem, st>>>(G, H, W, pitch, d2, site);
+    else dt::row_kernel<<<grid, T, smem, st>>>(G, H, W, pitch, d2);
+    return cudaGetLastError() == cudaSuccess ? DT_OK : DT_ECUDA;
 }
