@@ -448,9 +448,9 @@ static int stage_meta(recon_ctx *c, const recon_tile *tiles, int n, const int *v
 // engine: when the context's wavefront settings are all at their defaults.
 // Setting any of them (recon_set_param, RECON_*, recon_autotune) or passing
 // variants or an order asks for the wavefront engine. The merging engine was
-// faster at every size, marker, connectivity and operation measured, by 1.25
-// (4096^2, h-dome: 402 -> 323 us) to 16 times (3000^2, border-seeded: 4.42 ->
-// 0.28 ms), so there is no size below or above which the other is chosen.
+// faster at every size, marker, connectivity and operation measured, by 1.5
+// (4096^2, h-dome: 403 -> 272 us) to 18 times (3000^2, border-seeded: 4.26 ->
+// 0.24 ms), so there is no size below or above which the other is chosen.
 static bool use_forest(const recon_ctx *c)
 {
     return c->bh == 128 && c->k == 1 && c->grid == 0 && c->bands == 4 && c->use_tma == 1 && c->revisit_scans == 0 &&

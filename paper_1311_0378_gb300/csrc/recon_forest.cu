@@ -13,8 +13,8 @@
 // the wavefront (about 7 000 sequential levels on a border-seeded 4096^2 tile).
 //
 // Three launches per group of tiles, one CTA per 64 x 64 block:
-//   block_kernel  splits the block into the basins of its mask (every pixel
-//     follows its highest neighbour; R(p) = min(I(p), R(top of its basin))),
+//   block_kernel  splits the block into basins of its mask (every pixel follows
+//     a neighbour at least as high; R(p) = min(I(p), R(top of its basin))),
 //     lists the passes between them, which lie at the saddles of the mask, and
 //     runs Boruvka's rounds on that small graph.
 //     A region whose heaviest edge leads out of the block stops there: it
@@ -30,15 +30,17 @@
 // interleaving, and walks of logarithmic expected length.
 //
 // Measured on GB300 (whole call, the wavefront engine -> this one): a 4096^2
-// tile seeded from its border, 4-connected, 5.74 -> 0.457 ms; with an h-dome
-// marker, 8-connected, 0.402 -> 0.323 ms; 200 tiles of 256 .. 4096 pixels a
-// side (910 Mpx, both markers) 54.4 -> 15.3 ms; 512^2 0.235 -> 0.098 ms.
-// block_kernel takes most of it (0.33 of 0.40 ms of kernel time on the
-// border-seeded tile) and is bound by instruction issue (66% of the issue slots,
-// 49% of the shared-memory pipe; DRAM below 10%), so what counts is instructions
-// per pixel: saddles instead of all pixel pairs cut its time from 0.71 to 0.46 ms,
-// and code small enough for the instruction cache (rolled loops) to 0.33.
+// tile seeded from its border, 4-connected, 6.04 -> 0.346 ms; with an h-dome
+// marker, 8-connected, 0.403 -> 0.272 ms; 200 tiles of 256 .. 4096 pixels a
+// side (910 Mpx, both markers) 54.2 -> 12.3 ms; 512^2 0.231 -> 0.093 ms.
+// block_kernel takes most of it (0.22 of 0.29 ms of kernel time on the
+// border-seeded tile) and is bound by instruction issue and the shared-memory
+// pipe (about 65% and 50%; DRAM below 10%), so what counts is warp instructions
+// a block: 30 600 (h-dome) to 40 900 (border), 76 500 and 94 900 at first. Saddles instead of
+// all pixel pairs, arcs of four pixels at once in byte lanes, loops rolled to fit
+// the instruction cache, and lists that stay dense made the difference.
 #include <climits>
+#include <cstddef>
 #include "recon_forest.h"
 
 namespace rf {
@@ -67,26 +69,18 @@ struct Smem {
     static constexpr int NB = (CONN == 8 ? BPX / 4 : BPX / 2) + 32;
     alignas(16) uint16_t L[NCELL];    // labels: a cell number, or ROOT | basin
     alignas(16) uint32_t img[IMG];    // byte image of I, then the bytes of J
-    uint32_t tab[TAB];                // saddles, then passes: region << 20 | region << 8 | weight, 0 = none
+    uint32_t tab[TAB];                // passes: region << 20 | region << 8 | weight, 0 = none
     uint32_t best[NB];                // heaviest edge of a live region to a region or out of the block; FINAL, NODE
     uint32_t sv[NB];                  // its heaviest source edge
     uint16_t comp[NB], up[NB];        // region's root (at the end cap << 8 | node slot), link to the region merged into
     uint8_t capw[NB];                 // weight of the up link; a final root's value; a node root's slot
     uint32_t link[MAX_TERM];          // node links: weight << 8 | parent slot (RES = source)
     uint8_t hT[BS + 2], hB[BS + 2], hL[BS], hR[BS];   // mask of the pixels around the block
-    unsigned nb, nt, nsad, nmore;     // basins, nodes, saddles, passes beyond one per saddle
+    unsigned nb, nt, ne, nj;          // basins, nodes, passes, passes between nodes
+    unsigned nlive[2];                // live roots, by round parity
     int tile;
     unsigned local;
 };
-
-__device__ __forceinline__ uint32_t pmax(uint32_t a, uint32_t b)
-{
-    uint32_t r;
-    asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-__device__ __forceinline__ uint32_t even_plane(uint32_t w) { return __byte_perm(w, 0u, 0x4240); }
-__device__ __forceinline__ uint32_t odd_plane(uint32_t w) { return __byte_perm(w, 0u, 0x4341); }
 
 __device__ __forceinline__ unsigned long long now_ns()
 {
@@ -182,57 +176,49 @@ __device__ __forceinline__ int dir_off(unsigned d)
     return (int)r;
 }
 
-// One word of four pixels against its neighbours, even pixels in one u16x2
-// plane, odd ones in the other. rows: words left, centre, right of the rows
-// above, at and below. A neighbour is upper when it is higher, or equal and
-// later; as keys I << 3 | direction, when its key is at least I << 3 | 4.
-//   kE, kO: the largest key, i.e. the highest neighbour and its direction;
-//   returns a byte per pixel: the saddle arcs. The upper neighbours form arcs on
-// the ring around a pixel. Inside an arc they hang together without the pixel
-// (ring neighbours are adjacent; for 8-connectivity so are N and E and so on,
-// for 4-connectivity the corner between them must be upper too), so passes lie
-// only at pixels with two or more arcs: bit k is set where an arc starts (ring
-// order N, NE, E, SE, S, SW, W, NW), and no bit when there are fewer than two.
+// One word of four pixels (bytes) against its neighbours. rows: words left,
+// centre, right of the rows above, at and below. A neighbour is upper when it is
+// higher, or equal and later in the image. The upper neighbours form arcs on the
+// ring around a pixel (order N, NE, E, SE, S, SW, W, NW). Inside an arc they hang
+// together without the pixel: ring neighbours are adjacent; for 8-connectivity so
+// are N and E and so on, for 4-connectivity the corner between them must be upper
+// too. Returns a byte per pixel with bit k set where an arc starts; bit 0 (N) when
+// the ring is one closed arc; no bit when there is no upper neighbour.
 template <int CONN>
-__device__ __forceinline__ uint32_t classify(const uint32_t (&l)[3], const uint32_t (&c)[3], const uint32_t (&r)[3],
-                                             uint32_t &kE, uint32_t &kO)
+__device__ __forceinline__ uint32_t arc_starts(const uint32_t (&l)[3], const uint32_t (&c)[3], const uint32_t (&r)[3])
 {
-    uint32_t e[3], o[3], we[3], eo[3];
+    constexpr uint32_t H = 0x80808080u, ONES = 0x01010101u;
+    const uint32_t own = c[1], ol = own & ~H, oh = own | H;
+    uint32_t w[3], e[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        e[a] = even_plane(c[a]) << 3;
-        o[a] = odd_plane(c[a]) << 3;
-        we[a] = __funnelshift_l(odd_plane(l[a]) << 3, o[a], 16);    // left neighbours of the even pixels
-        eo[a] = __funnelshift_r(e[a], even_plane(r[a]) << 3, 16);   // right neighbours of the odd pixels
+        w[a] = __funnelshift_l(l[a], c[a], 8);   // left neighbours
+        e[a] = __funnelshift_r(c[a], r[a], 8);   // right neighbours
     }
-    auto plane = [](uint32_t nw, uint32_t n, uint32_t ne, uint32_t w, uint32_t own, uint32_t ea, uint32_t sw, uint32_t so,
-                    uint32_t se, uint32_t &key) {
-        // bit 15 of each lane is set so that the subtractions below do not borrow across lanes
-        const uint32_t k[8] = {n | 0x80018001u, ne | 0x80028002u, ea | 0x80048004u, se | 0x80078007u,
-                               so | 0x80068006u, sw | 0x80058005u, w | 0x80038003u, nw | 0x80008000u};
-        key = __vimax3_u16x2(k[0], k[2], k[4]);
-        key = pmax(key, k[6]);
-        if (CONN == 8) {
-            key = __vimax3_u16x2(key, k[1], k[3]);
-            key = __vimax3_u16x2(key, k[5], k[7]);
-        }
-        key &= 0x7FFF7FFFu;
-        const uint32_t ref = own | 0x00040004u;
-        uint32_t m = 0;   // upper neighbours in ring order
-#pragma unroll
-        for (int b = 0; b < 8; ++b) m |= ((k[b] - ref) >> (15 - b)) & (0x00010001u << b);
-        const uint32_t mm = m * 0x101u, both = (mm >> 1) & (mm >> 7) & 0x00AA00AAu;   // corners between two upper ones
-        m = CONN == 8 ? (m | both) : ((m & 0x00550055u) | (m & both));
-        const uint32_t s = m & ~((m * 0x101u) >> 7) & 0x00FF00FFu;                    // arc starts
-        const uint32_t two = s & ((s | 0x01000100u) - 0x00010001u);                   // nonzero with two or more
-        return s & ((((two & 0x00FF00FFu) + 0x00FF00FFu) >> 8 & 0x00010001u) * 0xFFu);
-    };
-    const uint32_t sE = plane(we[0], e[0], o[0], we[1], e[1], o[1], we[2], e[2], o[2], kE);
-    const uint32_t sO = plane(e[0], o[0], eo[0], e[1], o[1], eo[1], e[2], o[2], eo[2], kO);
-    return sE | sO << 8;
+    // high bit of each byte: a later neighbour is at least as high / an earlier one is higher.
+    // Bytes compare by their high bits, and where those agree by a subtraction of the low seven
+    // bits below a guard bit.
+    auto later = [&](uint32_t q) { const uint32_t t = (q | H) - ol; return (q & ~own) | (~(q ^ own) & t); };
+    auto earlier = [&](uint32_t q) { const uint32_t t = oh - (q & ~H); return ~((own & ~q) | (~(own ^ q) & t)); };
+    uint32_t m = (earlier(c[0]) >> 7) & ONES;
+    m |= (earlier(e[0]) >> 6) & (ONES << 1);
+    m |= (later(e[1]) >> 5) & (ONES << 2);
+    m |= (later(e[2]) >> 4) & (ONES << 3);
+    m |= (later(c[2]) >> 3) & (ONES << 4);
+    m |= (later(w[2]) >> 2) & (ONES << 5);
+    m |= (earlier(w[1]) >> 1) & (ONES << 6);
+    m |= earlier(w[0]) & H;
+    const uint32_t both = (((m >> 1) & 0x2A2A2A2Au) | ((m << 7) & H)) & (m << 1);   // corners (odd bits) between two upper ones
+    m = CONN == 8 ? (m | both) : ((m & 0x55555555u) | (m & both));
+    const uint32_t prev = ((m << 1) & 0xFEFEFEFEu) | ((m >> 7) & ONES);             // bit k: position k - 1 is upper
+    const uint32_t closed = ((m & ~H) + ONES) & m & H;
+    return (m & ~prev) | closed >> 7;
 }
 
-// Cell offset of ring position k (see classify).
+// High bit of each nonzero byte.
+__device__ __forceinline__ uint32_t nonzero_bytes(uint32_t v) { return (((v & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | v) & 0x80808080u; }
+
+// Cell offset of ring position k (see arc_starts).
 __device__ __forceinline__ int ring_off(unsigned k)
 {
     constexpr uint32_t LO = (uint32_t)(uint8_t)(-ST) | (uint32_t)(uint8_t)(-ST + 1) << 8 | 1u << 16 |
@@ -261,31 +247,32 @@ __device__ __forceinline__ bool join(F &f, unsigned a, unsigned b, unsigned w)
 {
     for (int it = 0; it < MAX_STEPS; ++it) {
         if (a == b) return true;
-        if (a == F::SOURCE || (b != F::SOURCE && f.before(b, a))) { const unsigned x = a; a = b; b = x; }
-        // a: the node of lower priority; step towards its root at weight w
-        const auto la = f.load(a);
-        if (f.weight(la) >= w) {
-            a = f.parent(la);
-            continue;
-        }
-        if (b != F::SOURCE) {
-            const auto lb = f.load(b);
-            if (f.weight(lb) >= w) {
-                b = f.parent(lb);
-                continue;
-            }
-        }
-        if (f.cas(a, la, f.word(w, b))) {   // displaced: a's former parent, at its lighter weight
-            a = b;
-            b = f.parent(la);
-            w = f.weight(la);
+        // both ends step towards their roots at weight w; the source is its own root
+        const typename F::Word la = a == F::SOURCE ? 0 : f.load(a), lb = b == F::SOURCE ? 0 : f.load(b);
+        const bool ua = a != F::SOURCE && f.weight(la) >= w, ub = b != F::SOURCE && f.weight(lb) >= w;
+        if (ua) a = f.parent(la);
+        if (ub) b = f.parent(lb);
+        if (ua || ub) continue;
+        // two roots: the one of lower priority is linked, and what that displaces (its former
+        // parent, at a lighter weight) is added next
+        const bool swap = a == F::SOURCE || (b != F::SOURCE && f.before(b, a));
+        const unsigned lo = swap ? b : a, hi = swap ? a : b;
+        const typename F::Word l = swap ? lb : la;
+        if (f.cas(lo, l, f.word(w, hi))) {
+            a = hi;
+            b = f.parent(l);
+            w = f.weight(l);
             if (w == 0) return true;        // every node reaches the source at weight 0
+        } else {
+            a = lo;
+            b = hi;
         }
     }
     return false;
 }
 
 struct SharedLinks {
+    typedef uint32_t Word;
     static constexpr unsigned SOURCE = RES;
     uint32_t *link;
     unsigned base;
@@ -298,6 +285,7 @@ struct SharedLinks {
 };
 
 struct GlobalLinks {
+    typedef unsigned long long Word;
     static constexpr unsigned SOURCE = SRC;
     unsigned long long *link;
     __device__ unsigned long long load(unsigned n) const { return *(volatile unsigned long long *)&link[n]; }
@@ -345,8 +333,9 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
             S.local = blk - P.base[t];
             S.nb = 1;
             S.nt = 0;
-            S.nsad = 0;
-            S.nmore = 0;
+            S.ne = 0;
+            S.nj = 0;
+            S.nlive[0] = S.nlive[1] = 0;
         }
     }
     __syncthreads();
@@ -417,7 +406,7 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
             S.L[(tid + 1) * ST + X0 - 1] = ROOT;
             S.L[(tid + 2) * ST] = ROOT;
         }
-        if (tid == 0) { S.sv[0] = 0u; S.best[0] = 0u; }
+        if (tid == 0) { S.sv[0] = 0u; S.capw[0] = 0; }
         bool bad = false;
         if (P.check && !D.fill)
             bad = (__vcmpgtu4(vj.x, vi.x) | __vcmpgtu4(vj.y, vi.y) | __vcmpgtu4(vj.z, vi.z) | __vcmpgtu4(vj.w, vi.w)) != 0;
@@ -432,10 +421,10 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
     }
 
     if (tid == 0) tick[1] = now_ns();
-    // Basins: every pixel points to its highest neighbour (the later one of
-    // equals), if that one is higher or equal and later; the others are tops.
+    // Basins: every pixel points to the first upper neighbour of its first arc
+    // (its heaviest edges all weigh its own height); pixels without one are tops.
     // A warp takes two rows at a time, a lane one word of four pixels (a loop,
-    // not unrolled: this kernel is bound by instruction fetch before anything else).
+    // not unrolled: code that does not fit the instruction cache costs more).
 #pragma unroll 1
     for (int it = 0; it < BS / 2; it += NT / 32) {
         const int row = 2 * (it + warp) + (lane >> 4), cw = lane & 15;
@@ -443,21 +432,13 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
         const uint32_t l[3] = {at[-IST - 1], at[-1], at[IST - 1]};
         const uint32_t m[3] = {at[-IST], at[0], at[IST]};
         const uint32_t q[3] = {at[-IST + 1], at[1], at[IST + 1]};
-        uint32_t kE, kO;
-        const uint32_t saddle = classify<CONN>(l, m, q, kE, kO);
-        const uint32_t k4[4] = {kE & 0xFFFFu, kO & 0xFFFFu, kE >> 16, kO >> 16};
+        const uint32_t high = nonzero_bytes(m[1]);   // pixels of height 0 have value 0, like the outside (basin 0)
+        const uint32_t starts = arc_starts<CONN>(l, m, q) & ((high >> 7) * 255u);
+        const uint32_t rest = starts & ((starts | 0x80808080u) - 0x01010101u);   // without the lowest: further arcs
+        const uint32_t tops = high & ~nonzero_bytes(starts);
         const int cell = (row + 1) * ST + X0 + 4 * cw;
-        uint32_t f[4], arcs[4];
-        unsigned top[4], mine = 0;   // tops in the low half, saddles in the high half
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const uint32_t v = (m[1] >> (8 * b)) & 255u;
-            // height 0 has value 0, like the outside (basin 0)
-            f[b] = v ? (uint32_t)(cell + b + dir_off(k4[b] & 7u)) : ROOT;
-            top[b] = v && k4[b] < (v << 3 | 4u);
-            arcs[b] = v ? (saddle >> (8 * b)) & 255u : 0u;
-            mine += top[b] | (arcs[b] ? 0x10000u : 0u);
-        }
+        // numbers for the tops (low half), places for the passes (high half)
+        const unsigned mine = __popc(tops) | __popc(rest) << 16;
         unsigned incl = mine;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
@@ -467,25 +448,31 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
         unsigned id = 0, slot = 0;
         if (lane == 31) {
             id = atomicAdd(&S.nb, incl & 0xFFFFu);
-            slot = atomicAdd(&S.nsad, incl >> 16);
+            slot = atomicAdd(&S.ne, incl >> 16);
         }
         id = __shfl_sync(FULL, id, 31) + ((incl - mine) & 0xFFFFu);
         slot = __shfl_sync(FULL, slot, 31) + ((incl - mine) >> 16);
         const uint32_t jw = bj[row * (BS / 4) + cw];
+        uint32_t f[4];
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            if (top[b]) {
-                S.sv[id] = (jw >> (8 * b)) & 255u;   // the top's own source edge
-                S.best[id] = 0u;
-                f[b] = ROOT | id++;
-            }
-            // a saddle: weight << 24 | cell << 11 | direction of the highest neighbour << 8 | arc starts
-            if (arcs[b]) {
-                if (slot < TAB) S.tab[slot] = (m[1] >> (8 * b)) << 24 | (uint32_t)(cell + b) << 11 | (k4[b] & 7u) << 8 | arcs[b];
-                ++slot;
-            }
+            const uint32_t sb = (starts >> (8 * b)) & 255u;
+            f[b] = sb ? (uint32_t)(cell + b + ring_off(__ffs(sb) - 1)) : ROOT;
         }
         *(uint2 *)&S.L[cell] = make_uint2(f[0] | f[1] << 16, f[2] | f[3] << 16);
+        asm volatile("" ::: "memory");   // the tops' labels, of another type, come after
+#pragma unroll 1
+        for (uint32_t bits = tops; bits; bits &= bits - 1, ++id) {
+            const unsigned k = __ffs(bits) >> 3;         // (high bits of the bytes: 8, 16, 24, 32)
+            S.L[cell + (int)k - 1] = (uint16_t)(ROOT | id);
+            S.sv[id] = (jw >> (8 * k - 8)) & 255u;       // the top's own source edge
+        }
+        // a pass lies at a pixel and leads to a further arc of it: weight << 16 | cell << 3 | ring position
+#pragma unroll 1
+        for (uint32_t bits = rest; bits; bits &= bits - 1, ++slot) {
+            const unsigned k = __ffs(bits) - 1;
+            if (slot < TAB) S.tab[slot] = ((m[1] >> (k & 24u)) & 255u) << 16 | (unsigned)(cell + (int)(k >> 3)) << 3 | (k & 7u);
+        }
     }
     __syncthreads();
     const unsigned nb = S.nb;
@@ -493,74 +480,97 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
     // takes its target's label until that is a basin; all warps do so at once,
     // so paths halve as they are walked (each step goes to a higher (value,
     // number), so they end). 16 pixels a thread, their loads in flight together.
+#pragma unroll 1
+    for (unsigned b = tid; b < nb; b += NT) {
+        S.best[b] = b ? 0u : FINAL;   // (the outside has value 0)
+        S.up[b] = S.comp[b] = (uint16_t)b;
+    }
     {
-        const int p0 = ((warp >> 1) * 16 + 1) * ST + X0 + (warp & 1) * 32 + lane;   // 32 columns x 16 rows a warp
         volatile uint16_t *L = S.L;
-        const uint8_t *jb = (const uint8_t *)bj + (warp >> 1) * 16 * BS + (warp & 1) * 32 + lane;
+        const int row0 = 2 * warp + (lane >> 4), cw = lane & 15;   // words as above: rows row0 + 16 i
+        uint2 *const word = (uint2 *)&S.L[(row0 + 1) * ST + X0 + 4 * cw];
+        constexpr int STEP = 16 * ST / 4;
         unsigned l[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) l[i] = L[p0 + i * ST];
-        bool more = true;
-        while (more) {
+        for (int i = 0; i < 4; ++i) {
+            const uint2 v = word[i * STEP];
+            l[4 * i] = v.x & 0xFFFFu;
+            l[4 * i + 1] = v.x >> 16;
+            l[4 * i + 2] = v.y & 0xFFFFu;
+            l[4 * i + 3] = v.y >> 16;
+        }
+        for (;;) {
+            unsigned all = ROOT;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) all &= l[k];
+            if (all) break;
             unsigned n[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) n[i] = (l[i] & ROOT) ? l[i] : L[l[i]];
-            more = false;
+            for (int k = 0; k < 16; ++k) n[k] = (l[k] & ROOT) ? l[k] : L[l[k]];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                if (n[i] != l[i]) L[p0 + i * ST] = (uint16_t)n[i];
-                l[i] = n[i];
-                more |= !(n[i] & ROOT);
+            for (int i = 0; i < 4; ++i) {
+                *(volatile uint32_t *)&word[i * STEP].x = n[4 * i] | n[4 * i + 1] << 16;
+                *(volatile uint32_t *)&word[i * STEP].y = n[4 * i + 2] | n[4 * i + 3] << 16;
             }
+#pragma unroll
+            for (int k = 0; k < 16; ++k) l[k] = n[k];
         }
         unsigned over = 0;   // pixels with a heavier source edge than their basin has so far
 #pragma unroll
-        for (int i = 0; i < 16; ++i) over |= (jb[i * BS] > S.sv[l[i] & 0x7FFFu] ? 1u : 0u) << i;
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t jw = bj[(row0 + 16 * i) * (BS / 4) + cw];
+            if (jw == 0u) continue;
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                over |= (((jw >> (8 * b)) & 255u) > S.sv[l[4 * i + b] & 0x7FFFu] ? 1u : 0u) << (4 * i + b);
+        }
 #pragma unroll 1
         for (; over; over &= over - 1) {
-            const int i = __ffs(over) - 1;
-            atomicMax(&S.sv[S.L[p0 + i * ST] & 0x7FFFu], (uint32_t)jb[i * BS]);
+            const int k = __ffs(over) - 1, i = k >> 2, row = row0 + 16 * i;
+            const unsigned j = ((const uint8_t *)bj)[row * BS + 4 * cw + (k & 3)];
+            atomicMax(&S.sv[S.L[(row + 1) * ST + X0 + 4 * cw + (k & 3)] & 0x7FFFu], j);
         }
     }
     __syncthreads();
     if (tid == 0) tick[2] = now_ns();
+    // (a predicated reduction: no branch, and no atomic when the key does not raise the maximum)
+    const unsigned best0 = (unsigned)__cvta_generic_to_shared(S.best);
     auto offer = [&](unsigned a, uint32_t key) {
-        if (key > *(volatile uint32_t *)&S.best[a]) atomicMax(&S.best[a], key);
+        asm volatile("{\n .reg .pred p;\n .reg .u32 c;\n ld.volatile.shared.u32 c, [%0];\n setp.gt.u32 p, %1, c;\n"
+                     " @p red.shared.max.u32 [%0], %1;\n}" :: "r"(best0 + 4u * a), "r"(key) : "memory");
     };
-    // Passes: a saddle joins its own basin to the one each arc starts in. The
-    // arc of its highest neighbour needs none (that is its own basin): with the
-    // ring turned so that this neighbour comes last, its arc's start is the
-    // last one set. A pass no heavier than the source edges of both ends is
-    // never taken. A saddle's first pass takes the saddle's place in the list,
-    // further ones follow behind. The first round's maxima are taken here too.
-    const unsigned nsad = S.nsad;
-    if (nsad <= TAB) {
+    // Passes join a saddle's own basin to the one the arc starts in. A pass no
+    // heavier than the source edges of both ends is never taken. The first
+    // round's maxima are taken here too.
+    const unsigned ne = S.ne;
+    const bool listed = ne <= TAB;   // else: pairs of pixels instead of passes
+    // Each warp has an eighth of the list to itself and keeps it dense: what a
+    // pass (of the kernel over the list) drops is closed up, places only shrink.
+    const unsigned seg0 = listed ? (ne * warp) / (NT / 32) : 0u;
+    unsigned mine = listed ? (ne * (warp + 1)) / (NT / 32) - seg0 : 0u;   // the warp's passes
+    auto close_up = [&](unsigned &to, uint32_t e) {   // keeps nonzero e; returns its place (warp-wide)
+        const unsigned keep = __ballot_sync(FULL, e != 0u), at = to + __popc(keep & ((1u << lane) - 1u));
+        if (e) S.tab[at] = e;
+        to += __popc(keep);
+        return at;
+    };
+    {
+        unsigned to = seg0;
 #pragma unroll 1
-        for (unsigned i = tid; i < nsad; i += NT) {
-            const uint32_t e = S.tab[i], p = (e >> 11) & 0x1FFFu, w = e >> 24;
-            const unsigned turn = ((0x34526107u >> (4 * ((e >> 8) & 7u))) & 7u) + 1u;   // that neighbour's ring position + 1
-            uint32_t arcs = e & 255u, first = 0u;
-            arcs &= ~(1u << ((31 - __clz((arcs * 0x101u >> turn) & 255u) + turn) & 7u));
-            const unsigned a = S.L[p] & 0x7FFFu;
-            const bool above = w > S.sv[a];
-#pragma unroll 1
-            for (; arcs; arcs &= arcs - 1) {
-                const unsigned b = S.L[(int)p + ring_off(__ffs(arcs) - 1)] & 0x7FFFu;
-                if (a == b || !(above || w > S.sv[b])) continue;
-                const uint32_t n = a << 20 | b << 8 | w;
-                unsigned at = i;
-                if (first == 0u) {
-                    first = n;
-                } else {
-                    at = atomicAdd(&S.nmore, 1u) + nsad;
-                    if (at >= TAB) break;
-                    S.tab[at] = n;
-                }
-                offer(a, w << 24 | K_EDGE | at);
-                offer(b, w << 24 | K_EDGE | at);
+        for (unsigned k = 0; k < mine; k += 32) {
+            uint32_t n = 0u;
+            if (k + lane < mine) {
+                const uint32_t e = S.tab[seg0 + k + lane], p = (e >> 3) & 0x1FFFu, w = e >> 16;
+                const unsigned a = S.L[p] & 0x7FFFu, b = S.L[(int)p + ring_off(e & 7u)] & 0x7FFFu;
+                if (a != b && (w > S.sv[a] || w > S.sv[b])) n = a << 20 | b << 8 | w;
             }
-            S.tab[i] = first;
+            const unsigned at = close_up(to, n);
+            if (n) {
+                offer(n >> 20, n << 24 | K_EDGE | at);
+                offer((n >> 8) & 0xFFFu, n << 24 | K_EDGE | at);
+            }
         }
+        mine = to - seg0;
     }
     // this thread's edge out of the block: pixel tid & 63 of side tid >> 6 (top, bottom, left, right)
     unsigned ob, ow;
@@ -577,17 +587,10 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
         ob = S.L[(py + 1) * ST + X0 + px] & 0x7FFFu;
         if (ow) offer(ob, ow << 24 | K_OUT);
     }
-#pragma unroll 1
-    for (unsigned b = tid; b < nb; b += NT) {
-        S.comp[b] = (uint16_t)b;
-        S.up[b] = (uint16_t)b;
-    }
     __syncthreads();
-    const unsigned ne = nsad + S.nmore;
-    const bool listed = ne <= TAB;   // else: pairs of pixels instead of passes
     if (!listed) {
 #pragma unroll 1
-        for (unsigned b = tid; b < nb; b += NT) S.best[b] = 0u;
+        for (unsigned b = 1 + tid; b < nb; b += NT) S.best[b] = 0u;
         __syncthreads();
     }
 
@@ -596,24 +599,48 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
     // source, to another region (numbers break ties, the same for both ends,
     // so only the two ends of one edge can choose each other) or out of the
     // block, where it stops as a node.
+    // Live roots: in the first round all basins, then a list, which at least
+    // halves with every round (a live root stops, merges or takes in another):
+    // one of NB / 2 places for the odd rounds, one of NB / 4 for the even ones,
+    // where the bytes of J were.
+    uint16_t *const lists = (uint16_t *)bj;
+    static_assert(Smem<CONN>::NB / 2 + Smem<CONN>::NB / 4 <= BPX / 2, "lists");
+    unsigned nlive = nb - 1;
     int rounds = 0;
     for (;; ++rounds) {
+        const uint16_t *now = lists + (rounds & 1 ? 0 : Smem<CONN>::NB / 2);
+        uint16_t *next = lists + (rounds & 1 ? Smem<CONN>::NB / 2 : 0);
         // edges: to their present ends; one inside a region is dropped
         if (rounds || !listed) {
-            if (ow) offer(S.comp[ob], ow << 24 | K_OUT);
+            if (tid == 0) S.nlive[rounds & 1] = 0;   // last read two rounds ago
+            ob = S.comp[ob];
+            if (ow) offer(ob, ow << 24 | K_OUT);
             if (listed) {
+                unsigned to = seg0;
 #pragma unroll 1
-                for (unsigned i = tid; i < ne; i += NT) {
-                    uint32_t e = S.tab[i];
-                    if (e == 0u) continue;
-                    const unsigned a = S.comp[e >> 20], b = S.comp[(e >> 8) & 0xFFFu];
-                    const uint32_t n = a == b ? 0u : (a << 20 | b << 8 | (e & 255u));
-                    if (n != e) S.tab[i] = n;
-                    if (n == 0u) continue;
-                    offer(a, e << 24 | K_EDGE | i);
-                    offer(b, e << 24 | K_EDGE | i);
+                for (unsigned k = 0; k < mine; k += 32) {
+                    uint32_t n = 0u;
+                    if (k + lane < mine) {
+                        const uint32_t e = S.tab[seg0 + k + lane];
+                        const unsigned a = S.comp[e >> 20], b = S.comp[(e >> 8) & 0xFFFu];
+                        if (a != b) n = a << 20 | b << 8 | (e & 255u);
+                    }
+                    const unsigned at = close_up(to, n);
+                    if (n) {
+                        offer(n >> 20, n << 24 | K_EDGE | at);
+                        offer((n >> 8) & 0xFFFu, n << 24 | K_EDGE | at);
+                    }
                 }
+                mine = to - seg0;
             } else {
+#pragma unroll 1
+                for (unsigned b = 1 + tid; b < nb; b += NT) {   // all pixels' basins need their roots
+                    unsigned t = b;
+#pragma unroll 1
+                    for (unsigned u; (u = S.up[t]) != t;) t = u;
+                    S.comp[b] = (uint16_t)t;
+                }
+                __syncthreads();
                 each_pair(S, [&](unsigned a, unsigned b, unsigned w, unsigned i) {
                     a = S.comp[a];
                     b = S.comp[b];
@@ -625,10 +652,9 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
             __syncthreads();
         }
 #pragma unroll 1
-        for (unsigned b = tid; b < nb; b += NT) {
-            if (S.up[b] != b) continue;
+        for (unsigned k = tid; k < nlive; k += NT) {
+            const unsigned b = rounds ? now[k] : k + 1;
             const uint32_t key = S.best[b], src = S.sv[b] << 24 | K_SOURCE;
-            if (key >= FINAL) continue;
             if (src > key) {
                 S.capw[b] = (uint8_t)(src >> 24);
                 *(volatile uint32_t *)&S.best[b] = FINAL;
@@ -657,33 +683,35 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
             S.capw[b] = (uint8_t)(key >> 24);
         }
         __syncthreads();
-        bool live = false;
+        // the live roots' new roots (the list and `ob` name no others), and what they bring along
 #pragma unroll 1
-        for (unsigned b = tid; b < nb; b += NT) {
-            const unsigned was = S.comp[b];
-            unsigned t = was;
+        for (unsigned k = tid; k < nlive; k += NT) {
+            const unsigned b = rounds ? now[k] : k + 1;
+            unsigned t = b;
 #pragma unroll 1
-            while (S.up[t] != t) t = S.up[t];
-            if (t != was) {
+            for (unsigned u; (u = S.up[t]) != t;) t = u;
+            if (t != b) {   // merged this round
                 S.comp[b] = (uint16_t)t;
-                if (was == b && S.sv[b] > *(volatile uint32_t *)&S.sv[t]) atomicMax(&S.sv[t], S.sv[b]);   // merged this round
-            } else if (t == b && S.best[b] < FINAL) {
-                live = true;
+                if (S.sv[b] > *(volatile uint32_t *)&S.sv[t]) atomicMax(&S.sv[t], S.sv[b]);
+            } else if (S.best[b] < FINAL) {
                 S.best[b] = 0u;
+                next[atomicAdd(&S.nlive[rounds & 1], 1u)] = (uint16_t)b;
             }
         }
-        if (!__syncthreads_or(live)) break;
+        __syncthreads();
+        nlive = S.nlive[rounds & 1];
+        if (nlive == 0) break;
     }
 
     // Per basin its cap (or final value) and node, cap << 8 | node slot, in comp.
     const unsigned nt = S.nt;
 #pragma unroll 1
     for (unsigned b = tid; b < nb; b += NT) {
-        const unsigned root = S.comp[b];
-        const bool node = S.best[root] == NODE;
-        unsigned v = node ? 255u : S.capw[root];
+        unsigned v = 255u, root = b;
 #pragma unroll 1
-        for (unsigned t = b; t != root; t = S.up[t]) v = min(v, (unsigned)S.capw[t]);
+        for (unsigned t; (t = S.up[root]) != root; root = t) v = min(v, (unsigned)S.capw[root]);
+        const bool node = S.best[root] == NODE;
+        if (!node) v = min(v, (unsigned)S.capw[root]);
         S.comp[b] = (uint16_t)(v << 8 | (node ? S.capw[root] : RES));
         if (node && b == root) S.link[S.capw[b]] = S.sv[b] << 8 | RES;
     }
@@ -700,11 +728,14 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
             if ((w << 8 | RES) > *(volatile uint32_t *)l) atomicMax(l, w << 8 | RES);
             return 0u;
         };
+        // (best and sv, next to each other, are no longer needed: room for every pass)
+        uint32_t *const joins = S.best;
+        static_assert(2 * Smem<CONN>::NB >= TAB && offsetof(Smem<CONN>, sv) == offsetof(Smem<CONN>, best) + sizeof(S.best), "joins");
         if (listed) {
 #pragma unroll 1
-            for (unsigned i = tid; i < ne; i += NT) {
-                const uint32_t e = S.tab[i];
-                if (e) S.tab[i] = ends(e >> 20, (e >> 8) & 0xFFFu, e & 255u);
+            for (unsigned k = lane; k < mine; k += 32) {
+                const uint32_t e = S.tab[seg0 + k], z = ends(e >> 20, (e >> 8) & 0xFFFu, e & 255u);
+                if (z) joins[atomicAdd(&S.nj, 1u)] = z;   // gathered, so that whole warps join
             }
         } else {
             each_pair(S, [&](unsigned a, unsigned b, unsigned w, unsigned) { ends(a, b, w); });
@@ -713,10 +744,11 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
         SharedLinks F{S.link, blk * MAX_TERM};
         bool ok = true;
         if (listed) {
+            const unsigned nj = S.nj;
 #pragma unroll 1
-            for (unsigned i = tid; i < ne; i += NT) {
-                const uint32_t e = S.tab[i];
-                if (e) ok &= join(F, e >> 16, (e >> 8) & 255u, e & 255u);
+            for (unsigned i = tid; i < nj; i += NT) {
+                const uint32_t e = joins[i];
+                ok &= join(F, e >> 16, (e >> 8) & 255u, e & 255u);
             }
         } else {
             // (the sources' part was done above; links may now point to nodes)
