@@ -552,7 +552,7 @@ static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, int *done)
         P.px = (uint16_t *)c->d_forest;
         P.link = (unsigned long long *)(P.px + nb * rf::BPX);
         P.rim = (uint16_t *)(P.link + nb * rf::MAX_TERM);
-        P.nterm = (unsigned *)(P.rim + nb * 4 * rf::BS);
+        P.block = (rf::Block *)(P.rim + nb * 4 * rf::BS);
         P.ctl = c->last_ctl;
         P.tile_err = (int *)(c->d_fmeta + off_err);
         P.work = c->last_work;

@@ -317,8 +317,10 @@ __device__ __noinline__ void each_pair(Smem<CONN> &S, F f)
     }
 }
 
+// Five CTAs an SM where shared memory allows it (8-connectivity: 43 KB; 4: 56 KB
+// for twice the basins): 10.95 ms on the 910 Mpx batch, 11.13 with four.
 template <int CONN>
-__global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
+__global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(Params P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Smem<CONN> &S = *reinterpret_cast<Smem<CONN> *>(smem_raw);
@@ -414,7 +416,7 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
             if (tid == 0) {
                 atomicExch(&P.tile_err[D.index], 2);
                 atomicMin(&P.ctl->err_tile, D.index);
-                P.nterm[blk] = 0;
+                P.block[blk] = Block{S.tile, S.local, D.nbx, 0u};
             }
             return;
         }
@@ -768,7 +770,9 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
                 (unsigned long long)(l >> 8) << 32 | (par == RES ? SRC : blk * MAX_TERM + par);
         }
     }
-    if (tid == 0) P.nterm[blk] = nt;
+    if (tid == 0)
+        P.block[blk] = Block{S.tile, S.local, D.nbx,
+                             nt | (bx + 1 < D.nbx ? B_RIGHT : 0u) | (by + 1 < D.nby ? B_DOWN : 0u) | (by > 0 ? B_UP : 0u)};
 
     if (tid == 0) tick[4] = now_ns();
     // Results: the pixels themselves when everything is final, else (cap, node)
@@ -825,61 +829,71 @@ __global__ void __launch_bounds__(NT, 4) block_kernel(Params P)
 
 // Joins across block borders: a CTA of 128 threads handles the edges from its
 // block's right column (warps 0, 1) and bottom row (warps 2, 3) to the blocks
-// E, NE, SE and S, SW of it (the other diagonals belong to those blocks).
-// Lanes that hold the same pair of nodes let the heaviest edge stand for all.
+// E, NE, SE and S, SW of it (the other diagonals belong to those blocks). Bound
+// by the latency of dependent loads (walks are 1 to 6 links long on average, L2
+// accesses each), so everything before the walks takes two, and a lane whose
+// neighbour holds the same two nodes with a heavier edge leaves it to that lane.
+// 20 us on a 4096^2 h-dome tile, 27 us seeded from the border (34 and 40 us with a
+// search for the tile first and a warp-wide match and maximum before each join).
 template <int CONN>
 __global__ void __launch_bounds__(128) rim_kernel(Params P)
 {
-    __shared__ int s_tile;
-    if (threadIdx.x < 32) {
-        const int t = find_tile(P, blockIdx.x);
-        if (threadIdx.x == 0) s_tile = t;
-    }
-    __syncthreads();
-    const Tile D = P.tiles[s_tile];
-    if (*(volatile int *)&P.tile_err[D.index]) return;
-    const unsigned blk = blockIdx.x, local = blk - P.base[s_tile];
-    const int by = (int)(local / (unsigned)D.nbx), bx = (int)(local - (unsigned)by * D.nbx);
+    const unsigned blk = blockIdx.x;
     const bool right = threadIdx.x < 64;
-    const int k = threadIdx.x & 63;
-    if (right ? bx + 1 >= D.nbx : by + 1 >= D.nby) return;   // warp-uniform
-    const uint16_t *rim = P.rim + (size_t)blk * 4 * BS;
-    const unsigned pv = right ? rim[3 * BS + k] : rim[BS + k];
+    const int k = threadIdx.x & 63, lane = threadIdx.x & 31;
+    const Block B = P.block[blk];
+    const unsigned pv = P.rim[(size_t)blk * 4 * BS + (right ? 3 * BS : BS) + k];
+    if (!(B.nterm & (right ? B_RIGHT : B_DOWN))) return;   // warp-uniform
+    const bool failed = P.tile_err[P.tiles[B.tile].index] != 0;
+    // opposite pixels k, k - 1, k + 1: their line in the block across, or a corner of the next one
+    constexpr int ND = CONN == 8 ? 3 : 1;
+    unsigned qn[ND], w[ND];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        const int q = k + (d == 0 ? 0 : 2 * d - 3);
+        unsigned nb = right ? blk + 1 : blk + B.nbx;
+        int at = right ? 2 * BS + q : q;                  // left column / top row
+        bool there = true;
+        if (q < 0) {                                      // NE: its bottom row, x = 0
+            there = right && (B.nterm & B_UP);
+            nb = blk + 1 - B.nbx;
+            at = BS;
+        } else if (q >= BS) {                             // SE: its top row, x = 0
+            there = right && (B.nterm & B_DOWN);
+            nb = blk + 1 + B.nbx;
+            at = 0;
+        }
+        const unsigned qv = there ? P.rim[(size_t)nb * 4 * BS + at] : RES;
+        qn[d] = (qv & 255u) == RES ? SRC : nb * MAX_TERM + (qv & 255u);
+        w[d] = min(pv >> 8, qv >> 8);
+    }
+    if (failed) return;
     const unsigned pn = (pv & 255u) == RES ? SRC : blk * MAX_TERM + (pv & 255u);
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        if (pn == qn[d]) w[d] = 0;
+#pragma unroll
+        for (int e = 0; e < d; ++e)
+            if (qn[e] == qn[d]) {
+                w[e] = max(w[e], w[d]);
+                w[d] = 0;
+            }
+    }
     GlobalLinks F{P.link};
     bool ok = true;
 #pragma unroll
-    for (int d = -1; d <= 1; ++d) {
-        if (CONN == 4 && d != 0) continue;
-        unsigned qn = SRC, w = 0;
-        const int q = k + d;
-        unsigned nb = 0;
-        const uint16_t *src = nullptr;
-        if (right) {
-            if (q < 0) {
-                if (by > 0) { nb = blk + 1 - D.nbx; src = P.rim + (size_t)nb * 4 * BS + BS; }          // NE: its bottom row, x = 0
-            } else if (q >= BS) {
-                if (by + 1 < D.nby) { nb = blk + 1 + D.nbx; src = P.rim + (size_t)nb * 4 * BS; }       // SE: its top row, x = 0
-            } else {
-                nb = blk + 1;
-                src = P.rim + (size_t)nb * 4 * BS + 2 * BS + q;
-            }
-        } else if (q >= 0 && q < BS) {
-            nb = blk + D.nbx;
-            src = P.rim + (size_t)nb * 4 * BS + q;
-        }
-        if (src) {
-            const unsigned qv = *src;
-            qn = (qv & 255u) == RES ? SRC : nb * MAX_TERM + (qv & 255u);
-            w = min(pv >> 8, qv >> 8);
-        }
-        if (pn == qn) w = 0;
-        const unsigned long long pair = (unsigned long long)pn << 32 | qn;
-        const unsigned same = __match_any_sync(FULL, pair);
-        const unsigned top = __reduce_max_sync(same, w);
-        const unsigned ties = __ballot_sync(FULL, w && w == top) & same;
-        if (ties && __ffs(ties) - 1 == (int)(threadIdx.x & 31)) ok &= join(F, pn, qn, w);
-        __syncwarp();
+    for (int d = 0; d < ND; ++d) {
+        const unsigned pl = __shfl_up_sync(FULL, pn, 1), ql = __shfl_up_sync(FULL, qn[d], 1), wl = __shfl_up_sync(FULL, w[d], 1);
+        const unsigned pr = __shfl_down_sync(FULL, pn, 1), qr = __shfl_down_sync(FULL, qn[d], 1),
+                       wr = __shfl_down_sync(FULL, w[d], 1);
+        if (lane > 0 && pl == pn && ql == qn[d] && wl >= w[d]) w[d] = 0;
+        if (lane < 31 && pr == pn && qr == qn[d] && wr > w[d]) w[d] = 0;
+    }
+#pragma unroll 1
+    for (int d = 0; d < ND; ++d) {
+        const unsigned n = d == 0 ? qn[0] : (d == 1 ? qn[ND > 1 ? 1 : 0] : qn[ND > 2 ? 2 : 0]);
+        const unsigned v = d == 0 ? w[0] : (d == 1 ? w[ND > 1 ? 1 : 0] : w[ND > 2 ? 2 : 0]);
+        if (v) ok &= join(F, pn, n, v);
     }
     if (!ok) atomicCAS(&P.ctl->abort, 0, (int)rk::AB_MERGE);
 }
@@ -888,18 +902,15 @@ __global__ void __launch_bounds__(128) rim_kernel(Params P)
 // of its pixels.
 __global__ void __launch_bounds__(NT) value_kernel(Params P)
 {
-    __shared__ int s_tile;
     __shared__ uint8_t R[256];
     const unsigned blk = blockIdx.x;
-    const unsigned nt = P.nterm[blk];
-    if (nt == 0) return;
-    if (threadIdx.x < 32) {
-        const int t = find_tile(P, blk);
-        if (threadIdx.x == 0) s_tile = t;
-    }
     const int r = threadIdx.x >> 2, c = threadIdx.x & 3;
+    const Block B = P.block[blk];
+    const unsigned nt = B.nterm & 255u;
+    if (nt == 0) return;
     const uint4 *src = (const uint4 *)(P.px + (size_t)blk * BPX + r * BS + 16 * c);
     const uint4 q0 = src[0], q1 = src[1];
+    const Tile D = P.tiles[B.tile];
     R[threadIdx.x] = 255;
     if (threadIdx.x < nt) {
         unsigned n = blk * MAX_TERM + threadIdx.x, v = 255;
@@ -914,10 +925,8 @@ __global__ void __launch_bounds__(NT) value_kernel(Params P)
         R[threadIdx.x] = (uint8_t)v;
     }
     __syncthreads();
-    const Tile D = P.tiles[s_tile];
     if (P.tile_err[D.index]) return;
-    const unsigned local = blk - P.base[s_tile];
-    const int by = (int)(local / (unsigned)D.nbx), bx = (int)(local - (unsigned)by * D.nbx);
+    const int by = (int)(B.local / (unsigned)B.nbx), bx = (int)(B.local - (unsigned)by * B.nbx);
     const int y = by * BS + r, x = bx * BS + 16 * c;
     if (y >= D.H) return;
     const uint32_t o[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};

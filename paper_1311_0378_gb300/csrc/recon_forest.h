@@ -24,8 +24,17 @@ struct Tile {
     int index;            // the tile's index in the caller's batch
 };
 
+// What the later kernels need to know of a block, in one 16-byte load.
+struct alignas(16) Block {
+    int tile;             // of the group
+    unsigned local;       // block of the tile
+    int nbx;              // the tile's blocks across
+    unsigned nterm;       // nodes, and which neighbours exist
+};
+constexpr unsigned B_RIGHT = 1u << 8, B_DOWN = 1u << 9, B_UP = 1u << 10;
+
 // Scratch of one launch group, per block: 2 bytes per pixel (value, node), the
-// same for the four boundary lines, the node links, the node count.
+// same for the four boundary lines, the node links, the block's record.
 struct Params {
     const Tile *tiles;            // tiles of the group
     const unsigned *base;         // ntiles + 1 cumulative block counts
@@ -34,7 +43,7 @@ struct Params {
     uint16_t *px;                 // nblocks * BPX
     uint16_t *rim;                // nblocks * 4 * BS: top, bottom, left, right lines
     unsigned long long *link;     // nblocks * MAX_TERM: weight << 32 | parent node
-    unsigned *nterm;              // nblocks
+    Block *block;                 // nblocks
     rk::Ctl *ctl;
     int *tile_err;                // by caller's tile index
     rk::Work *work;               // by caller's tile index
@@ -44,7 +53,7 @@ struct Params {
 
 inline size_t scratch_bytes(size_t nblocks)
 {
-    return nblocks * (sizeof(uint16_t) * (BPX + 4 * BS) + sizeof(unsigned long long) * MAX_TERM + sizeof(unsigned));
+    return nblocks * (sizeof(uint16_t) * (BPX + 4 * BS) + sizeof(unsigned long long) * MAX_TERM + sizeof(Block));
 }
 
 }  // namespace rf
