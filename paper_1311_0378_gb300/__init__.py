@@ -15,6 +15,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from typing import Optional, Sequence, Tuple
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
@@ -341,6 +342,14 @@ def _check_pair(I, J):
                          % (tuple(I.shape), I.device, tuple(J.shape), J.device))
 
 
+def _plain_pair(I, J, T, u8, device: int) -> bool:
+    """Whether _check_pair(I, J) passes for two plain tensors on CUDA device
+    `device`; False leaves the answer to _check_pair. (A large batch of small
+    tiles spends most of its time in these checks: each attribute is read once.)"""
+    return (type(I) is T and type(J) is T and I.dtype is u8 and J.dtype is u8 and I.is_cuda and J.is_cuda
+            and I.get_device() == device and J.get_device() == device and I.is_contiguous() and J.is_contiguous())
+
+
 def context_for(device, stream=None, flags: int = RECON_FLAG_SYNC):
     """A context kept per (device index, stream, flags) for the tensor calls;
     `stream` is a torch.cuda.Stream (None: torch's current stream on that
@@ -367,23 +376,53 @@ def run(I, J, conn: int = 8, op: int = RECON_OP_DILATE, ctx=None):
     return J
 
 
+_TILE = struct.Struct("@QQ5i4x")   # recon_tile: I, J, H, W, pitch, conn, op
+assert _TILE.size == ctypes.sizeof(recon_tile)
+
+
+def _pair_tiles(pairs, conn: int, op: int):
+    """The recon_tile array of a batch of plain tensors on one device, or None
+    when one of them needs the full checks (or does not fit the fields)."""
+    import torch
+    T, u8, pack, rows = torch.Tensor, torch.uint8, _TILE.pack, []
+    conn, op = ctypes.c_int(conn).value, ctypes.c_int(op).value
+    first = pairs[0][1]
+    if type(first) is not T or not first.is_cuda:
+        return None
+    device = first.get_device()
+    try:
+        for I, J in pairs:
+            if not _plain_pair(I, J, T, u8, device):
+                return None
+            shape = I.shape
+            if len(shape) != 2 or J.shape != shape:
+                return None
+            H, W = shape
+            rows.append(pack(I.data_ptr(), J.data_ptr(), H, W, W, conn, op))
+    except struct.error:
+        return None
+    return (recon_tile * len(rows)).from_buffer_copy(b"".join(rows))
+
+
 def batch(pairs, conn: int = 8, op: int = RECON_OP_DILATE, ctx=None):
-    """Reconstructs every (I, J) pair in one persistent launch, each J in place,
+    """Reconstructs every (I, J) pair in one call, each J in place,
     and returns the list of J. Tensors as for run(); tiles may differ in size
     and must not share memory. Raises ReconError (with the failing tile from
     recon_last_error_tile in the message) on failure."""
     pairs = list(pairs)
     if not pairs:
         raise ValueError("batch needs at least one (I, J) pair")
-    for I, J in pairs:
-        _check_pair(I, J)
-    dev = pairs[0][1].device
-    if any(J.device != dev for _, J in pairs):
-        raise ValueError("all tiles of a batch must be on one device")
-    c = ctx if ctx is not None else context_for(dev)
-    tiles = [(I.data_ptr(), J.data_ptr(), int(I.shape[0]), int(I.shape[1]), int(I.shape[1]), conn, op)
-             for I, J in pairs]
-    st = recon_batch(c, tiles)
+    tiles = _pair_tiles(pairs, conn, op)
+    if tiles is None:
+        for I, J in pairs:
+            _check_pair(I, J)
+        dev = pairs[0][1].device
+        if any(J.device != dev for _, J in pairs):
+            raise ValueError("all tiles of a batch must be on one device")
+        tiles = _tiles([(I.data_ptr(), J.data_ptr(), int(I.shape[0]), int(I.shape[1]), int(I.shape[1]), conn, op)
+                        for I, J in pairs])
+    c = ctx if ctx is not None else context_for(pairs[0][1].device)
+    st = lib().recon_batch(c, tiles, len(pairs))
     if st != RECON_OK:
         raise ReconError(st, "batch (first failing tile %d)" % recon_last_error_tile(c))
     return [J for _, J in pairs]
