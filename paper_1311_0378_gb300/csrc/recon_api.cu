@@ -54,6 +54,8 @@ struct recon_ctx {
     // region-merging engine: status + work + tile lists (one upload), block scratch
     unsigned char *d_fmeta = nullptr; size_t cap_fmeta = 0;
     unsigned char *d_forest = nullptr; size_t cap_forest = 0;
+    rf::Status *d_status = nullptr;   // two, for calls on one tile: which one is next; -1: not usable any more
+    int status_turn = 0;
     // status and work counters of the last call (either engine's)
     rk::Ctl *last_ctl = nullptr; rk::Work *last_work = nullptr;
     rk::Ctl *h_ctl = nullptr;   // pinned: the status word as recon_sync reads it
@@ -147,6 +149,13 @@ extern "C" int recon_init(recon_ctx **out, int device, void *cuda_stream, unsign
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev1);
     if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_ctl, sizeof(rk::Ctl));
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_ctl, sizeof(rk::Ctl));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_status, 2 * sizeof(rf::Status));
+    if (e == cudaSuccess) {
+        rf::Status clear[2];
+        memset(clear, 0, sizeof(clear));
+        clear[0].ctl.err_tile = clear[1].ctl.err_tile = INT_MAX;
+        e = cudaMemcpy(c->d_status, clear, sizeof(clear), cudaMemcpyHostToDevice);
+    }
     if (e == cudaSuccess) e = rf_configure();
     if (e == cudaSuccess) {
         int occ = 0;
@@ -194,6 +203,7 @@ extern "C" int recon_free(recon_ctx *c)
     cudaFree(c->d_spill);
     cudaFree(c->d_fmeta);
     cudaFree(c->d_forest);
+    cudaFree(c->d_status);
     cudaFree(c->d_img);
     cudaFree(c->d_dt);
     cudaFree(c->d_train);
@@ -455,20 +465,52 @@ static int stage_meta(recon_ctx *c, const recon_tile *tiles, int n, const int *v
 // engine: when the context's wavefront settings are all at their defaults.
 // Setting any of them (recon_set_param, RECON_*, recon_autotune) or passing
 // variants or an order asks for the wavefront engine. The merging engine was
-// faster at every size, marker, connectivity and operation measured, by 1.5
-// (4096^2, h-dome: 403 -> 272 us) to 18 times (3000^2, border-seeded: 4.26 ->
-// 0.24 ms), so there is no size below or above which the other is chosen.
+// faster at every size, marker, connectivity and operation measured, by 1.8
+// (4096^2, h-dome: 405 -> 229 us) to 24 times (holes filled: 2.66 -> 0.112 ms),
+// so there is no size below or above which the other is chosen.
 static bool use_forest(const recon_ctx *c)
 {
     return c->bh == 128 && c->k == 1 && c->grid == 0 && c->bands == 4 && c->use_tma == 1 && c->revisit_scans == 0 &&
            c->scan_gain == 2048 && !c->phantom && !c->trace_on;
 }
 
-// Runs the batch on the region-merging engine: one upload (status, counters,
-// tile lists), then up to three launches per group of tiles. *done = 0 when the
-// batch does not fit that engine (nothing was launched). Launched directly, not
-// as a graph: a graph would be rebuilt whenever a call brings other buffers.
-static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, int *done)
+static rf::Tile forest_tile(const recon_tile &T, int index)
+{
+    rf::Tile d;
+    memset(&d, 0, sizeof(d));
+    d.I = T.I; d.J = T.J; d.H = T.H; d.W = T.W; d.pitch = T.pitch;
+    d.nbx = (T.W - 1) / rf::BS + 1;
+    d.nby = (T.H - 1) / rf::BS + 1;
+    d.dual = T.op != RECON_OP_DILATE ? 1 : 0;
+    d.fill = T.op == RECON_OP_FILL_HOLES ? 1 : 0;
+    d.index = index;
+    return d;
+}
+
+static rf::Params forest_params(const recon_ctx *c, unsigned nblocks, int ntiles, int flat)
+{
+    rf::Params P;
+    memset(&P, 0, sizeof(P));
+    const size_t nb = nblocks;
+    P.ntiles = ntiles;
+    P.nblocks = nblocks;
+    P.flat = flat;
+    P.px = (uint16_t *)c->d_forest;
+    P.link = (unsigned long long *)(P.px + nb * rf::BPX);
+    P.rim = (uint16_t *)(P.link + nb * rf::MAX_TERM);
+    P.block = (rf::Block *)(P.rim + nb * 4 * rf::BS);
+    P.ctl = c->last_ctl;
+    P.work = c->last_work;
+    P.check = (c->flags & RECON_FLAG_NO_CHECK) ? 0 : 1;
+    return P;
+}
+
+// Runs the batch on the region-merging engine. One tile: up to three launches
+// that carry it. More: one upload (status, counters, tile lists), then up to
+// three launches per group of tiles. *done = 0 when the batch does not fit that
+// engine (nothing was launched). Launched directly, not as a graph: a graph
+// would be rebuilt whenever a call brings other buffers.
+static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, bool capturing, int *done)
 {
     *done = 0;
     struct Group { int conn, first, count; unsigned nblocks; int flat; size_t off_base; };
@@ -505,15 +547,39 @@ static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, int *done)
         g.off_base = total;
         total += align_up(sizeof(unsigned) * ((size_t)g.count + 1), 16);
     }
+    // One tile travels with its launches. (A captured call runs again and again, and so clears its own status.)
+    const bool one = n == 1 && c->status_turn >= 0 && !capturing;
     const size_t need = rf::scratch_bytes(most);
     int rc;
-    if (c->cap_fmeta < total || c->cap_forest < need) {
+    if ((!one && c->cap_fmeta < total) || c->cap_forest < need) {
         CK(cudaStreamSynchronize(c->stream));
-        if (c->last_ctl == (rk::Ctl *)c->d_fmeta) c->launched = 0;   // that call's status goes with the buffer
-        if ((rc = grow(&c->d_fmeta, &c->cap_fmeta, total))) return rc;
+        if (!one && c->last_ctl == (rk::Ctl *)c->d_fmeta) c->launched = 0;   // that call's status goes with the buffer
+        if (!one && (rc = grow(&c->d_fmeta, &c->cap_fmeta, total))) return rc;
         rc = grow(&c->d_forest, &c->cap_forest, need);
         if (rc == RECON_ENOMEM) return RECON_OK;   // the wavefront engine needs far less scratch
         if (rc) return rc;
+    }
+    if (one) {
+        rf::Status *const st = c->d_status + c->status_turn;
+        *done = 1;
+        c->last_n = 1;
+        c->last_err_tile = -1;
+        c->host_status = 0;
+        c->last_ctl = &st->ctl;
+        c->last_work = &st->work;
+        rf::Params P = forest_params(c, most, 1, groups[0].flat);
+        P.one = forest_tile(tiles[0], 0);
+        P.tile_err = &st->tile_err;
+        P.next = c->d_status + (1 - c->status_turn);
+        const int turn = 1 - c->status_turn;
+        c->status_turn = -1;   // until all launches went through
+        CK(cudaEventRecord(c->ev0, c->stream));
+        CK(rf_launch(tiles[0].conn, &P, c->stream));
+        CK(cudaEventRecord(c->ev1, c->stream));
+        c->status_turn = turn;
+        c->launched = 1;
+        if (c->flags & RECON_FLAG_SYNC) return recon_sync(c);
+        return RECON_OK;
     }
     if ((rc = ensure_stage(c, total))) return rc;
     unsigned char *h = c->h_meta;
@@ -523,16 +589,7 @@ static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, int *done)
     for (const Group &g : groups) {
         unsigned *base = (unsigned *)(h + g.off_base), acc = 0;
         for (int i = 0; i < g.count; ++i) {
-            const int t = seq[g.first + i];
-            const recon_tile &T = tiles[t];
-            rf::Tile d;
-            memset(&d, 0, sizeof(d));
-            d.I = T.I; d.J = T.J; d.H = T.H; d.W = T.W; d.pitch = T.pitch;
-            d.nbx = (T.W - 1) / rf::BS + 1;
-            d.nby = (T.H - 1) / rf::BS + 1;
-            d.dual = T.op != RECON_OP_DILATE ? 1 : 0;
-            d.fill = T.op == RECON_OP_FILL_HOLES ? 1 : 0;
-            d.index = t;
+            const rf::Tile d = forest_tile(tiles[seq[g.first + i]], seq[g.first + i]);
             ft[g.first + i] = d;
             base[i] = acc;
             acc += (unsigned)(d.nbx * d.nby);
@@ -549,22 +606,10 @@ static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, int *done)
     CK(cudaEventRecord(c->meta_free, c->stream));
     CK(cudaEventRecord(c->ev0, c->stream));
     for (const Group &g : groups) {
-        rf::Params P;
-        memset(&P, 0, sizeof(P));
+        rf::Params P = forest_params(c, g.nblocks, g.count, g.flat);
         P.tiles = (const rf::Tile *)(c->d_fmeta + off_tiles) + g.first;
         P.base = (const unsigned *)(c->d_fmeta + g.off_base);
-        P.ntiles = g.count;
-        P.nblocks = g.nblocks;
-        const size_t nb = g.nblocks;
-        P.px = (uint16_t *)c->d_forest;
-        P.link = (unsigned long long *)(P.px + nb * rf::BPX);
-        P.rim = (uint16_t *)(P.link + nb * rf::MAX_TERM);
-        P.block = (rf::Block *)(P.rim + nb * 4 * rf::BS);
-        P.ctl = c->last_ctl;
         P.tile_err = (int *)(c->d_fmeta + off_err);
-        P.work = c->last_work;
-        P.check = (c->flags & RECON_FLAG_NO_CHECK) ? 0 : 1;
-        P.flat = g.flat;
         CK(rf_launch(g.conn, &P, c->stream));
     }
     CK(cudaEventRecord(c->ev1, c->stream));
@@ -585,14 +630,13 @@ static int batch_impl(recon_ctx *c, const recon_tile *tiles, int n, const int *v
     CK(cudaSetDevice(c->device));
 
     if (!variant && !order && use_forest(c)) {
-        if (!(c->flags & RECON_FLAG_NO_GRAPH)) {
-            // a stream the caller is capturing is refused, as the graph path below refuses it
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-            CK(cudaStreamIsCapturing(c->stream, &cap));
-            if (cap != cudaStreamCaptureStatusNone) return RECON_ECUDA;
-        }
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(c->stream, &cap));
+        const bool capturing = cap != cudaStreamCaptureStatusNone;
+        // a stream the caller is capturing is refused, as the graph path below refuses it
+        if (capturing && !(c->flags & RECON_FLAG_NO_GRAPH)) return RECON_ECUDA;
         int done = 0;
-        const int frc = forest_batch(c, tiles, n, &done);
+        const int frc = forest_batch(c, tiles, n, capturing, &done);
         if (done || frc != RECON_OK) return frc;
     }
 

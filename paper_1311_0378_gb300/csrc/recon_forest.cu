@@ -25,20 +25,22 @@
 // Nodes are kept in a forest of weighted links: the region of a at weight w is
 // what hangs together by links of weight >= w, and its root is found by walking
 // them up from a. An edge (a, b, w) is added by linking the two regions' roots
-// at w; the lighter link that this displaces is added again further up. Links are single 64-bit words changed by compare-and-swap, and
-// every link goes to a node of higher (hashed) priority: no cycles in any
-// interleaving, and walks of logarithmic expected length.
+// at w; the lighter link that this displaces is added again further up. Links
+// are single 64-bit words changed by compare-and-swap, and every link goes to a
+// node of higher (hashed) priority: no cycles in any interleaving, and walks of
+// logarithmic expected length.
 //
 // Measured on GB300 (whole call, the wavefront engine -> this one): a 4096^2
-// tile seeded from its border, 4-connected, 6.04 -> 0.346 ms; with an h-dome
-// marker, 8-connected, 0.403 -> 0.272 ms; 200 tiles of 256 .. 4096 pixels a
-// side (910 Mpx, both markers) 54.2 -> 12.3 ms; 512^2 0.231 -> 0.093 ms.
-// block_kernel takes most of it (0.22 of 0.29 ms of kernel time on the
+// tile seeded from its border, 4-connected, 6.04 -> 0.312 ms; with an h-dome
+// marker, 8-connected, 0.405 -> 0.229 ms; 200 tiles of 256 .. 4096 pixels a
+// side (910 Mpx, both markers) 57.0 -> 10.9 ms; 512^2 0.233 -> 0.072 ms.
+// block_kernel takes most of it (0.22 of 0.27 ms of kernel time on the
 // border-seeded tile) and is bound by instruction issue and the shared-memory
 // pipe (about 65% and 50%; DRAM below 10%), so what counts is warp instructions
-// a block: 30 600 (h-dome) to 40 900 (border), 76 500 and 94 900 at first. Saddles instead of
-// all pixel pairs, arcs of four pixels at once in byte lanes, loops rolled to fit
-// the instruction cache, and lists that stay dense made the difference.
+// a block: 30 600 (h-dome) to 40 900 (border), 76 500 and 94 900 at first.
+// Saddles instead of all pixel pairs, arcs of four pixels at once in byte
+// lanes, loops rolled to fit the instruction cache, and lists that stay dense
+// made the difference.
 #include <climits>
 #include <cstddef>
 #include "recon_forest.h"
@@ -80,6 +82,8 @@ struct Smem {
     unsigned nlive[2];                // live roots, by round parity
     int tile;
     unsigned local;
+    Block rec;                        // what is left for the other kernels
+    unsigned long long tick[6];
 };
 
 __device__ __forceinline__ unsigned long long now_ns()
@@ -88,6 +92,15 @@ __device__ __forceinline__ unsigned long long now_ns()
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
+
+// The next kernel of a group may be launched while this one still runs (its
+// CTAs fill the places that the last CTAs leave free); it waits for all of this
+// one's results before it reads any. 512^2: 78 -> 74 us a call; the 910 Mpx batch
+// 10.95 -> 10.83 ms of kernel time.
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ const Tile &tile_of(const Params &P, int t) { return P.tiles ? P.tiles[t] : P.one; }
 
 // The tile of block b of the group (warp-wide 32-ary search).
 __device__ __forceinline__ int find_tile(const Params &P, unsigned b)
@@ -318,21 +331,24 @@ __device__ __noinline__ void each_pair(Smem<CONN> &S, F f)
 }
 
 // Five CTAs an SM where shared memory allows it (8-connectivity: 43 KB; 4: 56 KB
-// for twice the basins): 10.95 ms on the 910 Mpx batch, 11.13 with four.
+// for twice the basins), in 48 registers without spills: 10.40 ms on the 910 Mpx
+// batch. With the timers and the tile's record in registers instead of shared
+// memory there were spills and it took 10.95 ms, with four CTAs 11.13.
 template <int CONN>
-__global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(Params P)
+__global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __grid_constant__ Params P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Smem<CONN> &S = *reinterpret_cast<Smem<CONN> *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned blk = blockIdx.x;
-    unsigned long long tick[6];   // thread 0: start and end of the phases (recon_work.phase_ns)
-    if (tid == 0) tick[0] = now_ns();
+    if (tid == 0) S.tick[0] = now_ns();   // start and end of the phases (recon_work.phase_ns)
+    if (P.next && blk == 0 && tid < (int)(sizeof(Status) / 4))
+        ((unsigned *)P.next)[tid] = tid == (int)(offsetof(rk::Ctl, err_tile) / 4) ? (unsigned)INT_MAX : 0u;
     if (warp == 0) {
         const int t = find_tile(P, blk);
         if (lane == 0) {
             S.tile = t;
-            S.local = blk - P.base[t];
+            S.local = blk - (P.tiles ? P.base[t] : 0u);
             S.nb = 1;
             S.nt = 0;
             S.ne = 0;
@@ -341,9 +357,12 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(Params P)
         }
     }
     __syncthreads();
-    const Tile D = P.tiles[S.tile];
+    const Tile D = tile_of(P, S.tile);
     const int by = (int)(S.local / (unsigned)D.nbx), bx = (int)(S.local - (unsigned)by * D.nbx);
     const int y0 = by * BS, x0 = bx * BS;
+    if (tid == 0)
+        S.rec = Block{S.tile, S.local, D.nbx,
+                      (bx + 1 < D.nbx ? B_RIGHT : 0u) | (by + 1 < D.nby ? B_DOWN : 0u) | (by > 0 ? B_UP : 0u)};
     const bool vec = (D.pitch % 16) == 0 && ((uintptr_t)D.I % 16) == 0 && ((uintptr_t)D.J % 16) == 0;
     const int r = tid >> 2, c = tid & 3;         // this thread's run: row r, columns 16c .. 16c + 15
     const int y = y0 + r, x = x0 + 16 * c;
@@ -422,7 +441,8 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(Params P)
         }
     }
 
-    if (tid == 0) tick[1] = now_ns();
+    allow_next();
+    if (tid == 0) S.tick[1] = now_ns();
     // Basins: every pixel points to the first upper neighbour of its first arc
     // (its heaviest edges all weigh its own height); pixels without one are tops.
     // A warp takes two rows at a time, a lane one word of four pixels (a loop,
@@ -534,7 +554,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(Params P)
         }
     }
     __syncthreads();
-    if (tid == 0) tick[2] = now_ns();
+    if (tid == 0) S.tick[2] = now_ns();
     // (a predicated reduction: no branch, and no atomic when the key does not raise the maximum)
     const unsigned best0 = (unsigned)__cvta_generic_to_shared(S.best);
     auto offer = [&](unsigned a, uint32_t key) {
@@ -596,7 +616,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(Params P)
         __syncthreads();
     }
 
-    if (tid == 0) tick[3] = now_ns();
+    if (tid == 0) S.tick[3] = now_ns();
     // Boruvka's rounds. A live region takes the heaviest of its edges: to the
     // source, to another region (numbers break ties, the same for both ends,
     // so only the two ends of one edge can choose each other) or out of the
@@ -770,12 +790,11 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(Params P)
                 (unsigned long long)(l >> 8) << 32 | (par == RES ? SRC : blk * MAX_TERM + par);
         }
     }
-    if (tid == 0)
-        P.block[blk] = Block{S.tile, S.local, D.nbx,
-                             nt | (bx + 1 < D.nbx ? B_RIGHT : 0u) | (by + 1 < D.nby ? B_DOWN : 0u) | (by > 0 ? B_UP : 0u)};
+    if (tid == 0) P.block[blk] = Block{S.rec.tile, S.rec.local, S.rec.nbx, S.rec.nterm | nt};
 
-    if (tid == 0) tick[4] = now_ns();
+    if (tid == 0) S.tick[4] = now_ns();
     // Results: the pixels themselves when everything is final, else (cap, node)
+    const Tile &E = tile_of(P, S.tile);   // (read again: not kept in registers through the rounds)
     {
         const int cell = (r + 1) * ST + X0 + 16 * c;
         const uint4 iv = *(const uint4 *)&bi[(r + 1) * IST + 4 + 4 * c];
@@ -796,8 +815,9 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(Params P)
         if (nt == 0) {
             uint32_t w[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) w[j] = __byte_perm(o[2 * j], o[2 * j + 1], 0x7531) ^ (D.dual ? FULL : 0u);
-            if (y < D.H) store16(D.J + (size_t)y * D.pitch + x, D.W - x, make_uint4(w[0], w[1], w[2], w[3]), vec);
+            for (int j = 0; j < 4; ++j) w[j] = __byte_perm(o[2 * j], o[2 * j + 1], 0x7531) ^ (E.dual ? FULL : 0u);
+            if (y < E.H) store16(E.J + (size_t)y * E.pitch + x, E.W - x, make_uint4(w[0], w[1], w[2], w[3]),
+                                 (E.pitch % 16) == 0 && ((uintptr_t)E.J % 16) == 0);
         } else {
             uint4 *dst = (uint4 *)(P.px + (size_t)blk * BPX + r * BS + 16 * c);
             dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
@@ -815,15 +835,15 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(Params P)
         }
     }
     if (tid == 0) {
-        tick[5] = now_ns();
-        rk::Work &wk = P.work[D.index];
+        S.tick[5] = now_ns();
+        rk::Work &wk = P.work[E.index];
         atomicAdd(&wk.visits, 1ull);
         atomicAdd(&wk.seeds, (unsigned long long)(nb - 1));
         atomicAdd(&wk.pops, (unsigned long long)ne);
         atomicAdd(&wk.levels, (unsigned long long)rounds + 1);
-        atomicAdd(&wk.busy_ns, tick[5] - tick[0]);
+        atomicAdd(&wk.busy_ns, S.tick[5] - S.tick[0]);
 #pragma unroll
-        for (int k = 0; k < 5; ++k) atomicAdd(&wk.phase_ns[k], tick[k + 1] - tick[k]);
+        for (int k = 0; k < 5; ++k) atomicAdd(&wk.phase_ns[k], S.tick[k + 1] - S.tick[k]);
     }
 }
 
@@ -836,15 +856,17 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(Params P)
 // 20 us on a 4096^2 h-dome tile, 27 us seeded from the border (34 and 40 us with a
 // search for the tile first and a warp-wide match and maximum before each join).
 template <int CONN>
-__global__ void __launch_bounds__(128) rim_kernel(Params P)
+__global__ void __launch_bounds__(128) rim_kernel(const __grid_constant__ Params P)
 {
     const unsigned blk = blockIdx.x;
     const bool right = threadIdx.x < 64;
     const int k = threadIdx.x & 63, lane = threadIdx.x & 31;
+    allow_next();
+    wait_previous();
     const Block B = P.block[blk];
     const unsigned pv = P.rim[(size_t)blk * 4 * BS + (right ? 3 * BS : BS) + k];
     if (!(B.nterm & (right ? B_RIGHT : B_DOWN))) return;   // warp-uniform
-    const bool failed = P.tile_err[P.tiles[B.tile].index] != 0;
+    const bool failed = P.tile_err[tile_of(P, B.tile).index] != 0;
     // opposite pixels k, k - 1, k + 1: their line in the block across, or a corner of the next one
     constexpr int ND = CONN == 8 ? 3 : 1;
     unsigned qn[ND], w[ND];
@@ -900,17 +922,18 @@ __global__ void __launch_bounds__(128) rim_kernel(Params P)
 
 // R of the block's nodes (the lightest link of their path to the source), then
 // of its pixels.
-__global__ void __launch_bounds__(NT) value_kernel(Params P)
+__global__ void __launch_bounds__(NT) value_kernel(const __grid_constant__ Params P)
 {
     __shared__ uint8_t R[256];
     const unsigned blk = blockIdx.x;
     const int r = threadIdx.x >> 2, c = threadIdx.x & 3;
+    wait_previous();
     const Block B = P.block[blk];
     const unsigned nt = B.nterm & 255u;
     if (nt == 0) return;
     const uint4 *src = (const uint4 *)(P.px + (size_t)blk * BPX + r * BS + 16 * c);
     const uint4 q0 = src[0], q1 = src[1];
-    const Tile D = P.tiles[B.tile];
+    const Tile D = tile_of(P, B.tile);
     R[threadIdx.x] = 255;
     if (threadIdx.x < nt) {
         unsigned n = blk * MAX_TERM + threadIdx.x, v = 255;
@@ -957,14 +980,29 @@ extern "C" cudaError_t rf_configure()
     return e;
 }
 
+// Launches kernel f behind the one before it on the stream, as its dependent.
+template <class F>
+static cudaError_t launch_after(F f, unsigned grid, int threads, const rf::Params *P, cudaStream_t st)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f, *P);
+}
+
 extern "C" cudaError_t rf_launch(int conn, const rf::Params *P, cudaStream_t st)
 {
     if (conn == 8) rf::block_kernel<8><<<P->nblocks, rf::NT, sizeof(rf::Smem<8>), st>>>(*P);
     else rf::block_kernel<4><<<P->nblocks, rf::NT, sizeof(rf::Smem<4>), st>>>(*P);
-    if (!P->flat) {
-        if (conn == 8) rf::rim_kernel<8><<<P->nblocks, 128, 0, st>>>(*P);
-        else rf::rim_kernel<4><<<P->nblocks, 128, 0, st>>>(*P);
-        rf::value_kernel<<<P->nblocks, rf::NT, 0, st>>>(*P);
-    }
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    if (P->flat || e != cudaSuccess) return e;
+    e = conn == 8 ? launch_after(rf::rim_kernel<8>, P->nblocks, 128, P, st) : launch_after(rf::rim_kernel<4>, P->nblocks, 128, P, st);
+    if (e == cudaSuccess) e = launch_after(rf::value_kernel, P->nblocks, rf::NT, P, st);
+    return e;
 }
