@@ -279,27 +279,27 @@ __global__ void adam_kernel(float *theta, float *grad, float *m, float *v, int t
 // shared memory, each CTA updates its CL-th of the parameters (Adam's moments
 // stay with it for the whole epoch) and writes them into every CTA's copy. Two
 // cluster barriers a step replace two launches and the global atomics.
-// A step is bound by latency, not arithmetic (6 x 5504 weights x 256 samples =
-// 8.5 MFLOP): mlp_grad's 16 CTAs of 64 threads took one sample at a time, with
-// 32-way bank conflicts in the 64 x 64 layer (a thread per row of stride 64);
-// here the rows are 65 apart and a warp works on 32 units x 4 samples.
-// Measured on an epoch of 4096 samples in 16 batches of 256 (whole call): 2483 us
-// with two launches a step and allocations per call, 271 us now; the error of the
-// weights against 64 bits is 2e-7 (5e-7 before). Larger batches only take more
-// chunks per CTA (about 3 us per 256 samples); mlp_grad needs about twice that.
+// A step is bound by latency and shared-memory loads, not arithmetic (6 x 5504
+// weights x 256 samples = 8.5 MFLOP): mlp_grad's 16 CTAs of 64 threads took one
+// sample at a time, with 32-way bank conflicts in the 64 x 64 layer (a thread per
+// row of stride 64); here the rows are 65 apart, a thread works on one unit of
+// four samples, and the next samples are on their way while these are worked on.
+// An epoch of 16 steps takes 216 us a call, 2473 with those launches.
+// Sixteen CTAs of 256 threads where the device can place them (a cluster that
+// large is not portable), otherwise eight of 512 (262 us; 32 samples a chunk).
 namespace cg = cooperative_groups;
-constexpr int CL = 8, TT = 512, TS = 32;          // CTAs, threads, samples at a time
 constexpr int S1 = D0 + 1, S2 = D1 + 1;           // weight row strides: odd, so that a column has no bank conflicts
 constexpr int PW1 = 0, PB1 = PW1 + D1 * S1, PW2 = PB1 + D1, PB2 = PW2 + D2 * S2, PW3 = PB2 + D2,
               PB3 = PW3 + D3 * D2, PPAD = (PB3 + D3 + 3) / 4 * 4;
-constexpr int OWN = (NP + CL - 1) / CL;           // parameters a CTA updates
-constexpr int OPT = (OWN + TT - 1) / TT;          // per thread
 
+template <int CL>
 struct TrainSmem {
+    static constexpr int TT = 4096 / CL, TS = 256 / CL;   // threads; samples at a time: four a unit and thread group
     float P[PPAD];                                 // weights, padded rows
     float G[(NP + 3) / 4 * 4];                     // this CTA's gradient, flat layout
     alignas(16) float a1[TS][D1], a2[TS][D2], dz1[TS][D1], dz2[TS][D2];
-    float x[TS][D0], t[TS][D3], dy[TS][D3];
+    alignas(16) float x[TS][D0];
+    float t[TS][D3], dy[TS][D3];
     float loss;
 };
 
@@ -312,15 +312,23 @@ __device__ __forceinline__ int padded(int i)       // flat parameter index -> pl
 }
 static_assert(PW3 - PB2 == OW3 - OB2 && PB3 - PB2 == OB3 - OB2, "layout");
 
-__global__ void __launch_bounds__(TT) train_kernel(float *theta, float *m, float *v, const float *X, const float *T,
-                                                   const int *idx, int n, int batch, int step0, float lr, float b1,
-                                                   float b2, float eps, float *loss)
+template <int CL>
+__global__ void __launch_bounds__(TrainSmem<CL>::TT) train_kernel(float *theta, float *m, float *v, const float *X,
+                                                                  const float *T, const int *idx, int n, int batch,
+                                                                  int step0, float lr, float b1, float b2, float eps,
+                                                                  float *loss)
 {
+    typedef TrainSmem<CL> Sm;
+    constexpr int TT = Sm::TT, TS = Sm::TS, NG = TT / 64;   // NG thread groups, 4 samples each
+    constexpr int OWN = (NP + CL - 1) / CL, OPT = (OWN + TT - 1) / TT;   // parameters a CTA (a thread) updates
+    constexpr int RW = D2 / NG, IW = (D0 + NG - 1) / NG;    // W2 rows, inputs of W1 whose gradients a thread adds up
+    constexpr int NF = (TS * (D0 + D3) + TT - 1) / TT;      // inputs and targets a thread fetches
+    static_assert(TS == 4 * NG, "four samples a group");
     extern __shared__ __align__(16) unsigned char train_smem[];
-    TrainSmem &S = *reinterpret_cast<TrainSmem *>(train_smem);
+    Sm &S = *reinterpret_cast<Sm *>(train_smem);
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank(), tid = threadIdx.x;
-    const int j = tid & 63, g = tid >> 6;          // unit and group of four samples (or eight rows)
+    const int j = tid & 63, g = tid >> 6;
     for (int i = tid; i < NP; i += TT) S.P[padded(i)] = theta[i];
     float mo[OPT], vo[OPT];                        // Adam's moments of this thread's parameters
 #pragma unroll
@@ -330,31 +338,64 @@ __global__ void __launch_bounds__(TT) train_kernel(float *theta, float *m, float
         mo[q] = mine ? m[i] : 0.0f;
         vo[q] = mine ? v[i] : 0.0f;
     }
+    // this CTA's samples of the batch at s0: [lo, hi) of it, in chunks of TS (at least one, maybe empty)
+    auto share = [&](int s0, int &lo, int &hi) {
+        const int nb = min(batch, n - s0), per = (nb + CL - 1) / CL;
+        lo = min(nb, rank * per);
+        hi = min(nb, lo + per);
+    };
+    float next[NF];                                // the next chunk's inputs and targets
+    auto fetch = [&](int s0, int c0, int hi) {
+#pragma unroll
+        for (int q = 0; q < NF; ++q) {
+            const int e = tid + q * TT, s = e / (D0 + D3), f = e - s * (D0 + D3);
+            next[q] = 0.0f;
+            if (s < TS && c0 + s < hi) {
+                const size_t row = (size_t)idx[s0 + c0 + s];
+                next[q] = f < D0 ? X[row * D0 + f] : T[row * D3 + f - D0];
+            }
+        }
+    };
     float lsum = 0.0f;
-    int step = step0;
+    int step = step0, lo, hi;
+    share(0, lo, hi);
+    fetch(0, lo, hi);
     for (int s0 = 0; s0 < n; s0 += batch) {
-        const int nb = min(batch, n - s0);
-        const float invN = 1.0f / (float)nb;
-        const int per = (nb + CL - 1) / CL, lo = min(nb, rank * per), hi = min(nb, lo + per);
-        float gw2[8] = {0, 0, 0, 0, 0, 0, 0, 0}, gw1[3] = {0, 0, 0}, gb = 0.0f;
-        for (int c0 = lo; c0 < hi; c0 += TS) {
-            const int nc = min(TS, hi - c0);
+        const float invN = 1.0f / (float)min(batch, n - s0);
+        const bool last = n - s0 <= batch;
+        float gw2[RW], gw1[IW], gb2 = 0.0f, gb1 = 0.0f, gw3 = 0.0f, gb3 = 0.0f;
+#pragma unroll
+        for (int q = 0; q < RW; ++q) gw2[q] = 0.0f;
+#pragma unroll
+        for (int q = 0; q < IW; ++q) gw1[q] = 0.0f;
+        int c0 = lo;
+        do {
+            const int nc = min(TS, hi - c0);       // (negative or 0 when there is nothing to do)
             __syncthreads();                       // the chunk before (or the weights' update) is done with S
-            for (int e = tid; e < TS * (D0 + D3); e += TT) {
-                const int s = e / (D0 + D3), f = e - s * (D0 + D3);
-                const size_t row = s < nc ? (size_t)idx[s0 + c0 + s] : 0;
-                if (f < D0) S.x[s][f] = s < nc ? X[row * D0 + f] : 0.0f;
-                else S.t[s][f - D0] = s < nc ? T[row * D3 + f - D0] : 0.0f;
+#pragma unroll
+            for (int q = 0; q < NF; ++q) {
+                const int e = tid + q * TT, s = e / (D0 + D3), f = e - s * (D0 + D3);
+                if (s < TS) (f < D0 ? S.x[s][f] : S.t[s][f - D0]) = next[q];
             }
             __syncthreads();
+            if (c0 + TS < hi) {
+                fetch(s0, c0 + TS, hi);
+            } else if (!last) {
+                int l2, h2;
+                share(s0 + batch, l2, h2);
+                fetch(s0 + batch, l2, h2);
+            }
             float z[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) z[q] = S.P[PB1 + j];
-#pragma unroll 4
-            for (int i = 0; i < D0; ++i) {
-                const float w = S.P[PW1 + j * S1 + i];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) z[q] = fmaf(w, S.x[4 * g + q][i], z[q]);
+            for (int i = 0; i < D0; i += 4) {
+                const float *w = &S.P[PW1 + j * S1 + i];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 a = *(const float4 *)&S.x[4 * g + q][i];
+                    z[q] = fmaf(w[3], a.w, fmaf(w[2], a.z, fmaf(w[1], a.y, fmaf(w[0], a.x, z[q]))));
+                }
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) S.a1[4 * g + q][j] = 4 * g + q < nc ? fmaxf(z[q], 0.0f) : 0.0f;
@@ -374,13 +415,18 @@ __global__ void __launch_bounds__(TT) train_kernel(float *theta, float *m, float
 #pragma unroll
             for (int q = 0; q < 4; ++q) S.a2[4 * g + q][j] = 4 * g + q < nc ? fmaxf(z[q], 0.0f) : 0.0f;
             __syncthreads();
-            if (tid < TS * D3) {                   // output layer: a thread per sample and output
-                const int s = tid >> 1, o = tid & 1;
-                float y = S.P[PB3 + o];
-                for (int k = 0; k < D2; ++k) y = fmaf(S.P[PW3 + o * D2 + k], S.a2[s][k], y);
-                const float e = s < nc ? y - S.t[s][o] : 0.0f;
-                S.dy[s][o] = e * invN;
-                lsum += 0.5f * e * e * invN;
+            {   // output layer: eight threads per sample and output, eight products each
+                const int s = tid >> 4, o = (tid >> 3) & 1, p = tid & 7;
+                float y = 0.0f;
+#pragma unroll
+                for (int k = 0; k < D2 / 8; ++k) y = fmaf(S.P[PW3 + o * D2 + 8 * k + p], S.a2[s][8 * k + p], y);
+#pragma unroll
+                for (int d = 4; d; d >>= 1) y += __shfl_xor_sync(0xFFFFFFFFu, y, d);
+                if (p == 0) {
+                    const float e = s < nc ? y + S.P[PB3 + o] - S.t[s][o] : 0.0f;
+                    S.dy[s][o] = e * invN;
+                    lsum += 0.5f * e * e * invN;
+                }
             }
             __syncthreads();
 #pragma unroll
@@ -405,46 +451,41 @@ __global__ void __launch_bounds__(TT) train_kernel(float *theta, float *m, float
 #pragma unroll
             for (int q = 0; q < 4; ++q) S.dz1[4 * g + q][j] = S.a1[4 * g + q][j] > 0.0f ? z[q] : 0.0f;
             __syncthreads();
-            // gradients of the chunk: W2 rows 8g .. 8g + 7, column j; W1 elements tid + q TT; biases and W3
+            // gradients of the chunk, all in one pass over its samples: W2 rows RW g ..., column j; W1 row j,
+            // columns g, g + NG, ...; the biases and W3 where a thread has their terms at hand
 #pragma unroll 4
             for (int s = 0; s < TS; ++s) {
-                const float a = S.a1[s][j];
-                const float4 d0 = *(const float4 *)&S.dz2[s][8 * g], d1 = *(const float4 *)&S.dz2[s][8 * g + 4];
-                gw2[0] = fmaf(d0.x, a, gw2[0]); gw2[1] = fmaf(d0.y, a, gw2[1]);
-                gw2[2] = fmaf(d0.z, a, gw2[2]); gw2[3] = fmaf(d0.w, a, gw2[3]);
-                gw2[4] = fmaf(d1.x, a, gw2[4]); gw2[5] = fmaf(d1.y, a, gw2[5]);
-                gw2[6] = fmaf(d1.z, a, gw2[6]); gw2[7] = fmaf(d1.w, a, gw2[7]);
-            }
+                const float a = S.a1[s][j], d1 = S.dz1[s][j];
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const int o = tid + q * TT;
-                if (o < D1 * D0) {
-                    const int r = o / D0, i = o - r * D0;
-#pragma unroll 4
-                    for (int s = 0; s < TS; ++s) gw1[q] = fmaf(S.dz1[s][r], S.x[s][i], gw1[q]);
+                for (int q = 0; q < RW; q += 4) {
+                    const float4 d = *(const float4 *)&S.dz2[s][RW * g + q];
+                    gw2[q] = fmaf(d.x, a, gw2[q]);
+                    gw2[q + 1] = fmaf(d.y, a, gw2[q + 1]);
+                    gw2[q + 2] = fmaf(d.z, a, gw2[q + 2]);
+                    gw2[q + 3] = fmaf(d.w, a, gw2[q + 3]);
                 }
-            }
-            if (tid < D1) {
-                for (int s = 0; s < TS; ++s) gb += S.dz1[s][tid];
-            } else if (tid < 2 * D1) {
-                for (int s = 0; s < TS; ++s) gb += S.dz2[s][tid - D1];
-            } else if (tid < 2 * D1 + D3 * D2) {
-                const int o = (tid - 2 * D1) >> 6;
-                for (int s = 0; s < TS; ++s) gb = fmaf(S.dy[s][o], S.a2[s][j], gb);
-            } else if (tid < 2 * D1 + D3 * D2 + D3) {
-                for (int s = 0; s < TS; ++s) gb += S.dy[s][tid - 2 * D1 - D3 * D2];
-            }
-        }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) S.G[OW2 + (8 * g + q) * D1 + j] = gw2[q];
+                for (int q = 0; q < IW; ++q)
+                    if (g + q * NG < D0) gw1[q] = fmaf(d1, S.x[s][g + q * NG], gw1[q]);
+                if (g == 0) gb1 += d1;
+                else if (g == 1) gb2 += S.dz2[s][j];
+                if (g >= NG - 2) gw3 = fmaf(S.dy[s][g - (NG - 2)], S.a2[s][j], gw3);
+                if (tid < D3) gb3 += S.dy[s][tid];
+            }
+            c0 += TS;
+        } while (c0 < hi);
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (tid + q * TT < D1 * D0) S.G[OW1 + tid + q * TT] = gw1[q];
-        if (tid < D1) S.G[OB1 + tid] = gb;
-        else if (tid < 2 * D1 + D3 * D2 + D3) S.G[OB2 + tid - D1] = gb;
-        cl.sync();                                 // every CTA's gradient is in place
+        for (int q = 0; q < RW; ++q) S.G[OW2 + (RW * g + q) * D1 + j] = gw2[q];
+#pragma unroll
+        for (int q = 0; q < IW; ++q)
+            if (g + q * NG < D0) S.G[OW1 + j * D0 + g + q * NG] = gw1[q];
+        if (g == 0) S.G[OB1 + j] = gb1;
+        else if (g == 1) S.G[OB2 + j] = gb2;
+        if (g >= NG - 2) S.G[OW3 + (g - (NG - 2)) * D2 + j] = gw3;
+        if (tid < D3) S.G[OB3 + tid] = gb3;
         ++step;
-        const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
+        const float k1 = 1.0f - powf(b1, (float)step), k2 = 1.0f - powf(b2, (float)step);
+        cl.sync();                                 // every CTA's gradient is in place
 #pragma unroll
         for (int q = 0; q < OPT; ++q) {
             const int o = tid + q * TT, i = rank * OWN + o;
@@ -456,7 +497,7 @@ __global__ void __launch_bounds__(TT) train_kernel(float *theta, float *m, float
                 for (int r = 0; r < CL; ++r) grad += gr[r];
                 mo[q] = b1 * mo[q] + (1.0f - b1) * grad;
                 vo[q] = b2 * vo[q] + (1.0f - b2) * grad * grad;
-                const float mh = mo[q] / c1, vh = vo[q] / c2;
+                const float mh = mo[q] / k1, vh = vo[q] / k2;
                 float *p = &S.P[padded(i)];
                 const float w = *p - lr * mh / (sqrtf(vh) + eps);
 #pragma unroll
@@ -464,6 +505,8 @@ __global__ void __launch_bounds__(TT) train_kernel(float *theta, float *m, float
             }
         }
         cl.sync();                                 // every CTA has the new weights; the gradients may be overwritten
+        if (!last) share(s0 + batch, lo, hi);
+        else break;                                // (s0 + batch may not fit an int)
     }
 #pragma unroll
     for (int q = 0; q < OPT; ++q) {
@@ -557,24 +600,41 @@ cudaError_t rl_adam(float *theta, float *grad, float *m, float *v, int t, float 
     return cudaGetLastError();
 }
 
+template <int CL>
+static cudaError_t train_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr, cudaStream_t st)
+{
+    typedef rl::TrainSmem<CL> Sm;
+    cudaError_t e = cudaFuncSetAttribute(rl::train_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sm));
+    if (e == cudaSuccess && CL > 8)
+        e = cudaFuncSetAttribute(rl::train_kernel<CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    *cfg = cudaLaunchConfig_t{};
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = CL;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cfg->gridDim = dim3(CL);
+    cfg->blockDim = dim3(Sm::TT);
+    cfg->dynamicSmemBytes = sizeof(Sm);
+    cfg->stream = st;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+    return e;
+}
+
 cudaError_t rl_train_epoch(float *theta, float *m, float *v, const float *X, const float *T, const int *idx, int n,
                            int batch, int step0, float lr, float *loss, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(rl::train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(rl::TrainSmem));
-    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = rl::CL;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(rl::CL);
-    cfg.blockDim = dim3(rl::TT);
-    cfg.dynamicSmemBytes = sizeof(rl::TrainSmem);
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, rl::train_kernel, theta, m, v, X, T, idx, n, batch, step0, lr, 0.9f, 0.999f, 1e-8f,
+    int clusters = 0;
+    cudaError_t e = train_config<16>(&cfg, &attr, st);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, rl::train_kernel<16>, &cfg);
+    if (e == cudaSuccess && clusters > 0)
+        return cudaLaunchKernelEx(&cfg, rl::train_kernel<16>, theta, m, v, X, T, idx, n, batch, step0, lr, 0.9f, 0.999f,
+                                  1e-8f, loss);
+    cudaGetLastError();   // this device cannot place sixteen CTAs together
+    e = train_config<8>(&cfg, &attr, st);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchKernelEx(&cfg, rl::train_kernel<8>, theta, m, v, X, T, idx, n, batch, step0, lr, 0.9f, 0.999f, 1e-8f,
                               loss);
 }
