@@ -31,16 +31,16 @@
 // logarithmic expected length.
 //
 // Measured on GB300 (whole call, the wavefront engine -> this one): a 4096^2
-// tile seeded from its border, 4-connected, 6.04 -> 0.312 ms; with an h-dome
-// marker, 8-connected, 0.405 -> 0.229 ms; 200 tiles of 256 .. 4096 pixels a
-// side (910 Mpx, both markers) 57.0 -> 10.9 ms; 512^2 0.233 -> 0.072 ms.
-// block_kernel takes most of it (0.22 of 0.27 ms of kernel time on the
+// tile seeded from its border, 4-connected, 6.04 -> 0.295 ms; with an h-dome
+// marker, 8-connected, 0.403 -> 0.208 ms; 200 tiles of 256 .. 4096 pixels a
+// side (910 Mpx, both markers) 57.0 -> 9.85 ms; 512^2 0.231 -> 0.069 ms.
+// block_kernel takes most of it (0.20 of 0.245 ms of kernel time on the
 // border-seeded tile) and is bound by instruction issue and the shared-memory
-// pipe (about 65% and 50%; DRAM below 10%), so what counts is warp instructions
-// a block: 30 600 (h-dome) to 40 900 (border), 76 500 and 94 900 at first.
-// Saddles instead of all pixel pairs, arcs of four pixels at once in byte
-// lanes, loops rolled to fit the instruction cache, and lists that stay dense
-// made the difference.
+// pipe (about 65% and 53%; DRAM below 4%), so what counts is warp instructions
+// a block: 26 700 (h-dome) to 37 500 (border), 76 500 and 94 900 at first.
+// Saddles instead of all pixel pairs, arcs and targets of four pixels at once in
+// byte lanes, loops rolled to fit the instruction cache, and lists that stay
+// dense made the difference.
 #include <climits>
 #include <cstddef>
 #include "recon_forest.h"
@@ -53,10 +53,12 @@ constexpr int NT = 256;            // threads per CTA: one 16-pixel run each
 // The cell right of a row's last pixel is the first cell of the next row.
 constexpr int ST = BS + 8, X0 = 8;
 constexpr int NCELL = (BS + 2) * ST + 8;
-constexpr int IST = 20;            // row stride of the byte image in words (interior at word 4)
+constexpr int IST = ST / 4;        // row stride of the byte image in words, interior at word 2: a pixel's
+                                   // byte has the number of its cell
 constexpr int JOFF = (BS + 2) * IST + 4, IMG = JOFF + BPX / 4;   // where J's bytes start, words in all
+static_assert(X0 == 8 && ST == 72, "layout");
 constexpr int TAB = 2048;          // passes a block can list (noise has about 1150)
-constexpr unsigned ROOT = 0x8000u; // label flag: a basin number, not a pointer to a cell
+constexpr unsigned ROOT = 0x8000u; // label flag: a basin number, not a place of a cell
 constexpr unsigned FINAL = 0xFFFFFFFEu, NODE = 0xFFFFFFFFu;   // best[] of a region that stopped
 // edge kinds of a region's heaviest edge (weight << 24 | kind | number): the larger wins a tie
 constexpr unsigned K_SOURCE = 2u << 22, K_EDGE = 1u << 22, K_OUT = 0u;
@@ -69,7 +71,7 @@ constexpr int MAX_STEPS = 1 << 20;      // bound of every walk
 template <int CONN>
 struct Smem {
     static constexpr int NB = (CONN == 8 ? BPX / 4 : BPX / 2) + 32;
-    alignas(16) uint16_t L[NCELL];    // labels: a cell number, or ROOT | basin
+    alignas(16) uint16_t L[NCELL];    // labels: a cell's place in bytes, or ROOT | basin
     alignas(16) uint32_t img[IMG];    // byte image of I, then the bytes of J
     uint32_t tab[TAB];                // passes: region << 20 | region << 8 | weight, 0 = none
     uint32_t best[NB];                // heaviest edge of a live region to a region or out of the block; FINAL, NODE
@@ -243,6 +245,25 @@ __device__ __forceinline__ int ring_off(unsigned k)
     return (int)r;
 }
 
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return r;
+}
+
+// Cell offsets of four ring positions (bytes), plus RING0.
+constexpr int RING0 = ST + 1;
+__device__ __forceinline__ uint32_t ring_offs(uint32_t k)
+{
+    constexpr uint32_t LO = (uint32_t)(RING0 - ST) | (uint32_t)(RING0 - ST + 1) << 8 | (uint32_t)(RING0 + 1) << 16 |
+                            (uint32_t)(RING0 + ST + 1) << 24;
+    constexpr uint32_t HI = (uint32_t)(RING0 + ST) | (uint32_t)(RING0 + ST - 1) << 8 | (uint32_t)(RING0 - 1) << 16 |
+                            (uint32_t)(RING0 - ST - 1) << 24;
+    const uint32_t n = k | k >> 4;                    // positions 0 and 1 in byte 0, 2 and 3 in byte 2
+    return prmt(LO, HI, prmt(n, 0u, 0x4420u));
+}
+
 // Priority of a node: links go to higher priorities, the source last.
 __device__ __forceinline__ uint32_t priority(uint32_t node)
 {
@@ -325,7 +346,7 @@ __device__ __noinline__ void each_pair(Smem<CONN> &S, F f)
         const int py = (int)(px / BS), qx = (int)(px % BS);
         const int dx = d == 0 ? 1 : (int)d - 2, dy = d != 0;
         const unsigned a = S.L[(py + 1) * ST + X0 + qx], b = S.L[(py + dy + 1) * ST + X0 + qx + dx];
-        const unsigned w = min(img[(py + 1) * IST * 4 + 16 + qx], img[(py + dy + 1) * IST * 4 + 16 + qx + dx]);
+        const unsigned w = min(img[(py + 1) * ST + X0 + qx], img[(py + dy + 1) * ST + X0 + qx + dx]);
         if (w && a != b) f(a & 0x7FFFu, b & 0x7FFFu, w, i);
     }
 }
@@ -412,12 +433,13 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
                 vj = make_uint4(w[0], w[1], w[2], w[3]);
             }
         }
-        *(uint4 *)&bi[(r + 1) * IST + 4 + 4 * c] = vi;
+        *(uint2 *)&bi[(r + 1) * IST + 2 + 4 * c] = make_uint2(vi.x, vi.y);
+        *(uint2 *)&bi[(r + 1) * IST + 4 + 4 * c] = make_uint2(vi.z, vi.w);
         if (tid < IST) bi[tid] = 0u;                                   // row above
         else if (tid < 2 * IST) bi[(BS + 1) * IST + tid - IST] = 0u;   // row below
         else if (tid >= 64 && tid < 64 + BS + 3) {                     // words left of row q and right of row q - 1
             const int q = tid - 64;
-            if (q < BS + 2) bi[q * IST + 3] = 0u;
+            if (q < BS + 2) bi[q * IST + 1] = 0u;
             if (q) bi[q * IST] = 0u;
         }
         *(uint4 *)&bj[r * (BS / 4) + 4 * c] = vj;
@@ -445,22 +467,46 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     if (tid == 0) S.tick[1] = now_ns();
     // Basins: every pixel points to the first upper neighbour of its first arc
     // (its heaviest edges all weigh its own height); pixels without one are tops.
-    // A warp takes two rows at a time, a lane one word of four pixels (a loop,
-    // not unrolled: code that does not fit the instruction cache costs more).
-#pragma unroll 1
-    for (int it = 0; it < BS / 2; it += NT / 32) {
-        const int row = 2 * (it + warp) + (lane >> 4), cw = lane & 15;
-        const uint32_t *at = &bi[(row + 1) * IST + 4 + cw];
-        const uint32_t l[3] = {at[-IST - 1], at[-1], at[IST - 1]};
-        const uint32_t m[3] = {at[-IST], at[0], at[IST]};
-        const uint32_t q[3] = {at[-IST + 1], at[1], at[IST + 1]};
-        const uint32_t high = nonzero_bytes(m[1]);   // pixels of height 0 have value 0, like the outside (basin 0)
-        const uint32_t starts = arc_starts<CONN>(l, m, q) & ((high >> 7) * 255u);
-        const uint32_t rest = starts & ((starts | 0x80808080u) - 0x01010101u);   // without the lowest: further arcs
-        const uint32_t tops = high & ~nonzero_bytes(starts);
+    // A lane takes a word of four pixels in each of four rows: 4.5 loads and a
+    // quarter of a warp's scan a word instead of 9 and one (10 500 instructions
+    // a block with a row each and the labels pixel by pixel; on the 910 Mpx
+    // batch 10.40 ms, 9.54 now).
+    {
+        constexpr int RL = BS / (NT / 16);
+        const int row = RL * (2 * warp + (lane >> 4)), cw = lane & 15;
         const int cell = (row + 1) * ST + X0 + 4 * cw;
+        uint32_t rest[RL], tops = 0u;    // further arcs; pixels without any (bit 8 b + 7 - row)
+        unsigned passes = 0;
+        {
+            const uint32_t *at = &bi[(row + 1) * IST + 2 + cw];
+            uint32_t l[3] = {0u, at[-IST - 1], at[-1]}, m[3] = {0u, at[-IST], at[0]}, q[3] = {0u, at[-IST + 1], at[1]};
+#pragma unroll
+            for (int h = 0; h < RL; ++h) {
+#pragma unroll
+                for (int k = 0; k < 2; ++k) { l[k] = l[k + 1]; m[k] = m[k + 1]; q[k] = q[k + 1]; }
+                l[2] = at[(h + 1) * IST - 1]; m[2] = at[(h + 1) * IST]; q[2] = at[(h + 1) * IST + 1];
+                const uint32_t high = nonzero_bytes(m[1]);   // pixels of height 0 have value 0, like the outside (basin 0)
+                const uint32_t starts = arc_starts<CONN>(l, m, q) & ((high >> 7) * 255u);
+                rest[h] = starts & ((starts | 0x80808080u) - 0x01010101u);   // without the lowest: further arcs
+                const uint32_t some = nonzero_bytes(starts);
+                tops |= (high & ~some) >> h;
+                passes += __popc(rest[h]);
+                // the targets' cells, as 16-bit lanes: ring position of the first arc (ones below its bit, counted
+                // per byte), looked up for all four pixels at once
+                uint32_t t = (starts & ~rest[h]) - (some >> 7);
+                t -= (t >> 1) & 0x55555555u;
+                t = (t & 0x33333333u) + ((t >> 2) & 0x33333333u);
+                t = (t + (t >> 4)) & 0x0F0F0F0Fu;
+                const uint32_t off = ring_offs(t);
+                const uint32_t from = (unsigned)(cell + h * ST - RING0) * 0x10001u + 0x10000u;
+                const uint32_t f0 = from + prmt(off, 0u, 0x4140u), f1 = from + 0x20002u + prmt(off, 0u, 0x4342u);
+                const uint32_t m0 = prmt(some, 0u, 0x9988u), m1 = prmt(some, 0u, 0xBBAAu);
+                *(uint2 *)&S.L[cell + h * ST] = make_uint2((2u * f0 & m0) | (ROOT * 0x10001u & ~m0), (2u * f1 & m1) | (ROOT * 0x10001u & ~m1));
+            }
+        }
+        asm volatile("" ::: "memory");   // the tops' labels, of another type, come after
         // numbers for the tops (low half), places for the passes (high half)
-        const unsigned mine = __popc(tops) | __popc(rest) << 16;
+        const unsigned mine = __popc(tops) | passes << 16;
         unsigned incl = mine;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
@@ -474,26 +520,24 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
         }
         id = __shfl_sync(FULL, id, 31) + ((incl - mine) & 0xFFFFu);
         slot = __shfl_sync(FULL, slot, 31) + ((incl - mine) >> 16);
-        const uint32_t jw = bj[row * (BS / 4) + cw];
-        uint32_t f[4];
+        const uint8_t *const j0 = (const uint8_t *)&bj[row * (BS / 4) + cw];
+#pragma unroll 1
+        for (; tops; ++id) {
+            const unsigned k = 31 - __clz(tops), b = k >> 3, h = ~k & 7u;
+            tops ^= 1u << k;
+            S.L[cell + (int)(h * ST + b)] = (uint16_t)(ROOT | id);
+            S.sv[id] = j0[h * BS + b];                       // the top's own source edge
+        }
+        // a pass lies at a pixel and leads to a further arc of it: cell << 3 | ring position
+        const bool fits = slot + passes <= TAB;
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const uint32_t sb = (starts >> (8 * b)) & 255u;
-            f[b] = sb ? (uint32_t)(cell + b + ring_off(__ffs(sb) - 1)) : ROOT;
-        }
-        *(uint2 *)&S.L[cell] = make_uint2(f[0] | f[1] << 16, f[2] | f[3] << 16);
-        asm volatile("" ::: "memory");   // the tops' labels, of another type, come after
+        for (int h = 0; h < RL; ++h) {
 #pragma unroll 1
-        for (uint32_t bits = tops; bits; bits &= bits - 1, ++id) {
-            const unsigned k = __ffs(bits) >> 3;         // (high bits of the bytes: 8, 16, 24, 32)
-            S.L[cell + (int)k - 1] = (uint16_t)(ROOT | id);
-            S.sv[id] = (jw >> (8 * k - 8)) & 255u;       // the top's own source edge
-        }
-        // a pass lies at a pixel and leads to a further arc of it: weight << 16 | cell << 3 | ring position
-#pragma unroll 1
-        for (uint32_t bits = rest; bits; bits &= bits - 1, ++slot) {
-            const unsigned k = __ffs(bits) - 1;
-            if (slot < TAB) S.tab[slot] = ((m[1] >> (k & 24u)) & 255u) << 16 | (unsigned)(cell + (int)(k >> 3)) << 3 | (k & 7u);
+            for (uint32_t bits = fits ? rest[h] : 0u; bits; ++slot) {
+                const unsigned k = 31 - __clz(bits);
+                bits ^= 1u << k;
+                S.tab[slot] = 8u * (unsigned)(cell + h * ST) + k;
+            }
         }
     }
     __syncthreads();
@@ -508,7 +552,12 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
         S.up[b] = S.comp[b] = (uint16_t)b;
     }
     {
-        volatile uint16_t *L = S.L;
+        const unsigned L = (unsigned)__cvta_generic_to_shared(S.L);
+        auto label = [&](unsigned at) {
+            unsigned short v;
+            asm volatile("ld.volatile.shared.u16 %0, [%1];" : "=h"(v) : "r"(L + at) : "memory");
+            return (unsigned)v;
+        };
         const int row0 = 2 * warp + (lane >> 4), cw = lane & 15;   // words as above: rows row0 + 16 i
         uint2 *const word = (uint2 *)&S.L[(row0 + 1) * ST + X0 + 4 * cw];
         constexpr int STEP = 16 * ST / 4;
@@ -528,11 +577,11 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
             if (all) break;
             unsigned n[16];
 #pragma unroll
-            for (int k = 0; k < 16; ++k) n[k] = (l[k] & ROOT) ? l[k] : L[l[k]];
+            for (int k = 0; k < 16; ++k) n[k] = (l[k] & ROOT) ? l[k] : label(l[k]);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                *(volatile uint32_t *)&word[i * STEP].x = n[4 * i] | n[4 * i + 1] << 16;
-                *(volatile uint32_t *)&word[i * STEP].y = n[4 * i + 2] | n[4 * i + 3] << 16;
+                asm volatile("st.volatile.shared.v2.u32 [%0], {%1, %2};" :: "r"((unsigned)__cvta_generic_to_shared(&word[i * STEP])),
+                             "r"(n[4 * i] | n[4 * i + 1] << 16), "r"(n[4 * i + 2] | n[4 * i + 3] << 16) : "memory");
             }
 #pragma unroll
             for (int k = 0; k < 16; ++k) l[k] = n[k];
@@ -544,13 +593,13 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
             if (jw == 0u) continue;
 #pragma unroll
             for (int b = 0; b < 4; ++b)
-                over |= (((jw >> (8 * b)) & 255u) > S.sv[l[4 * i + b] & 0x7FFFu] ? 1u : 0u) << (4 * i + b);
+                over |= (((jw >> (8 * b)) & 255u) > S.sv[l[4 * i + b] - ROOT] ? 1u : 0u) << (4 * i + b);
         }
 #pragma unroll 1
         for (; over; over &= over - 1) {
             const int k = __ffs(over) - 1, i = k >> 2, row = row0 + 16 * i;
             const unsigned j = ((const uint8_t *)bj)[row * BS + 4 * cw + (k & 3)];
-            atomicMax(&S.sv[S.L[(row + 1) * ST + X0 + 4 * cw + (k & 3)] & 0x7FFFu], j);
+            atomicMax(&S.sv[S.L[(row + 1) * ST + X0 + 4 * cw + (k & 3)] - ROOT], j);
         }
     }
     __syncthreads();
@@ -582,7 +631,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
         for (unsigned k = 0; k < mine; k += 32) {
             uint32_t n = 0u;
             if (k + lane < mine) {
-                const uint32_t e = S.tab[seg0 + k + lane], p = (e >> 3) & 0x1FFFu, w = e >> 16;
+                const uint32_t e = S.tab[seg0 + k + lane], p = e >> 3, w = ((const uint8_t *)bi)[p];
                 const unsigned a = S.L[p] & 0x7FFFu, b = S.L[(int)p + ring_off(e & 7u)] & 0x7FFFu;
                 if (a != b && (w > S.sv[a] || w > S.sv[b])) n = a << 20 | b << 8 | w;
             }
@@ -605,7 +654,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
             if (side < 2 || k > 0) ow = max(ow, (unsigned)h[k - 1]);
             if (side < 2 || k < BS - 1) ow = max(ow, (unsigned)h[k + 1]);
         }
-        ow = min(ow, (unsigned)((const uint8_t *)bi)[(py + 1) * IST * 4 + 16 + px]);
+        ow = min(ow, (unsigned)((const uint8_t *)bi)[(py + 1) * ST + X0 + px]);
         ob = S.L[(py + 1) * ST + X0 + px] & 0x7FFFu;
         if (ow) offer(ob, ow << 24 | K_OUT);
     }
@@ -797,8 +846,8 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     const Tile &E = tile_of(P, S.tile);   // (read again: not kept in registers through the rounds)
     {
         const int cell = (r + 1) * ST + X0 + 16 * c;
-        const uint4 iv = *(const uint4 *)&bi[(r + 1) * IST + 4 + 4 * c];
-        const uint32_t iw[4] = {iv.x, iv.y, iv.z, iv.w};
+        const uint2 i0 = *(const uint2 *)&bi[(r + 1) * IST + 2 + 4 * c], i1 = *(const uint2 *)&bi[(r + 1) * IST + 4 + 4 * c];
+        const uint32_t iw[4] = {i0.x, i0.y, i1.x, i1.y};
         uint32_t o[8];   // 16 x (value << 8 | node slot)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
