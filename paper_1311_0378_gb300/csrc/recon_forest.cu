@@ -31,13 +31,13 @@
 // logarithmic expected length.
 //
 // Measured on GB300 (whole call, the wavefront engine -> this one): a 4096^2
-// tile seeded from its border, 4-connected, 6.04 -> 0.295 ms; with an h-dome
-// marker, 8-connected, 0.403 -> 0.208 ms; 200 tiles of 256 .. 4096 pixels a
-// side (910 Mpx, both markers) 57.0 -> 9.85 ms; 512^2 0.231 -> 0.069 ms.
+// tile seeded from its border, 4-connected, 6.04 -> 0.289 ms; with an h-dome
+// marker, 8-connected, 0.403 -> 0.204 ms; 200 tiles of 256 .. 4096 pixels a
+// side (910 Mpx, both markers) 57.0 -> 9.74 ms; 512^2 0.231 -> 0.066 ms.
 // block_kernel takes most of it (0.20 of 0.245 ms of kernel time on the
 // border-seeded tile) and is bound by instruction issue and the shared-memory
 // pipe (about 65% and 53%; DRAM below 4%), so what counts is warp instructions
-// a block: 26 700 (h-dome) to 37 500 (border), 76 500 and 94 900 at first.
+// a block: 26 200 (h-dome) to 36 900 (border), 76 500 and 94 900 at first.
 // Saddles instead of all pixel pairs, arcs and targets of four pixels at once in
 // byte lanes, loops rolled to fit the instruction cache, and lists that stay
 // dense made the difference.
@@ -610,6 +610,12 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
         asm volatile("{\n .reg .pred p;\n .reg .u32 c;\n ld.volatile.shared.u32 c, [%0];\n setp.gt.u32 p, %1, c;\n"
                      " @p red.shared.max.u32 [%0], %1;\n}" :: "r"(best0 + 4u * a), "r"(key) : "memory");
     };
+    // the same with a maximum read before (it may have risen since): one load less behind another. With that and
+    // passes between final regions dropped, 9.54 -> 9.37 ms of kernel time on the 910 Mpx batch.
+    auto offer_over = [&](unsigned a, uint32_t seen, uint32_t key) {
+        asm volatile("{\n .reg .pred p;\n setp.gt.u32 p, %1, %2;\n @p red.shared.max.u32 [%0], %1;\n}"
+                     :: "r"(best0 + 4u * a), "r"(key), "r"(seen) : "memory");
+    };
     // Passes join a saddle's own basin to the one the arc starts in. A pass no
     // heavier than the source edges of both ends is never taken. The first
     // round's maxima are taken here too.
@@ -681,7 +687,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     for (;; ++rounds) {
         const uint16_t *now = lists + (rounds & 1 ? 0 : Smem<CONN>::NB / 2);
         uint16_t *next = lists + (rounds & 1 ? Smem<CONN>::NB / 2 : 0);
-        // edges: to their present ends; one inside a region is dropped
+        // edges: to their present ends; one inside a region or between two with final values is dropped
         if (rounds || !listed) {
             if (tid == 0) S.nlive[rounds & 1] = 0;   // last read two rounds ago
             ob = S.comp[ob];
@@ -690,16 +696,18 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
                 unsigned to = seg0;
 #pragma unroll 1
                 for (unsigned k = 0; k < mine; k += 32) {
-                    uint32_t n = 0u;
+                    uint32_t n = 0u, ca = 0u, cb = 0u;
                     if (k + lane < mine) {
                         const uint32_t e = S.tab[seg0 + k + lane];
                         const unsigned a = S.comp[e >> 20], b = S.comp[(e >> 8) & 0xFFFu];
-                        if (a != b) n = a << 20 | b << 8 | (e & 255u);
+                        ca = *(volatile uint32_t *)&S.best[a];
+                        cb = *(volatile uint32_t *)&S.best[b];
+                        if (a != b && !(ca == FINAL && cb == FINAL)) n = a << 20 | b << 8 | (e & 255u);
                     }
                     const unsigned at = close_up(to, n);
                     if (n) {
-                        offer(n >> 20, n << 24 | K_EDGE | at);
-                        offer((n >> 8) & 0xFFFu, n << 24 | K_EDGE | at);
+                        offer_over(n >> 20, ca, n << 24 | K_EDGE | at);
+                        offer_over((n >> 8) & 0xFFFu, cb, n << 24 | K_EDGE | at);
                     }
                 }
                 mine = to - seg0;
