@@ -31,13 +31,13 @@
 // logarithmic expected length.
 //
 // Measured on GB300 (whole call, the wavefront engine -> this one): a 4096^2
-// tile seeded from its border, 4-connected, 6.04 -> 0.289 ms; with an h-dome
-// marker, 8-connected, 0.403 -> 0.204 ms; 200 tiles of 256 .. 4096 pixels a
-// side (910 Mpx, both markers) 57.0 -> 9.74 ms; 512^2 0.231 -> 0.066 ms.
-// block_kernel takes most of it (0.20 of 0.245 ms of kernel time on the
+// tile seeded from its border, 4-connected, 6.04 -> 0.280 ms; with an h-dome
+// marker, 8-connected, 0.403 -> 0.203 ms; 200 tiles of 256 .. 4096 pixels a
+// side (910 Mpx, both markers) 57.0 -> 9.44 ms; 512^2 0.231 -> 0.066 ms.
+// block_kernel takes most of it (0.195 of 0.235 ms of kernel time on the
 // border-seeded tile) and is bound by instruction issue and the shared-memory
-// pipe (about 65% and 53%; DRAM below 4%), so what counts is warp instructions
-// a block: 26 200 (h-dome) to 36 900 (border), 76 500 and 94 900 at first.
+// pipe (about 65% and 55%; DRAM below 4%), so what counts is warp instructions
+// a block: 25 200 (h-dome) to 35 000 (border), 76 500 and 94 900 at first.
 // Saddles instead of all pixel pairs, arcs and targets of four pixels at once in
 // byte lanes, loops rolled to fit the instruction cache, and lists that stay
 // dense made the difference.
@@ -352,9 +352,10 @@ __device__ __noinline__ void each_pair(Smem<CONN> &S, F f)
 }
 
 // Five CTAs an SM where shared memory allows it (8-connectivity: 43 KB; 4: 56 KB
-// for twice the basins), in 48 registers without spills: 10.40 ms on the 910 Mpx
-// batch. With the timers and the tile's record in registers instead of shared
-// memory there were spills and it took 10.95 ms, with four CTAs 11.13.
+// for twice the basins), in 48 registers without spills: with the timers and the tile's
+// record in registers instead of shared memory there were spills, 10.95 instead of
+// 10.40 ms of kernel time on the 910 Mpx batch when that was done, with four CTAs
+// 11.13.
 template <int CONN>
 __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __grid_constant__ Params P)
 {
@@ -470,7 +471,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     // A lane takes a word of four pixels in each of four rows: 4.5 loads and a
     // quarter of a warp's scan a word instead of 9 and one (10 500 instructions
     // a block with a row each and the labels pixel by pixel; on the 910 Mpx
-    // batch 10.40 ms, 9.54 now).
+    // batch 10.40 -> 9.54 ms of kernel time).
     {
         constexpr int RL = BS / (NT / 16);
         const int row = RL * (2 * warp + (lane >> 4)), cw = lane & 15;
@@ -604,18 +605,10 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     }
     __syncthreads();
     if (tid == 0) S.tick[2] = now_ns();
-    // (a predicated reduction: no branch, and no atomic when the key does not raise the maximum)
-    const unsigned best0 = (unsigned)__cvta_generic_to_shared(S.best);
-    auto offer = [&](unsigned a, uint32_t key) {
-        asm volatile("{\n .reg .pred p;\n .reg .u32 c;\n ld.volatile.shared.u32 c, [%0];\n setp.gt.u32 p, %1, c;\n"
-                     " @p red.shared.max.u32 [%0], %1;\n}" :: "r"(best0 + 4u * a), "r"(key) : "memory");
-    };
-    // the same with a maximum read before (it may have risen since): one load less behind another. With that and
-    // passes between final regions dropped, 9.54 -> 9.37 ms of kernel time on the 910 Mpx batch.
-    auto offer_over = [&](unsigned a, uint32_t seen, uint32_t key) {
-        asm volatile("{\n .reg .pred p;\n setp.gt.u32 p, %1, %2;\n @p red.shared.max.u32 [%0], %1;\n}"
-                     :: "r"(best0 + 4u * a), "r"(key), "r"(seen) : "memory");
-    };
+    // Maxima are taken without a look at the present one first: on the 910 Mpx
+    // batch the load and the compare cost more than the reductions they saved
+    // (9.39 -> 8.84 ms of kernel time).
+    auto offer = [&](unsigned a, uint32_t key) { atomicMax(&S.best[a], key); };
     // Passes join a saddle's own basin to the one the arc starts in. A pass no
     // heavier than the source edges of both ends is never taken. The first
     // round's maxima are taken here too.
@@ -687,7 +680,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     for (;; ++rounds) {
         const uint16_t *now = lists + (rounds & 1 ? 0 : Smem<CONN>::NB / 2);
         uint16_t *next = lists + (rounds & 1 ? Smem<CONN>::NB / 2 : 0);
-        // edges: to their present ends; one inside a region or between two with final values is dropped
+        // edges: to their present ends; one inside a region is dropped
         if (rounds || !listed) {
             if (tid == 0) S.nlive[rounds & 1] = 0;   // last read two rounds ago
             ob = S.comp[ob];
@@ -696,18 +689,16 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
                 unsigned to = seg0;
 #pragma unroll 1
                 for (unsigned k = 0; k < mine; k += 32) {
-                    uint32_t n = 0u, ca = 0u, cb = 0u;
+                    uint32_t n = 0u;
                     if (k + lane < mine) {
                         const uint32_t e = S.tab[seg0 + k + lane];
                         const unsigned a = S.comp[e >> 20], b = S.comp[(e >> 8) & 0xFFFu];
-                        ca = *(volatile uint32_t *)&S.best[a];
-                        cb = *(volatile uint32_t *)&S.best[b];
-                        if (a != b && !(ca == FINAL && cb == FINAL)) n = a << 20 | b << 8 | (e & 255u);
+                        if (a != b) n = a << 20 | b << 8 | (e & 255u);
                     }
                     const unsigned at = close_up(to, n);
                     if (n) {
-                        offer_over(n >> 20, ca, n << 24 | K_EDGE | at);
-                        offer_over((n >> 8) & 0xFFFu, cb, n << 24 | K_EDGE | at);
+                        offer(n >> 20, n << 24 | K_EDGE | at);
+                        offer((n >> 8) & 0xFFFu, n << 24 | K_EDGE | at);
                     }
                 }
                 mine = to - seg0;
@@ -771,7 +762,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
             for (unsigned u; (u = S.up[t]) != t;) t = u;
             if (t != b) {   // merged this round
                 S.comp[b] = (uint16_t)t;
-                if (S.sv[b] > *(volatile uint32_t *)&S.sv[t]) atomicMax(&S.sv[t], S.sv[b]);
+                atomicMax(&S.sv[t], S.sv[b]);
             } else if (S.best[b] < FINAL) {
                 S.best[b] = 0u;
                 next[atomicAdd(&S.nlive[rounds & 1], 1u)] = (uint16_t)b;
@@ -803,8 +794,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
             w = min(w, min(fa >> 8, fb >> 8));
             if (na == nb2 || w == 0) return 0u;
             if (na != RES && nb2 != RES) return na << 16 | nb2 << 8 | w;   // between two nodes
-            uint32_t *l = &S.link[na == RES ? nb2 : na];
-            if ((w << 8 | RES) > *(volatile uint32_t *)l) atomicMax(l, w << 8 | RES);
+            atomicMax(&S.link[na == RES ? nb2 : na], w << 8 | RES);
             return 0u;
         };
         // (best and sv, next to each other, are no longer needed: room for every pass)
