@@ -2,12 +2,13 @@
 """Throughput of grayscale morphological reconstruction on GB300.
 
 One step = the whole reconstruction of one batch of synthetic tiles through
-the C ABI (marker reset from its pristine copy, the learned schedule's
-planning pass, validation, scan pairs, queue propagation, neighbour
-notification, persistent launch replayed from a CUDA graph). Default workload
+the C ABI (marker reset from its pristine copy, validation, and the
+region-merging engine's launches; with a wavefront setting -- --block-h,
+--bands, --sweeps, --autotune -- instead the learned schedule's planning pass,
+scan pairs and queue propagation in one persistent launch). Default workload
 "uneven1000": 1000 tiles whose heights and widths are drawn from
 {256, 512, ..., 4096} (4.7 Gpx, h-dome and fill-holes markers 50/50,
-8-connectivity), reconstructed in one persistent launch. Metric:
+8-connectivity), reconstructed in one call. Metric:
 reconstructed Mpix/s. "single4096" is one 4096 x 4096 mask reconstructed four
 times (4-/8-connectivity x both markers); "batch64" is 64 tiles of 4096 x 4096.
 
@@ -17,10 +18,10 @@ same propagation work as the dilation tiles) or "fill_holes" (FillHoles of
 every distinct (mask, connectivity) of the workload; the output needs no
 reset, so a step is the library call alone) or "dt" (the distance transform of
 the workload's masks: objects I >= 100 and the space between them).
-The line's "compare" block (skip it with --no-compare) times the plain
-schedule, the per-tile launch loop, the learned schedule with and without its
-planning pass, and the sweep-only and queue-first halves of the method with
-their own rooflines. "cpu_baseline" is the CPU oracle on a bounded sample of
+The line's "compare" block (skip it with --no-compare) times the wavefront
+engine on the same batch: its plain schedule, the per-tile launch loop, the
+learned schedule with and without its planning pass, and the sweep-only and
+queue-first halves of the method with their own rooflines. "cpu_baseline" is the CPU oracle on a bounded sample of
 the workload, on all host cores and on one core. --microbench runs the
 random-access and atomic micro-benchmarks instead; --tile T reconstructs one
 tile alone (a small fixed case for profilers); --subset n keeps every n-th
@@ -63,12 +64,17 @@ def code_of(text):
     return "\n".join(l.strip() for l in text.splitlines() if l.strip())
 
 
-def kernel_hash(read=None):
-    """Hash of the reconstruction kernel's code (comments excluded), to tell
-    whether committed ncu counters still describe it."""
+WAVEFRONT_FILES = ("paper_1311_0378_gb300/csrc/recon_kernels.cu", "paper_1311_0378_gb300/csrc/recon_internal.h")
+MERGING_FILES = ("paper_1311_0378_gb300/csrc/recon_forest.cu", "paper_1311_0378_gb300/csrc/recon_forest.h",
+                 "paper_1311_0378_gb300/csrc/recon_internal.h")
+
+
+def kernel_hash(read=None, files=WAVEFRONT_FILES):
+    """Hash of an engine's code (comments excluded), to tell whether committed
+    ncu counters still describe it."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("paper_1311_0378_gb300/csrc/recon_kernels.cu", "paper_1311_0378_gb300/csrc/recon_internal.h"):
+    for f in files:
         if read:
             text = read(f)
         else:
@@ -86,10 +92,36 @@ def measured_traffic(workload):
             t = json.load(f)
     except OSError:
         return None
-    if t.get("kernel_source_sha256_16") != kernel_hash():
+    if t.get("kernel_source_sha256_16") != kernel_hash(files=MERGING_FILES):
         return None
     w = t.get("workloads", {}).get(workload)
     return w.get("dram_bytes_per_launch") if w else None
+
+
+def merging_launches(rc, ctx, tiles):
+    """Kernel launches of a batch on the region-merging engine, or None when the
+    context's settings ask for the wavefront engine. Tiles of one connectivity
+    form groups of up to 65536 blocks of 64 x 64; a group takes three launches
+    (one when every tile of it is a single block)."""
+    want = ((rc.RECON_P_BLOCK_H, 128), (rc.RECON_P_BANDS, 4), (rc.RECON_P_SWEEPS, 1),
+            (rc.RECON_P_TMA, 1), (rc.RECON_P_REVISIT_SCANS, 0), (rc.RECON_P_SCAN_GAIN, 2048))
+    if os.environ.get("RECON_GRID") or any(rc.recon_get_param(ctx, p) != v for p, v in want):
+        return None
+    n = 0
+    for conn in (8, 4):
+        left, flat = 0, True
+        for t in tiles:
+            if t.conn != conn:
+                continue
+            nb = -(-t.H // 64) * -(-t.W // 64)
+            if left and left + nb > 65536:
+                n += 1 if flat else 3
+                left, flat = 0, True
+            left += nb
+            flat = flat and nb == 1
+        if left:
+            n += 1 if flat else 3
+    return n
 
 
 def peaks():
@@ -346,9 +378,10 @@ def time_fn(fn, stream, J, J0, flush, reps=3):
 
 
 def compare_schedules(rc, ctx, stream, Is, Js, J0, tiles, desc, px, flush, args):
-    """Batched persistent launch vs a per-tile launch loop, and the learned
-    schedule vs the plain one, on the same tiles and GPU (outputs identical:
-    R is unique; the tests check it)."""
+    """The wavefront engine (explicit schedules ask for it): batched persistent
+    launch vs a per-tile launch loop, and the learned schedule vs the plain
+    one, on the same tiles and GPU (outputs identical: R is unique; the tests
+    check it)."""
     res = {}
     k_default = rc.recon_get_param(ctx, rc.RECON_P_SWEEPS)
     g_default = rc.recon_get_param(ctx, rc.RECON_P_SCAN_GAIN)
@@ -627,7 +660,7 @@ def main():
     ap.add_argument("--impl", default="gb300", choices=["gb300", "reference"])
     ap.add_argument("--workload", default="uneven1000",
                     choices=["uneven1000", "batch64", "single4096", "single512"],
-                    help="uneven1000 (default): 1000 tiles of uneven sizes, 4.7 Gpx, one persistent launch")
+                    help="uneven1000 (default): 1000 tiles of uneven sizes, 4.7 Gpx, one call")
     ap.add_argument("--op", default="dilate", choices=OPS,
                     help="dilate: reconstruction by dilation; erode: by erosion (complemented pairs); "
                          "fill_holes: FillHoles of the masks")
@@ -646,8 +679,8 @@ def main():
                     help="with --tile: KEY=VALUE context parameter, KEY a RECON_P_* suffix")
     ap.add_argument("--autotune", action="store_true")
     ap.add_argument("--schedule", default="learned", choices=["learned", "plain"],
-                    help="learned: the cost model picks each tile's variant and the packing order "
-                         "(planning runs inside every timed step); plain: context defaults")
+                    help="of the wavefront engine. learned: the cost model picks each tile's variant and the "
+                         "packing order (planning runs inside every timed step); plain: context defaults")
     ap.add_argument("--microbench", action="store_true",
                     help="run the random-access and atomic micro-benchmarks (Tables III-IV) instead")
     args = ap.parse_args()
@@ -716,6 +749,8 @@ def main():
               "schedule": args.schedule,
               "cost_model": ({"tiles": model_meta.get("tiles"), "variants": model_meta.get("variants")}
                              if model_meta else None)}
+    merging = merging_launches(rc, ctx, tiles)
+    params["engine"] = "wavefront" if merging is None else "region merging"
     px = sum(t.H * t.W for t in tiles)          # this rank's pixels per step
     job_px = sum(t.H * t.W for t in job)        # every rank's pixels per step
     flush = torch.empty(512 << 20, dtype=torch.uint8, device=dev)
@@ -801,12 +836,14 @@ def main():
     alg = ALG_BYTES_PER_PX[args.op]
     achieved = alg * px / (kms / 1e3) / 1e9
     traffic_key = w.name if args.op == "dilate" else "%s:%s" % (w.name, args.op)
-    traffic = measured_traffic(traffic_key) if args.subset == 1 and world == 1 else None
+    traffic = measured_traffic(traffic_key) if args.subset == 1 and world == 1 and merging is not None else None
     roof = {"bound": "hbm", "achieved": round(achieved, 2), "peak": pk["hbm_gbs"], "unit": "GB/s",
             "frac": round(achieved / pk["hbm_gbs"], 5), "traffic": traffic,
-            "kernel": "recon_persistent", "kernel_ms": round(kms, 4),
+            "kernel": "recon_persistent" if merging is None else "block_kernel, rim_kernel, value_kernel",
+            "kernel_ms": round(kms, 4),
             "alg_bytes_per_px": alg, "alg_bytes_per_launch": alg * px, "peak_source": src,
-            "limiter": "propagation depth and shared-memory latency of thin wavefronts (not DRAM)"}
+            "limiter": ("propagation depth and shared-memory latency of thin wavefronts (not DRAM)" if merging is None
+                        else "instruction issue and shared-memory latency of block_kernel (not DRAM)")}
     if traffic:
         roof["dram_GBps"] = round(traffic / (kms / 1e3) / 1e9, 2)
         roof["dram_frac"] = round(traffic / (kms / 1e3) / 1e9 / pk["hbm_gbs"], 5)
@@ -824,9 +861,9 @@ def main():
                    **params},
         "roofline": roof,
         "e2e": {"value": round(e2e, 2), "unit": "Mpix/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-        # per step: init + persistent kernel, plus features, finalize and MLP forward
-        # when learned, plus the marker kernel for FillHoles
-        "gpu_launches": ((5 if learned else 2) + (0 if reset_j else 1)) * args.steps,
+        # per step: the groups' launches, or init + persistent kernel, plus features, finalize
+        # and MLP forward when learned, plus the marker kernel for FillHoles
+        "gpu_launches": (((5 if learned else 2) + (0 if reset_j else 1)) if merging is None else merging) * args.steps,
         "compare": compare,
         "clocks": clk.summary(),
     }

@@ -465,8 +465,8 @@ static int stage_meta(recon_ctx *c, const recon_tile *tiles, int n, const int *v
 // engine: when the context's wavefront settings are all at their defaults.
 // Setting any of them (recon_set_param, RECON_*, recon_autotune) or passing
 // variants or an order asks for the wavefront engine. The merging engine was
-// faster at every size, marker, connectivity and operation measured, by 1.8
-// (4096^2, h-dome: 405 -> 229 us) to 24 times (holes filled: 2.66 -> 0.112 ms),
+// faster at every size, marker, connectivity and operation measured, by 2
+// (4096^2, h-dome: 403 -> 204 us) to 26 times (holes filled: 2.67 -> 0.104 ms),
 // so there is no size below or above which the other is chosen.
 static bool use_forest(const recon_ctx *c)
 {
