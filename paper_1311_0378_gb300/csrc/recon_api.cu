@@ -381,6 +381,7 @@ static int ensure_stage(recon_ctx *c, size_t total)
 {
     CK(cudaEventSynchronize(c->meta_free));
     if (c->cap_hmeta < total) {
+        drop_graph(c);   // its copy reads the buffer that goes
         if (c->h_meta) cudaFreeHost(c->h_meta);
         c->h_meta = nullptr;
         c->cap_hmeta = 0;
