@@ -84,6 +84,8 @@ struct recon_ctx {
     unsigned char *d_dt = nullptr; size_t cap_dt = 0;
     // training scratch (moments, epoch losses, two epochs' sample orders)
     unsigned char *d_train = nullptr; size_t cap_train = 0;
+    int *h_order = nullptr; size_t cap_order = 0;   // pinned: the orders as the host shuffles them
+    cudaEvent_t order_free[2] = {};                 // each one's copy is done
     // autotuner results: (size bucket, connectivities, marker class) -> {bh, bands, k, gain}
     std::map<std::tuple<int, int, int>, std::vector<int>> tune_cache;
     int tune_from_cache = 0;
@@ -207,6 +209,9 @@ extern "C" int recon_free(recon_ctx *c)
     cudaFree(c->d_img);
     cudaFree(c->d_dt);
     cudaFree(c->d_train);
+    if (c->h_order) cudaFreeHost(c->h_order);
+    for (cudaEvent_t e : c->order_free)
+        if (e) cudaEventDestroy(e);
     if (c->h_ctl) cudaFreeHost(c->h_ctl);
     if (c->h_meta) cudaFreeHost(c->h_meta);
     if (c->h_trace) cudaFreeHost(c->h_trace);
@@ -1070,8 +1075,24 @@ static uint64_t sm64(uint64_t z)
     return z ^ (z >> 31);
 }
 
+// The two sample orders of a training run in pinned memory, n indices each.
+static int ensure_orders(recon_ctx *c, size_t n)
+{
+    for (cudaEvent_t &e : c->order_free)
+        if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    if (c->cap_order < 2 * n) {
+        if (c->h_order) cudaFreeHost(c->h_order);
+        c->h_order = nullptr;
+        c->cap_order = 0;
+        CK(cudaMallocHost((void **)&c->h_order, sizeof(int) * 2 * n));
+        c->cap_order = 2 * n;
+    }
+    return RECON_OK;
+}
+
 // Epochs epoch0 .. epoch0 + epochs - 1 of mini-batch Adam, one launch each. The
-// host shuffles the next epoch while one runs; the two index buffers alternate.
+// host shuffles the next epoch while one runs: two orders take turns, each refilled
+// once the copy out of it, queued behind the epoch before, is done.
 // adam_mv NULL: moments in the context's scratch, starting at zero.
 static int train_epochs(recon_ctx *c, float *theta, float *adam_mv, int *step, int epoch0, const float *X, const float *T,
                         int n, int epochs, int batch, float lr, uint64_t seed, float *epoch_loss)
@@ -1081,6 +1102,7 @@ static int train_epochs(recon_ctx *c, float *theta, float *adam_mv, int *step, i
     const size_t off_loss = align_up(sizeof(float) * 2 * MLP_NPARAMS, 16);
     const size_t off_idx = align_up(off_loss + sizeof(float) * (size_t)epochs, 16);
     int rc = grow(&c->d_train, &c->cap_train, off_idx + sizeof(int) * 2 * (size_t)n);
+    if (rc == RECON_OK) rc = ensure_orders(c, (size_t)n);
     if (rc) return rc;
     float *mv = adam_mv ? adam_mv : (float *)c->d_train, *dl = (float *)(c->d_train + off_loss);
     int *didx = (int *)(c->d_train + off_idx);
@@ -1088,11 +1110,13 @@ static int train_epochs(recon_ctx *c, float *theta, float *adam_mv, int *step, i
     cudaError_t e = adam_mv ? cudaMemsetAsync(dl, 0, sizeof(float) * (size_t)epochs, c->stream)
                             : cudaMemsetAsync(c->d_train, 0, off_idx, c->stream);
     batch = std::min(batch, n);
-    std::vector<int> perm(n);
     int t = *step;
     const int nbatches = (n - 1) / batch + 1;
     for (int k = 0; k < epochs && e == cudaSuccess; ++k) {
         const int ep = epoch0 + k;   // the shuffle depends on the absolute epoch, so a resumed run repeats it
+        int *const perm = c->h_order + (size_t)(k & 1) * n, *const buf = didx + (size_t)(k & 1) * n;
+        if (k >= 2) e = cudaEventSynchronize(c->order_free[k & 1]);
+        if (e != cudaSuccess) break;
         // Fisher-Yates shuffle driven by SplitMix64 outputs of (seed, epoch)
         for (int i = 0; i < n; ++i) perm[i] = i;
         uint64_t st = sm64(seed ^ sm64((uint64_t)ep + 1));
@@ -1101,9 +1125,8 @@ static int train_epochs(recon_ctx *c, float *theta, float *adam_mv, int *step, i
             const int j = (int)(st % (uint64_t)(i + 1));
             std::swap(perm[i], perm[j]);
         }
-        int *buf = didx + (size_t)(k & 1) * n;
-        // returns once the pageable source is staged, so perm may be refilled
-        e = cudaMemcpyAsync(buf, perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream);
+        e = cudaMemcpyAsync(buf, perm, sizeof(int) * n, cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(c->order_free[k & 1], c->stream);
         if (e == cudaSuccess)
             e = rl_train_epoch(theta, mv, mv + MLP_NPARAMS, X, T, buf, n, batch, t, lr, dl + k, c->stream);
         t += nbatches;

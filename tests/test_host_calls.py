@@ -1,6 +1,8 @@
 """What the library's host code does around its kernels, on a CUDA runtime of
 host memory (host_runtime.cpp): which buffers outlive which work, what a failed
 allocation leaves behind, what a call reports."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -34,3 +36,37 @@ def test_graph_is_not_replayed_from_a_staging_buffer_that_is_gone(rc):
     assert rc.lib().ht_faults() == 0
     assert host_runtime.counts(rc)["graph"] == 3
     rc.recon_free(c)
+
+
+def mix(z):
+    z = (z + 0x9E3779B97F4A7C15) % (1 << 64)
+    z = ((z ^ (z >> 30)) * 0xBF58476D1CE4E5B9) % (1 << 64)
+    z = ((z ^ (z >> 27)) * 0x94D049BB133111EB) % (1 << 64)
+    return z ^ (z >> 31)
+
+
+def order(n, seed, epoch):
+    perm, st = list(range(n)), mix(seed ^ mix(epoch + 1))
+    for i in range(n - 1, 0, -1):
+        st = mix(st)
+        perm[i], perm[st % (i + 1)] = perm[st % (i + 1)], perm[i]
+    return perm
+
+
+@pytest.mark.parametrize("n,epochs", [(1, 3), (7, 1), (50, 2), (1000, 6), (20000, 3)])
+def test_every_epoch_trains_on_its_own_order(rc, n, epochs):
+    """The host shuffles ahead; an order is copied only when the device gets to it."""
+    c = rc.recon_init(0, 0, rc.RECON_FLAG_SYNC)
+    a = np.zeros(3 * rc.RECON_MLP_NPARAMS, np.float32)
+    X = np.zeros((n, 22), np.float32)
+    st, losses = rc.recon_mlp_train(c, a.ctypes.data, X.ctypes.data, X.ctypes.data, n, epochs, n, 1e-3, 5)
+    assert st == rc.RECON_OK and losses == [1.0] * epochs
+    st, step, losses = rc.recon_mlp_train_resume(c, a.ctypes.data, a.ctypes.data, epochs, epochs, X.ctypes.data,
+                                                 X.ctypes.data, n, 2, n, 1e-3, 5)
+    assert st == rc.RECON_OK and step == epochs + 2
+    got = (ctypes.c_int * (n * (epochs + 2)))()
+    assert rc.lib().ht_orders(got, len(got)) == len(got)
+    for e in range(epochs + 2):
+        assert list(got[e * n:(e + 1) * n]) == order(n, 5, e), e
+    rc.recon_free(c)
+    assert rc.lib().ht_faults() == 0
