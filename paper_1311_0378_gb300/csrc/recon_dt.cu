@@ -32,6 +32,7 @@ namespace dt {
 
 constexpr unsigned INF = 0x7FFFFFFFu;   // above every squared distance (2 * 32767^2); INF + dx^2 fits 32 bits
 constexpr uint32_t FAR = 32767u + 1u;   // more than any distance within a column
+constexpr int WMAX = 32768;             // widest row
 constexpr int PAD = 128;                // columns of INF at both ends of a row in shared memory
 
 // A kernel may be launched when the last CTAs of the one before it run, and
@@ -310,6 +311,13 @@ __global__ void row_site_kernel(const uint16_t *G, int H, int W, int pitch, unsi
 static size_t mask_bytes(int H, int W) { return (((size_t)((H + 31) / 32) * W * sizeof(uint32_t)) + 255) / 256 * 256; }
 static int g_pitch(int W) { return (W + 1) / 2 * 2; }
 
+// Shared memory of the row kernels: the padded row, its runs' minima, with sites the distances with their direction.
+static size_t row_smem(int W, bool site)
+{
+    return sizeof(uint32_t) * ((size_t)(W + 1) / 2 * 2 + 2 * dt::PAD + 2 + (W + 31) / 32) +
+           (site ? sizeof(uint16_t) * (size_t)W : 0);
+}
+
 size_t dt_scratch_bytes(int H, int W) { return mask_bytes(H, W) + (size_t)H * g_pitch(W) * sizeof(uint16_t); }
 
 // Launches a kernel behind the one before it on the stream, as its dependent.
@@ -342,11 +350,12 @@ int dt_run(const uint8_t *B, int H, int W, int *site, unsigned *d2, void *scratc
     // a CTA per row; more threads where a wide row's shared memory leaves room for few CTAs
     const int px = site ? W : (W + 1) / 2;
     const int T = W > 8192 ? 1024 : std::min(256, (px + 31) / 32 * 32);
-    const size_t smem = sizeof(uint32_t) * ((size_t)(W + 1) / 2 * 2 + 2 * dt::PAD + 2 + (W + 31) / 32) +
-                        (site ? sizeof(uint16_t) * (size_t)W : 0);
+    const size_t smem = row_smem(W, site != nullptr);
+    // the limit belongs to the kernel, not to the call: the same for every call (that of the widest row),
+    // so that calls of other threads cannot lower it between this line and the launch
     const void *fn = site ? (const void *)dt::row_site_kernel : (const void *)dt::row_kernel;
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)row_smem(dt::WMAX, site != nullptr)) != cudaSuccess)
         return DT_ECUDA;
     const int grid = std::min(H, 64 * std::max(1, sms));
     if (e == cudaSuccess)
