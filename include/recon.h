@@ -123,7 +123,9 @@ int recon_run_op(recon_ctx *ctx, const uint8_t *I, uint8_t *J, int H, int W, int
  * Tiles must not overlap in memory. With RECON_FLAG_LEARNED the cost model
  * chooses each tile's variant and the packing order when the wavefront engine
  * runs (never the pixel values).
- * 1 <= n <= 2^28 (RECON_EINVAL otherwise).
+ * 1 <= n <= 2^28 (RECON_EINVAL otherwise). A stream under capture is refused
+ * (RECON_ECUDA; the capture stays valid), by every reconstruction call on a
+ * context.
  * On a device error, recon_last_error_tile names the first failing tile. */
 int recon_batch(recon_ctx *ctx, const recon_tile *tiles, int n);
 

@@ -516,7 +516,7 @@ static rf::Params forest_params(const recon_ctx *c, unsigned nblocks, int ntiles
 // three launches per group of tiles. *done = 0 when the batch does not fit that
 // engine (nothing was launched). Launched directly, not as a graph: a graph
 // would be rebuilt whenever a call brings other buffers.
-static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, bool capturing, int *done)
+static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, int *done)
 {
     *done = 0;
     struct Group { int conn, first, count; unsigned nblocks; int flat; size_t off_base; };
@@ -553,8 +553,7 @@ static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, bool captu
         g.off_base = total;
         total += align_up(sizeof(unsigned) * ((size_t)g.count + 1), 16);
     }
-    // One tile travels with its launches. (A captured call runs again and again, and so clears its own status.)
-    const bool one = n == 1 && c->status_turn >= 0 && !capturing;
+    const bool one = n == 1 && c->status_turn >= 0;   // one tile travels with its launches
     const size_t need = rf::scratch_bytes(most);
     int rc;
     if ((!one && c->cap_fmeta < total) || c->cap_forest < need) {
@@ -635,14 +634,15 @@ static int batch_impl(recon_ctx *c, const recon_tile *tiles, int n, const int *v
                 return RECON_EINVAL;
     CK(cudaSetDevice(c->device));
 
+    // A stream that the caller is capturing is refused before anything touches it: the calls wait for
+    // events, upload lists that the next call refills, and take turns with status areas.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(c->stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return RECON_ECUDA;
+
     if (!variant && !order && use_forest(c)) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CK(cudaStreamIsCapturing(c->stream, &cap));
-        const bool capturing = cap != cudaStreamCaptureStatusNone;
-        // a stream the caller is capturing is refused, as the graph path below refuses it
-        if (capturing && !(c->flags & RECON_FLAG_NO_GRAPH)) return RECON_ECUDA;
         int done = 0;
-        const int frc = forest_batch(c, tiles, n, capturing, &done);
+        const int frc = forest_batch(c, tiles, n, &done);
         if (done || frc != RECON_OK) return frc;
     }
 

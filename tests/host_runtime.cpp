@@ -38,6 +38,7 @@ std::map<unsigned char *, size_t> live, dead;
 size_t dev_bytes = 0, dev_limit = SIZE_MAX;
 std::map<unsigned char *, size_t> dev;   // sizes of device allocations
 int faults = 0;
+int broken = 0;                          // waits for a stream under capture
 double now_ms = 0.0;                     // device clock: a kernel takes a nanosecond a pixel
 int n_merging = 0, n_wavefront = 0, n_graph = 0, n_plan = 0;
 std::vector<int> orders;                 // sample orders of the epochs trained
@@ -123,6 +124,8 @@ void fail(rk::Ctl *ctl, int *tile_err, int index)
 
 // ---- what the tests read and set
 extern "C" int ht_faults() { return faults; }
+extern "C" int ht_broken_captures() { return broken; }
+extern "C" int ht_graph_nodes(cudaGraph_t g) { return (int)g->ops.size(); }
 extern "C" void ht_device_limit(size_t bytes) { dev_limit = bytes; }
 extern "C" size_t ht_device_bytes() { return dev_bytes; }
 extern "C" void ht_counts(int *out)
@@ -198,7 +201,15 @@ cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t st)
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = new CUstream_st; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { delete s; return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t s) { run_to(s->last); return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t s)
+{
+    if (s->capture) {
+        ++broken;
+        return cudaErrorStreamCaptureUnsupported;
+    }
+    run_to(s->last);
+    return cudaSuccess;
+}
 cudaError_t cudaStreamQuery(cudaStream_t s) { return s->last <= done ? cudaSuccess : cudaErrorNotReady; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }   // one queue: in order
 cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus *st)

@@ -30,7 +30,8 @@ def _build(folder):
 
 def load(tmp_path):
     if not _built:
-        _built.append(_build(tempfile.mkdtemp()))
+        folder = tempfile.TemporaryDirectory()   # kept, and removed at exit, with the list
+        _built[:] = [_build(folder.name), folder]
     lib = shutil.copy(_built[0], str(tmp_path))
     spec = importlib.util.spec_from_file_location("recon_host", rc.__file__)
     m = importlib.util.module_from_spec(spec)

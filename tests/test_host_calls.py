@@ -70,3 +70,26 @@ def test_every_epoch_trains_on_its_own_order(rc, n, epochs):
         assert list(got[e * n:(e + 1) * n]) == order(n, 5, e), e
     rc.recon_free(c)
     assert rc.lib().ht_faults() == 0
+
+
+@pytest.mark.parametrize("flag", [0, "RECON_FLAG_NO_GRAPH"])
+@pytest.mark.parametrize("wavefront", [False, True])
+@pytest.mark.parametrize("n", [1, 3])
+def test_a_capturing_stream_is_refused_untouched(rc, flag, wavefront, n):
+    L, st = rc.lib(), ctypes.c_void_p()
+    assert L.cudaStreamCreateWithFlags(ctypes.byref(st), 0) == 0
+    c = rc.recon_init(0, st.value, rc.RECON_FLAG_SYNC | (getattr(rc, flag) if flag else 0))
+    tiles = [tile(70, 65) for _ in range(n)]
+    def run():
+        desc = [t[2] for t in tiles]
+        return rc.recon_batch_ex(c, desc, [1] * n, list(range(n))) if wavefront else rc.recon_batch(c, desc)
+    for warm in range(2):
+        assert L.cudaStreamBeginCapture(st, 0) == 0
+        assert run() == rc.RECON_ECUDA
+        g = ctypes.c_void_p()
+        assert L.cudaStreamEndCapture(st, ctypes.byref(g)) == 0
+        assert L.ht_broken_captures() == 0 and L.ht_graph_nodes(g) == 0 and L.cudaGraphDestroy(g) == 0
+        assert run() == rc.RECON_OK and done(tiles)
+        for t in tiles:
+            t[1][:] = 0
+    rc.recon_free(c)
