@@ -118,6 +118,17 @@ static int grow(T **p, size_t *cap, size_t need)
     return RECON_OK;
 }
 
+// Before the buffers of the last call's status and counters are replaced (which can fail): the status
+// moves to the host, where recon_sync finds it; the counters are given up.
+static int settle(recon_ctx *c)
+{
+    const int st = recon_sync(c);
+    c->last_n = 0;
+    if (st == RECON_ECUDA) return st;
+    c->host_status = 1;
+    return RECON_OK;
+}
+
 static void drop_graph(recon_ctx *c)
 {
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
@@ -557,10 +568,9 @@ static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, int *done)
     const size_t need = rf::scratch_bytes(most);
     int rc;
     if ((!one && c->cap_fmeta < total) || c->cap_forest < need) {
-        CK(cudaStreamSynchronize(c->stream));
-        if (!one && c->last_ctl == (rk::Ctl *)c->d_fmeta) c->launched = 0;   // that call's status goes with the buffer
-        if (!one && (rc = grow(&c->d_fmeta, &c->cap_fmeta, total))) return rc;
-        rc = grow(&c->d_forest, &c->cap_forest, need);
+        if ((rc = settle(c))) return rc;
+        rc = one ? RECON_OK : grow(&c->d_fmeta, &c->cap_fmeta, total);
+        if (rc == RECON_OK) rc = grow(&c->d_forest, &c->cap_forest, need);
         if (rc == RECON_ENOMEM) return RECON_OK;   // the wavefront engine needs far less scratch
         if (rc) return rc;
     }
@@ -672,7 +682,7 @@ static int batch_impl(recon_ctx *c, const recon_tile *tiles, int n, const int *v
     const bool need = c->cap_meta < bytes || c->cap_blocks < nblocks || c->cap_ring < ring_cap ||
                       c->cap_tiles < (size_t)n || c->cap_spill_ctas < (size_t)grid || !c->d_state || !c->d_ring;
     if (need) {
-        CK(cudaStreamSynchronize(c->stream));
+        if ((rc = settle(c))) return rc;
         drop_graph(c);
         if ((rc = grow(&c->d_meta, &c->cap_meta, bytes))) return rc;
         if (c->cap_blocks < nblocks || c->cap_ring < ring_cap || !c->d_state || !c->d_ring) {

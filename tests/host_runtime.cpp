@@ -22,13 +22,14 @@
 #include "recon_forest.h"
 #include "recon_learn.h"
 
+struct CUevent_st { size_t last = 0; double at = 0.0; };
+struct Op { std::function<void()> f; cudaEvent_t records; };
 struct CUstream_st {
-    std::vector<std::function<void()>> *capture = nullptr;
+    std::vector<Op> *capture = nullptr;
     size_t last = 0;   // number of its latest operation
 };
-struct CUevent_st { size_t last = 0; double at = 0.0; };
-struct CUgraph_st { std::vector<std::function<void()>> ops; };
-struct CUgraphExec_st { std::vector<std::function<void()>> ops; };
+struct CUgraph_st { std::vector<Op> ops; };
+struct CUgraphExec_st { std::vector<Op> ops; };
 
 namespace {
 
@@ -53,14 +54,15 @@ void run_to(size_t n)
     }
 }
 
-void put(cudaStream_t s, std::function<void()> f)
+void put(cudaStream_t s, std::function<void()> f, cudaEvent_t records = nullptr)
 {
     if (s->capture) {
-        s->capture->push_back(std::move(f));
+        s->capture->push_back(Op{std::move(f), records});
         return;
     }
     queue.push_back(std::move(f));
     s->last = ++queued;
+    if (records) records->last = queued;
 }
 
 bool overlaps(const std::map<unsigned char *, size_t> &m, const void *p, size_t n)
@@ -222,8 +224,7 @@ cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { *e = new CUeven
 cudaError_t cudaEventDestroy(cudaEvent_t e) { delete e; return cudaSuccess; }
 cudaError_t cudaEventRecordWithFlags(cudaEvent_t e, cudaStream_t s, unsigned)
 {
-    put(s, [=] { e->at = now_ms; });
-    if (!s->capture) e->last = s->last;
+    put(s, [=] { e->at = now_ms; }, e);
     return cudaSuccess;
 }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) { return cudaEventRecordWithFlags(e, s, 0); }
@@ -235,7 +236,7 @@ cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t a, cudaEvent_t b)
 }
 cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode)
 {
-    s->capture = new std::vector<std::function<void()>>;
+    s->capture = new std::vector<Op>;
     return cudaSuccess;
 }
 cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t *g)
@@ -255,8 +256,8 @@ cudaError_t cudaGraphExecDestroy(cudaGraphExec_t x) { delete x; return cudaSucce
 cudaError_t cudaGraphLaunch(cudaGraphExec_t x, cudaStream_t s)
 {
     ++n_graph;
-    for (auto &f : x->ops) put(s, f);
-    return cudaSuccess;   // (an event recorded inside keeps its place: waits for it may end early)
+    for (auto &op : x->ops) put(s, op.f, op.records);
+    return cudaSuccess;
 }
 
 // ---- wavefront kernels

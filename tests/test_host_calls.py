@@ -93,3 +93,51 @@ def test_a_capturing_stream_is_refused_untouched(rc, flag, wavefront, n):
         for t in tiles:
             t[1][:] = 0
     rc.recon_free(c)
+
+
+@pytest.mark.parametrize("first_wavefront", [False, True])
+@pytest.mark.parametrize("then_wavefront", [False, True])
+@pytest.mark.parametrize("violation", [False, True])
+def test_a_failed_allocation_leaves_nothing_stale(rc, first_wavefront, then_wavefront, violation):
+    """A call that cannot grow its buffers: the status of the call before it stays,
+    its counters are refused (their buffer may be gone), and the next call works."""
+    c = rc.recon_init(0, 0, 0)
+
+    def run(tiles, wavefront):
+        n, desc = len(tiles), [t[2] for t in tiles]
+        return rc.recon_batch_ex(c, desc, [1] * n, list(range(n))) if wavefront else rc.recon_batch(c, desc)
+    few, many = [tile(5, 5) for _ in range(3)], [tile(2, 2) for _ in range(3000)]
+    if violation:
+        few[1][1][0, 0] = 10
+    assert run(few, first_wavefront) == rc.RECON_OK
+    status = rc.RECON_EMARKER if violation else rc.RECON_OK
+    if not violation:
+        assert [w["visits"] for w in rc.recon_get_work(c, 3)] == [1, 1, 1]
+    rc.lib().ht_device_limit(rc.lib().ht_device_bytes())
+    assert run(many, then_wavefront) == rc.RECON_ENOMEM
+    assert rc.recon_sync(c) == status and rc.recon_last_error_tile(c) == (1 if violation else -1)
+    with pytest.raises(rc.ReconError):
+        rc.recon_get_work(c, 1)
+    assert rc.lib().ht_faults() == 0
+    rc.lib().ht_device_limit(1 << 40)
+    assert run(many, then_wavefront) == rc.RECON_OK and rc.recon_sync(c) == rc.RECON_OK and done(many)
+    assert len(rc.recon_get_work(c, 3000)) == 3000
+    rc.recon_free(c)
+    assert rc.lib().ht_faults() == 0
+
+
+@pytest.mark.parametrize("n", [1, 4])
+def test_the_wavefront_engine_takes_over_without_scratch(rc, n):
+    c = rc.recon_init(0, 0, rc.RECON_FLAG_SYNC)
+    tiles = [tile(700, 900) for _ in range(n)]
+    rc.lib().ht_device_limit(rc.lib().ht_device_bytes() + (1 << 19))
+    assert rc.recon_batch(c, [t[2] for t in tiles]) == rc.RECON_OK and done(tiles)
+    assert host_runtime.counts(rc)["wavefront"] == 1 and host_runtime.counts(rc)["merging"] == 0
+    assert all(w["scan_rows"] for w in rc.recon_get_work(c, n))
+    rc.lib().ht_device_limit(1 << 40)
+    for t in tiles:
+        t[1][:] = 0
+    assert rc.recon_batch(c, [t[2] for t in tiles]) == rc.RECON_OK and done(tiles)
+    assert host_runtime.counts(rc)["merging"] == 1
+    rc.recon_free(c)
+    assert rc.lib().ht_faults() == 0
