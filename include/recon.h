@@ -144,8 +144,8 @@ int recon_batch_ex(recon_ctx *ctx, const recon_tile *tiles, int n, const int *va
 int recon_run_host(recon_ctx *ctx, const uint8_t *I, uint8_t *J, int H, int W, int conn);
 
 /* End-to-end batch: tiles[].I / tiles[].J are HOST pointers; waits. The J of
- * a FillHoles tile is only written. A batch of 8 Mpx or more is cut into up to
- * four runs of consecutive tiles with about equal pixel counts, processed as
+ * a FillHoles tile is only written. A batch of 8 Mpx or more (256 Mpx on the
+ * wavefront engine) is cut into up to four runs of consecutive tiles with about equal pixel counts, processed as
  * a pipeline: a run's inputs are copied in one run ahead of its use, each run
  * is planned (RECON_FLAG_LEARNED, wavefront engine) while the run before it is reconstructed
  * and then queued behind it, and a run's results are copied back while the

@@ -28,10 +28,13 @@ extern "C" cudaError_t rk_launch_main(int bh, int grid, const rk::Params *P, cud
 extern "C" cudaError_t rk_launch_fill(const rk::TileDesc *tiles, const int *list, int nlist, cudaStream_t st);
 
 constexpr int HOST_SEGMENTS = 4;   // pipeline segments of the end-to-end (host buffer) calls
-// Batches of fewer bytes run as one segment: a segment more costs about 30 us of
-// launches, and hides at most three quarters of the shorter of copies and kernels
-// (24 tiles, 75 Mpx: 1.96 -> 1.69 ms; 8 Mpx copy in and out in about 90 us).
-constexpr size_t HOST_SEGMENT_MIN = (size_t)8 << 20;
+// Batches of fewer bytes run as one segment. On the merging engine a segment more
+// costs about 30 us of launches, and hides at most three quarters of the shorter of
+// copies and kernels (24 tiles, 75 Mpx: 1.96 -> 1.69 ms; 8 Mpx copy in and out in
+// about 90 us). On the wavefront engine it also waits for its own deepest
+// propagation (6 ms on a border-seeded 4096^2 tile, where 256 Mpx take about 5 ms to
+// copy in and out), and a batch in one segment is replayed as a graph.
+constexpr size_t HOST_SEGMENT_MIN = (size_t)8 << 20, HOST_SEGMENT_MIN_WAVEFRONT = (size_t)256 << 20;
 
 struct recon_ctx {
     int device = 0;
@@ -942,7 +945,7 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
         dt[t].pitch = tiles[t].W;
     }
     // segment boundaries: cut when a segment reaches total / HOST_SEGMENTS pixels
-    const int nseg_max = total >= HOST_SEGMENT_MIN ? HOST_SEGMENTS : 1;
+    const int nseg_max = total >= (use_forest(c) ? HOST_SEGMENT_MIN : HOST_SEGMENT_MIN_WAVEFRONT) ? HOST_SEGMENTS : 1;
     std::vector<int> seg_end;
     {
         size_t acc = 0;

@@ -141,3 +141,18 @@ def test_the_wavefront_engine_takes_over_without_scratch(rc, n):
     assert host_runtime.counts(rc)["merging"] == 1
     rc.recon_free(c)
     assert rc.lib().ht_faults() == 0
+
+
+def test_a_host_batch_on_the_wavefront_engine_is_one_launch(rc):
+    """Below 256 Mpx: one launch, replayed as a graph, reported as a whole."""
+    c = rc.recon_init(0, 0, 0)
+    assert rc.recon_set_param(c, rc.RECON_P_REVISIT_SCANS, 1) == rc.RECON_OK
+    tiles = [tile(1800, 1700) for _ in range(4)]
+    for k in (1, 2):
+        assert rc.recon_batch_host(c, [t[2] for t in tiles]) == rc.RECON_OK and done(tiles)
+        assert host_runtime.counts(rc) == dict(merging=0, wavefront=k, graph=k, plan=0)
+        assert [w["scan_rows"] for w in rc.recon_get_work(c, 4)] == [1800] * 4
+        for t in tiles:
+            t[1][:] = 0
+    rc.recon_free(c)
+    assert rc.lib().ht_faults() == 0
