@@ -154,8 +154,9 @@ int recon_run_host(recon_ctx *ctx, const uint8_t *I, uint8_t *J, int H, int W, i
  * copied back; on an error no later run's results are copied back, the call
  * returns once the runs already queued have finished, and
  * recon_last_error_tile (and recon_sync) report the failing tile by its index
- * in `tiles`. recon_get_work and recon_last_kernel_ms describe the last run
- * that was launched. */
+ * in `tiles`. recon_get_work and recon_last_kernel_ms describe the whole batch
+ * (the sum of its runs' times) below 256 Mpx, from there on the last run that
+ * was launched. */
 int recon_batch_host(recon_ctx *ctx, const recon_tile *tiles, int n);
 
 /* Waits for the context's stream; returns the device status of the last call. */

@@ -70,12 +70,16 @@ struct recon_ctx {
     cudaStream_t s_h2d = nullptr, s_d2h = nullptr, s_plan = nullptr;
     cudaEvent_t ev_in[HOST_SEGMENTS] = {}, ev_out[HOST_SEGMENTS] = {};
     rk::Ctl *h_seg_ctl = nullptr;   // pinned: each segment's control word, copied right after its kernel
+    cudaEvent_t ev_seg[HOST_SEGMENTS][2] = {};                // a segment's kernels start and end
+    rk::Work *h_work = nullptr; size_t cap_hwork = 0;         // pinned: all segments' counters
     // last call
     int last_n = 0;
     int launched = 0;
     int last_err_tile = -1;
     int last_abort = 0;
-    int host_status = 0;     // 1: last_err_tile / last_abort hold the last recon_batch_host call's status
+    int host_status = 0;     // 1: last_err_tile / last_abort hold the last call's status
+    int host_whole = 0;      // 1: h_work / host_ms hold the counters and the time of all its segments
+    float host_ms = 0.0f;
     // diagnostics: per-warp progress words in mapped host memory
     unsigned *h_trace = nullptr; unsigned *d_trace = nullptr; size_t cap_trace = 0; int trace_on = 0;
     // graph cache
@@ -130,6 +134,16 @@ static int settle(recon_ctx *c)
     if (st == RECON_ECUDA) return st;
     c->host_status = 1;
     return RECON_OK;
+}
+
+// A call's launches begin: where its status and the counters of its n tiles will be.
+static void begin_call(recon_ctx *c, int n, rk::Ctl *ctl, rk::Work *work)
+{
+    c->last_n = n;
+    c->last_err_tile = -1;
+    c->host_status = c->host_whole = 0;
+    c->last_ctl = ctl;
+    c->last_work = work;
 }
 
 static void drop_graph(recon_ctx *c)
@@ -239,7 +253,11 @@ extern "C" int recon_free(recon_ctx *c)
     if (c->s_h2d) cudaStreamDestroy(c->s_h2d);
     if (c->s_d2h) cudaStreamDestroy(c->s_d2h);
     if (c->s_plan) cudaStreamDestroy(c->s_plan);
+    for (auto &pair : c->ev_seg)
+        for (cudaEvent_t e : pair)
+            if (e) cudaEventDestroy(e);
     if (c->h_seg_ctl) cudaFreeHost(c->h_seg_ctl);
+    if (c->h_work) cudaFreeHost(c->h_work);
     if (c->own_stream) cudaStreamDestroy(c->stream);
     recon_sched_destroy(c->sched);
     delete c;
@@ -580,11 +598,7 @@ static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, int *done)
     if (one) {
         rf::Status *const st = c->d_status + c->status_turn;
         *done = 1;
-        c->last_n = 1;
-        c->last_err_tile = -1;
-        c->host_status = 0;
-        c->last_ctl = &st->ctl;
-        c->last_work = &st->work;
+        begin_call(c, 1, &st->ctl, &st->work);
         rf::Params P = forest_params(c, most, 1, groups[0].flat);
         P.one = forest_tile(tiles[0], 0);
         P.tile_err = &st->tile_err;
@@ -615,11 +629,7 @@ static int forest_batch(recon_ctx *c, const recon_tile *tiles, int n, int *done)
         base[g.count] = acc;
     }
     *done = 1;
-    c->last_n = n;
-    c->last_err_tile = -1;
-    c->host_status = 0;
-    c->last_ctl = (rk::Ctl *)c->d_fmeta;
-    c->last_work = (rk::Work *)(c->d_fmeta + off_work);
+    begin_call(c, n, (rk::Ctl *)c->d_fmeta, (rk::Work *)(c->d_fmeta + off_work));
     CK(cudaMemcpyAsync(c->d_fmeta, h, total, cudaMemcpyHostToDevice, c->stream));
     CK(cudaEventRecord(c->meta_free, c->stream));
     CK(cudaEventRecord(c->ev0, c->stream));
@@ -761,11 +771,7 @@ static int batch_impl(recon_ctx *c, const recon_tile *tiles, int n, const int *v
     memcpy(sig.data() + bytes + sizeof(P), &grid, sizeof(int));
     memcpy(sig.data() + bytes + sizeof(P) + sizeof(int), &c->bh, sizeof(int));
 
-    c->last_n = n;
-    c->last_err_tile = -1;
-    c->host_status = 0;
-    c->last_ctl = c->d_ctl;
-    c->last_work = c->d_work;
+    begin_call(c, n, c->d_ctl, c->d_work);
     const bool use_graph = !(c->flags & RECON_FLAG_NO_GRAPH);
     if (use_graph && c->gexec && sig == c->gsig) {
         // the graph records meta_free itself, right after its descriptor copy
@@ -859,7 +865,8 @@ extern "C" int recon_get_work(recon_ctx *c, recon_work *out, int n)
     CK(cudaStreamSynchronize(c->stream));
     if (n == 0) return RECON_OK;
     std::vector<rk::Work> w(n);
-    CK(cudaMemcpy(w.data(), c->last_work, sizeof(rk::Work) * n, cudaMemcpyDeviceToHost));
+    if (c->host_whole) std::copy(c->h_work, c->h_work + n, w.begin());
+    else CK(cudaMemcpy(w.data(), c->last_work, sizeof(rk::Work) * n, cudaMemcpyDeviceToHost));
     for (int i = 0; i < n; ++i) {
         out[i].visits = w[i].visits;
         out[i].scan_rows = w[i].scan_rows;
@@ -877,7 +884,8 @@ extern "C" int recon_last_kernel_ms(recon_ctx *c, float *ms)
     if (!c || !ms || !c->launched) return RECON_EINVAL;
     CK(cudaSetDevice(c->device));
     CK(cudaStreamSynchronize(c->stream));
-    CK(cudaEventElapsedTime(ms, c->ev0, c->ev1));
+    if (c->host_whole) *ms = c->host_ms;
+    else CK(cudaEventElapsedTime(ms, c->ev0, c->ev1));
     return RECON_OK;
 }
 
@@ -903,6 +911,8 @@ static int ensure_pipeline(recon_ctx *c)
     for (int s = 0; s < HOST_SEGMENTS; ++s) {
         if (!c->ev_in[s]) CK(cudaEventCreateWithFlags(&c->ev_in[s], cudaEventDisableTiming));
         if (!c->ev_out[s]) CK(cudaEventCreateWithFlags(&c->ev_out[s], cudaEventDisableTiming));
+        for (cudaEvent_t &e : c->ev_seg[s])
+            if (!e) CK(cudaEventCreate(&e));
     }
     if (!c->h_seg_ctl) CK(cudaMallocHost((void **)&c->h_seg_ctl, sizeof(rk::Ctl) * HOST_SEGMENTS));
     return RECON_OK;
@@ -956,6 +966,17 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
         }
     }
     const int nseg = (int)seg_end.size();
+    // A batch this small would be one launch on the wavefront engine; cut up, it still reports as one: the counters
+    // of all tiles, the kernel time of all segments, and a violation does not keep the other tiles from running.
+    const bool whole = nseg > 1 && total < HOST_SEGMENT_MIN_WAVEFRONT;
+    if (whole && c->cap_hwork < (size_t)n) {
+        if (c->h_work) cudaFreeHost(c->h_work);
+        c->h_work = nullptr;
+        c->cap_hwork = 0;
+        c->host_whole = c->last_n = 0;   // the call before may have its counters there
+        CK(cudaMallocHost((void **)&c->h_work, sizeof(rk::Work) * (size_t)n));
+        c->cap_hwork = (size_t)n;
+    }
     auto first = [&](int s) { return s ? seg_end[s - 1] : 0; };
     auto queue_inputs = [&](int s) -> int {
         for (int t = first(s); t < seg_end[s]; ++t) {
@@ -968,6 +989,7 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
         return RECON_OK;
     };
     const unsigned fl = c->flags;
+    int ran = 0;   // segments launched
     auto launch = [&](int s) -> int {
         const int t0 = first(s), ns = seg_end[s] - t0;
         std::vector<int> lv, lo;
@@ -980,14 +1002,23 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
             ord = lo.data();
         }
         CK(cudaStreamWaitEvent(c->stream, c->ev_in[s], 0));
+        auto own_events = [&] {
+            std::swap(c->ev0, c->ev_seg[s][0]);
+            std::swap(c->ev1, c->ev_seg[s][1]);
+        };
+        if (whole) own_events();
         const int brc = batch_impl(c, dt.data() + t0, ns, var, ord);
+        if (whole) own_events();
         if (brc != RECON_OK) return brc;
+        ++ran;
+        if (whole)
+            CK(cudaMemcpyAsync(c->h_work + t0, c->last_work, sizeof(rk::Work) * (size_t)ns, cudaMemcpyDeviceToHost, c->stream));
         CK(cudaMemcpyAsync(&c->h_seg_ctl[s], c->last_ctl, sizeof(rk::Ctl), cudaMemcpyDeviceToHost, c->stream));
         CK(cudaEventRecord(c->ev_out[s], c->stream));
         return RECON_OK;
     };
     c->flags = (fl & ~RECON_FLAG_SYNC) | (nseg > 1 ? RECON_FLAG_NO_GRAPH : 0u);
-    int err_tile = -1, abort_code = 0;
+    int err_tile = -1, abort_code = 0, failed = RECON_OK;
     rc = queue_inputs(0);
     if (rc == RECON_OK && nseg > 1) rc = queue_inputs(1);
     if (rc == RECON_OK) rc = launch(0);
@@ -998,13 +1029,14 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
         cudaError_t e = cudaEventSynchronize(c->ev_out[s]);
         if (e != cudaSuccess) { rc = cuda_status(e); break; }
         const rk::Ctl &h = c->h_seg_ctl[s];
-        if (h.abort || h.err_tile != INT_MAX) {   // this segment failed: its results stay on the device
+        // a segment failed: its results and those of the segments behind it stay on the device
+        if ((h.abort || h.err_tile != INT_MAX) && failed == RECON_OK) {
             abort_code = h.abort;
             err_tile = h.err_tile == INT_MAX ? -1 : first(s) + h.err_tile;   // in the caller's indexing
-            rc = h.abort ? RECON_ETIMEOUT : RECON_EMARKER;
-            break;
+            failed = h.abort ? RECON_ETIMEOUT : RECON_EMARKER;
         }
-        for (int t = first(s); t < seg_end[s] && rc == RECON_OK; ++t) {
+        if (failed != RECON_OK && !whole) break;
+        for (int t = first(s); t < seg_end[s] && rc == RECON_OK && failed == RECON_OK; ++t) {
             const recon_tile &T = tiles[t];
             rc = cuda_status(copy_rows(T.J, T.pitch, dt[t].J, T.W, T.W, T.H, cudaMemcpyDeviceToHost, c->s_d2h));
         }
@@ -1015,7 +1047,17 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
     c->last_err_tile = err_tile;
     c->last_abort = abort_code;
     c->host_status = 1;
+    if (whole) {
+        c->last_n = ran == nseg ? n : 0;
+        c->host_ms = 0.0f;
+        for (int s = 0; s < ran; ++s) {
+            float ms = 0.0f;
+            if (cudaEventElapsedTime(&ms, c->ev_seg[s][0], c->ev_seg[s][1]) == cudaSuccess) c->host_ms += ms;
+        }
+        c->host_whole = 1;
+    }
     if (rc != RECON_OK) return rc;
+    if (failed != RECON_OK) return failed;
     if (e0 != cudaSuccess) return cuda_status(e0);
     if (e1 != cudaSuccess) return cuda_status(e1);
     return cuda_status(e2);

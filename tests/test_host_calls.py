@@ -156,3 +156,30 @@ def test_a_host_batch_on_the_wavefront_engine_is_one_launch(rc):
             t[1][:] = 0
     rc.recon_free(c)
     assert rc.lib().ht_faults() == 0
+
+
+@pytest.mark.parametrize("bad", [None, 0, 4])
+def test_a_host_batch_in_segments_reports_as_a_whole(rc, bad):
+    """8 to 256 Mpx on the merging engine: several runs, but the counters are those
+    of all tiles and the time (a nanosecond a pixel here) that of all runs, also
+    when a tile is refused."""
+    c = rc.recon_init(0, 0, 0)
+    tiles = [tile(64 * (20 + k), 1700) for k in range(5)]
+    for rep in range(2):
+        if bad is not None:
+            tiles[bad][1][5, 6] = 10
+        want = rc.RECON_OK if bad is None else rc.RECON_EMARKER
+        assert rc.recon_batch_host(c, [t[2] for t in tiles]) == want
+        assert rc.recon_last_error_tile(c) == (-1 if bad is None else bad) and rc.recon_sync(c) == want
+        assert [w["visits"] for w in rc.recon_get_work(c, 5)] == [27 * (20 + k) for k in range(5)]
+        px = sum(I.size for k, (I, _, _) in enumerate(tiles) if k != bad)
+        assert rc.recon_last_kernel_ms(c) == pytest.approx(1e-6 * px, rel=1e-5)
+        assert host_runtime.counts(rc)["merging"] == 4 * (rep + 1)
+        for _, J, _ in tiles:
+            J[:] = 0
+    small = tile(70, 70)   # the next call's own figures
+    assert rc.recon_batch(c, [small[2]]) == rc.RECON_OK and rc.recon_sync(c) == rc.RECON_OK
+    assert [w["visits"] for w in rc.recon_get_work(c, 1)] == [4]
+    assert rc.recon_last_kernel_ms(c) == pytest.approx(1e-6 * 4900, rel=1e-2)
+    rc.recon_free(c)
+    assert rc.lib().ht_faults() == 0
