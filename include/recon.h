@@ -151,9 +151,10 @@ int recon_run_host(recon_ctx *ctx, const uint8_t *I, uint8_t *J, int H, int W, i
  * and then queued behind it, and a run's results are copied back while the
  * next run is reconstructed (copies from pinned host memory overlap the
  * reconstruction). Each run's device status is checked before its results are
- * copied back; on an error no later run's results are copied back, the call
- * returns once the runs already queued have finished, and
- * recon_last_error_tile (and recon_sync) report the failing tile by its index
+ * copied back; on an error no later run's results are copied back, and below
+ * 256 Mpx none of any run (there, results that can be refused are copied back
+ * once all runs have passed). The call returns once the runs already queued
+ * have finished, and recon_last_error_tile (and recon_sync) report the failing tile by its index
  * in `tiles`. recon_get_work and recon_last_kernel_ms describe the whole batch
  * (the sum of its runs' times) below 256 Mpx, from there on the last run that
  * was launched. */

@@ -989,6 +989,17 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
         return RECON_OK;
     };
     const unsigned fl = c->flags;
+    // ... and a violation in any tile leaves every J of the caller's as it was: no result goes back before all
+    // segments are through, unless none can be refused.
+    bool hold = false;
+    for (int t = 0; t < n; ++t) hold |= whole && tiles[t].op != RECON_OP_FILL_HOLES && !(fl & RECON_FLAG_NO_CHECK);
+    auto queue_results = [&](int s) -> int {
+        for (int t = first(s); t < seg_end[s]; ++t) {
+            const recon_tile &T = tiles[t];
+            CK(copy_rows(T.J, T.pitch, dt[t].J, T.W, T.W, T.H, cudaMemcpyDeviceToHost, c->s_d2h));
+        }
+        return RECON_OK;
+    };
     int ran = 0;   // segments launched
     auto launch = [&](int s) -> int {
         const int t0 = first(s), ns = seg_end[s] - t0;
@@ -1036,11 +1047,9 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
             failed = h.abort ? RECON_ETIMEOUT : RECON_EMARKER;
         }
         if (failed != RECON_OK && !whole) break;
-        for (int t = first(s); t < seg_end[s] && rc == RECON_OK && failed == RECON_OK; ++t) {
-            const recon_tile &T = tiles[t];
-            rc = cuda_status(copy_rows(T.J, T.pitch, dt[t].J, T.W, T.W, T.H, cudaMemcpyDeviceToHost, c->s_d2h));
-        }
+        if (!hold && failed == RECON_OK) rc = queue_results(s);
     }
+    for (int s = 0; hold && s < nseg && rc == RECON_OK && failed == RECON_OK; ++s) rc = queue_results(s);
     c->flags = fl;
     const cudaError_t e0 = cudaStreamSynchronize(c->stream);
     const cudaError_t e1 = cudaStreamSynchronize(c->s_h2d), e2 = cudaStreamSynchronize(c->s_d2h);

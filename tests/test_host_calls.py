@@ -183,3 +183,23 @@ def test_a_host_batch_in_segments_reports_as_a_whole(rc, bad):
     assert rc.recon_last_kernel_ms(c) == pytest.approx(1e-6 * 4900, rel=1e-2)
     rc.recon_free(c)
     assert rc.lib().ht_faults() == 0
+
+
+@pytest.mark.parametrize("op", ["RECON_OP_DILATE", "RECON_OP_FILL_HOLES"])
+@pytest.mark.parametrize("bad", [0, 4])
+def test_a_refused_host_batch_changes_nothing(rc, op, bad):
+    """The markers are as they were when any tile is refused (a FillHoles tile's J is
+    output only; in a batch with others it is left alone too)."""
+    c = rc.recon_init(0, 0, 0)
+    tiles = [tile(1300 + k, 1700) for k in range(5)]
+    tiles[bad][1][5, 6] = 10
+    desc = [t[2] + (rc.RECON_OP_DILATE if k == bad else getattr(rc, op),) for k, t in enumerate(tiles)]
+    before = [J.copy() for _, J, _ in tiles]
+    for _ in range(2):
+        assert rc.recon_batch_host(c, desc) == rc.RECON_EMARKER and rc.recon_last_error_tile(c) == bad
+        assert all((J == b).all() for (_, J, _), b in zip(tiles, before))
+    tiles[bad][1][5, 6] = 0
+    assert rc.recon_batch_host(c, desc) == rc.RECON_OK and done(tiles)
+    assert host_runtime.counts(rc)["merging"] == 12
+    rc.recon_free(c)
+    assert rc.lib().ht_faults() == 0
