@@ -19,8 +19,9 @@
  * the length of the propagation path, and it has no schedule. recon_run*,
  * recon_batch* and the host-buffer calls use the merging engine while all of
  * the context's wavefront settings (BLOCK_H, SWEEPS, GRID, BANDS, TMA,
- * REVISIT_SCANS, SCAN_GAIN, TEST_STALL, TRACE) hold their defaults, and the
- * wavefront engine otherwise, as recon_batch_ex with a variant or an order does.
+ * REVISIT_SCANS, SCAN_GAIN, TEST_STALL, TRACE) are left at their defaults, and
+ * the wavefront engine when one was set to another value (recon_set_param, the
+ * environment), as recon_batch_ex with a variant or an order does.
  *
  * Two more operations run on the same engine (recon_tile.op):
  *   reconstruction by erosion, the dual: R = lim_n eps_I^n(J),
@@ -258,11 +259,12 @@ int recon_last_kernel_ms(recon_ctx *ctx, float *ms);
  * calls that overlap on the GPU race: issue them one at a time. */
 int recon_run_noalloc(const uint8_t *I, uint8_t *J, int H, int W, int conn, void *cuda_stream);
 
-/* Autotuner: times every candidate block height {32, 64, 128} x bands
- * {2, 4} x first-visit scan pairs {0, 1, 2} x adaptive scan gain {0, 2048} on
- * this batch (each `reps` times after one warm-up run, J restored from a
- * device backup before every run), installs the fastest in the context and
- * writes it to best[4] = {block height, bands, scan pairs, scan gain}. J
+/* Autotuner of the wavefront engine: times every candidate block height {32, 64,
+ * 128} x bands {2, 4} x first-visit scan pairs {0, 1, 2} x adaptive scan gain
+ * {0, 2048} there on this batch (each `reps` times after one warm-up run, J restored from a
+ * device backup before every run), installs the fastest in the context, for
+ * the calls that run on that engine (it does not change which engine a call runs
+ * on, neither from trials nor from the cache), and writes it to best[4] = {block height, bands, scan pairs, scan gain}. J
  * holds its original marker on return. The paper tunes its scan-to-queue
  * switch point the same way (Sec. V-C). */
 int recon_autotune(recon_ctx *ctx, const recon_tile *tiles, int n, int reps, int *best);

@@ -46,6 +46,9 @@ struct recon_ctx {
     // defaults: 128-row blocks, one scan pair on a first visit, then more pairs
     // while a pair still raises >= 2048 pixels (first visits and revisits)
     int bh = 128, k = 1, grid = 0, bands = 4, order_policy = 1, phantom = 0, use_tma = 1, revisit_scans = 0, scan_gain = 2048;
+    // the four that the autotuner sets too, as the caller asked for them: these choose the engine (use_forest)
+    int ask_bh = 128, ask_k = 1, ask_bands = 4, ask_gain = 2048;
+    bool tuning = false;   // inside the autotuner's trials
     long long wait_ns = 2000000000ll;
     // device scratch
     unsigned char *d_meta = nullptr; size_t cap_meta = 0;      // descriptors + order tables
@@ -292,16 +295,16 @@ extern "C" int recon_set_param(recon_ctx *c, int key, int64_t v)
     switch (key) {
     case RECON_P_BLOCK_H:
         if (v != 32 && v != 64 && v != 128 && v != 256) return RECON_EINVAL;
-        c->bh = (int)v; break;
+        c->bh = c->ask_bh = (int)v; break;
     case RECON_P_SWEEPS:
         if (v < -1 || v > 64) return RECON_EINVAL;
-        c->k = (int)v; break;
+        c->k = c->ask_k = (int)v; break;
     case RECON_P_GRID:
         if (v < 0 || v > (1 << 20)) return RECON_EINVAL;
         c->grid = (int)v; break;
     case RECON_P_BANDS:
         if (v != 1 && v != 2 && v != 4) return RECON_EINVAL;
-        c->bands = (int)v; break;
+        c->bands = c->ask_bands = (int)v; break;
     case RECON_P_WAIT_NS:
         if (v < 1000 || v > 600000000000ll) return RECON_EINVAL;
         c->wait_ns = v; break;
@@ -322,7 +325,7 @@ extern "C" int recon_set_param(recon_ctx *c, int key, int64_t v)
         c->revisit_scans = (int)v; break;
     case RECON_P_SCAN_GAIN:
         if (v < 0 || v > (1 << 20)) return RECON_EINVAL;
-        c->scan_gain = (int)v; break;
+        c->scan_gain = c->ask_gain = (int)v; break;
     default: return RECON_EINVAL;
     }
     drop_graph(c);
@@ -500,16 +503,17 @@ static int stage_meta(recon_ctx *c, const recon_tile *tiles, int n, const int *v
 }
 
 // Whether a call without an explicit schedule runs on the region-merging
-// engine: when the context's wavefront settings are all at their defaults.
-// Setting any of them (recon_set_param, RECON_*, recon_autotune) or passing
-// variants or an order asks for the wavefront engine. The merging engine was
+// engine: when the caller left the context's wavefront settings at their defaults.
+// Setting any of them (recon_set_param, RECON_*) or passing variants or an order
+// asks for the wavefront engine. recon_autotune does not: its trials run on that
+// engine and what it installs applies there, but a call stays where it was. The merging engine was
 // faster at every size, marker, connectivity and operation measured, by 2
 // (4096^2, h-dome: 403 -> 204 us) to 26 times (holes filled: 2.67 -> 0.104 ms),
 // so there is no size below or above which the other is chosen.
 static bool use_forest(const recon_ctx *c)
 {
-    return c->bh == 128 && c->k == 1 && c->grid == 0 && c->bands == 4 && c->use_tma == 1 && c->revisit_scans == 0 &&
-           c->scan_gain == 2048 && !c->phantom && !c->trace_on;
+    return c->ask_bh == 128 && c->ask_k == 1 && c->grid == 0 && c->ask_bands == 4 && c->use_tma == 1 &&
+           c->revisit_scans == 0 && c->ask_gain == 2048 && !c->phantom && !c->trace_on && !c->tuning;
 }
 
 static rf::Tile forest_tile(const recon_tile &T, int index)
@@ -1254,8 +1258,8 @@ extern "C" int recon_sched_plan_batch(recon_ctx *c, const recon_tile *tiles, int
 
 // ---------------------------------------------------------------------------
 // autotuner: times candidate (block height, bands, first-visit scan pairs) on
-// the caller's batch and keeps the fastest. Results never differ (R is unique),
-// only the time does.
+// the caller's batch on the wavefront engine and keeps the fastest. Results never
+// differ (R is unique), only the time does.
 
 // The autotuner's cache key of a batch: size bucket = round(log2(mean tile
 // area)), the set of connectivities (bit 0: 4, bit 1: 8), and the marker
@@ -1349,6 +1353,7 @@ extern "C" int recon_autotune(recon_ctx *c, const recon_tile *tiles, int n, int 
     const int save_bh = c->bh, save_bands = c->bands, save_k = c->k, save_gain = c->scan_gain;
     const unsigned save_flags = c->flags;
     c->flags &= ~RECON_FLAG_SYNC;
+    c->tuning = true;
     float best_ms = 1e30f;
     int bb[4] = {save_bh, save_bands, save_k, save_gain};
     int rc = RECON_OK;
@@ -1382,6 +1387,7 @@ extern "C" int recon_autotune(recon_ctx *c, const recon_tile *tiles, int n, int 
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     cudaFree(bk);
     c->flags = save_flags;
+    c->tuning = false;
     drop_graph(c);
     if (rc != RECON_OK || e != cudaSuccess) {
         c->bh = save_bh; c->bands = save_bands; c->k = save_k; c->scan_gain = save_gain;

@@ -203,3 +203,33 @@ def test_a_refused_host_batch_changes_nothing(rc, op, bad):
     assert host_runtime.counts(rc)["merging"] == 12
     rc.recon_free(c)
     assert rc.lib().ht_faults() == 0
+
+
+def test_the_autotuner_tunes_the_wavefront_engine_and_moves_no_call(rc):
+    """Every trial runs on the wavefront engine; what it installs, from trials or from
+    a cache, applies there, and a call on default settings stays where it was."""
+    c, c2 = rc.recon_init(0, 0, rc.RECON_FLAG_SYNC), rc.recon_init(0, 0, rc.RECON_FLAG_SYNC)
+    t = tile(70, 80)
+
+    def installed(ctx):
+        return tuple(rc.recon_get_param(ctx, k) for k in (rc.RECON_P_BLOCK_H, rc.RECON_P_BANDS, rc.RECON_P_SWEEPS,
+                                                          rc.RECON_P_SCAN_GAIN))
+
+    def engine(ctx):
+        before = host_runtime.counts(rc)
+        t[1][:] = 0
+        assert rc.recon_batch(ctx, [t[2]]) == rc.RECON_OK and done([t])
+        return [k for k in ("merging", "wavefront") if host_runtime.counts(rc)[k] > before[k]]
+    st, best = rc.recon_autotune(c, [t[2]], 1)
+    assert st == rc.RECON_OK and not t[1].any() and best == installed(c) != (128, 4, 1, 2048)
+    assert host_runtime.counts(rc)["merging"] == 0 and host_runtime.counts(rc)["wavefront"] == 2 * 36
+    assert engine(c) == ["merging"]
+    assert rc.recon_autotune_cache_load(c2, rc.recon_autotune_cache(c)[1]) == rc.RECON_OK
+    t[1][:] = 0
+    assert rc.recon_autotune(c2, [t[2]], 1) == (rc.RECON_OK, best) and installed(c2) == best
+    assert engine(c2) == ["merging"]
+    assert rc.recon_set_param(c2, rc.RECON_P_REVISIT_SCANS, 1) == rc.RECON_OK and engine(c2) == ["wavefront"]
+    assert installed(c2) == best
+    rc.recon_free(c)
+    rc.recon_free(c2)
+    assert rc.lib().ht_faults() == 0
