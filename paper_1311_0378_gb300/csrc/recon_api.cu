@@ -92,6 +92,7 @@ struct recon_ctx {
     recon_sched *sched = nullptr;
     // distance transform scratch
     unsigned char *d_dt = nullptr; size_t cap_dt = 0;
+    unsigned dt_call = ~0u;   // number of the last call on it (~0: its header needs clearing)
     // training scratch (moments, epoch losses, two epochs' sample orders)
     unsigned char *d_train = nullptr; size_t cap_train = 0;
     int *h_order = nullptr; size_t cap_order = 0;   // pinned: the orders as the host shuffles them
@@ -1438,8 +1439,14 @@ extern "C" int recon_dt(recon_ctx *c, const uint8_t *B, uint32_t *d2, int32_t *s
         CK(cudaStreamSynchronize(c->stream));
         const int rc = grow(&c->d_dt, &c->cap_dt, need);
         if (rc) return rc;
+        c->dt_call = ~0u;
     }
-    if (dt_run(B, H, W, (int *)site, (unsigned *)d2, c->d_dt, c->sms, c->stream) != DT_OK) return RECON_ECUDA;
+    if (c->dt_call == ~0u) {   // new scratch, or the numbers start again
+        CK(cudaMemsetAsync(c->d_dt, 0, DT_HEADER, c->stream));
+        c->dt_call = 0;
+    }
+    ++c->dt_call;
+    if (dt_run(B, H, W, (int *)site, (unsigned *)d2, c->d_dt, c->dt_call, c->sms, c->stream) != DT_OK) return RECON_ECUDA;
     CK(cudaStreamSynchronize(c->stream));
     return RECON_OK;
 }

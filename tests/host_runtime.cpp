@@ -345,7 +345,7 @@ cudaError_t rl_train_epoch(float *, float *, float *, const float *, const float
     return cudaSuccess;
 }
 size_t dt_scratch_bytes(int H, int W) { return (size_t)H * W; }
-int dt_run(const uint8_t *, int, int, int *, unsigned *, void *, int, cudaStream_t) { return DT_OK; }
+int dt_run(const uint8_t *, int, int, int *, unsigned *, void *, unsigned, int, cudaStream_t) { return DT_OK; }
 
 // ---- entry points of the other files
 extern "C" int recon_run_noalloc(const uint8_t *, uint8_t *, int, int, int, void *) { return RECON_ECUDA; }
