@@ -219,7 +219,7 @@ __device__ __forceinline__ void load_row(const uint16_t *row, int W, int pitch, 
         }
         if (x < pitch) {
             q[x] = v;
-            if (SITE) gs[x] = (uint16_t)raw;
+            if (SITE && x < W) gs[x] = (uint16_t)raw;
         }
         const uint32_t mn = __reduce_min_sync(0xFFFFFFFFu, v);
         if ((threadIdx.x & 31) == 0) low[x >> 5] = mn;
