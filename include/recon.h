@@ -349,13 +349,16 @@ int recon_sched_plan_batch(recon_ctx *ctx, const recon_tile *tiles, int n, int *
                            float *pred);
 
 /* Bounds-checked build (librecon_checks.so, built with RECON_CHECKS): the
- * reconstruction kernel checks every wavefront queue slot and pixel offset
- * before using it, counts failed checks and skips those accesses instead of
+ * reconstruction kernels of both engines and the distance transform's check the
+ * places they compute -- queue slots and pixel offsets of the wavefront; labels,
+ * basin numbers, list places, node slots and node numbers of the merging engine;
+ * column words, column distances and row columns of the distance transform --
+ * before using them, count failed checks and skip those accesses instead of
  * making them (the stand-in for a memory checker). recon_checks reports
  * *enabled (1 in that build, 0 otherwise), the number of failed checks since
- * the last reset and the where-code of the first (1: queue slot, 2: wavefront
- * pixel, 3: pushed pixel); reset != 0 clears them. Returns 0, or nonzero on
- * bad arguments or a CUDA error. */
+ * the last reset and the where-code of a first one (csrc/recon_check.h);
+ * reset != 0 clears them. Returns 0, or nonzero on bad arguments or a CUDA
+ * error. */
 int recon_checks(int *enabled, unsigned *violations, unsigned *first, int reset);
 
 /* ---- distance transform (Table II) ----

@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "recon_check.h"
 #include "recon_dt.h"
 
 namespace dt {
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(128) mask_kernel(const uint8_t *B, int H, int 
     } else {
 #pragma unroll
         for (int b = 0; b < 4; ++b)
-            if (x + b < W) o[b] = m[b];
+            if (x + b < W && RK_CHECK(blockIdx.y < gridDim.y && 32 * (int)blockIdx.y < H, CK_WORD)) o[b] = m[b];
     }
 }
 
@@ -133,6 +134,9 @@ __global__ void __launch_bounds__(128) column_kernel(const uint32_t *M, int H, i
     const uint32_t m[2] = {M[(size_t)s * W + x], M[(size_t)s * W + xb]};
     if (LONG && !m[0] && empty_strip(some, call, G + x, y0, min(H, y0 + 32), pitch)) return;
     uint32_t up, dn;   // distances from the row before / after the strip
+    auto word = [&](int t, int c) {
+        return RK_CHECK(t >= 0 && t < ns && c < W, CK_WORD) ? M[(size_t)t * W + c] : 0u;
+    };
     {
         uint32_t u[2] = {FAR, FAR}, d[2] = {FAR, FAR};
         // a strip whose first (last) row is background needs no look above (below)
@@ -141,8 +145,8 @@ __global__ void __launch_bounds__(128) column_kernel(const uint32_t *M, int H, i
             uint32_t a[8], b[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                a[k] = more0 && t - k >= 0 ? M[(size_t)(t - k) * W + x] : 0u;
-                b[k] = more1 && t - k >= 0 ? M[(size_t)(t - k) * W + xb] : 0u;
+                a[k] = more0 && t - k >= 0 ? word(t - k, x) : 0u;
+                b[k] = more1 && t - k >= 0 ? word(t - k, xb) : 0u;
             }
 #pragma unroll
             for (int k = 7; k >= 0; --k) {
@@ -156,8 +160,8 @@ __global__ void __launch_bounds__(128) column_kernel(const uint32_t *M, int H, i
             uint32_t a[8], b[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                a[k] = more0 && t + k < ns ? M[(size_t)(t + k) * W + x] : 0u;
-                b[k] = more1 && t + k < ns ? M[(size_t)(t + k) * W + xb] : 0u;
+                a[k] = more0 && t + k < ns ? word(t + k, x) : 0u;
+                b[k] = more1 && t + k < ns ? word(t + k, xb) : 0u;
             }
 #pragma unroll
             for (int k = 7; k >= 0; --k) {
@@ -198,7 +202,7 @@ __global__ void __launch_bounds__(128) column_kernel(const uint32_t *M, int H, i
                 }
                 v = w;
             }
-            *(uint32_t *)(o + (size_t)r * pitch) = v;
+            if (RK_CHECK(y0 + r < H && x + 1 < pitch, CK_COLUMN)) *(uint32_t *)(o + (size_t)r * pitch) = v;
         }
     }
 }
@@ -217,7 +221,7 @@ __device__ __forceinline__ void load_row(const uint16_t *row, int W, int pitch, 
         } else {
             v = raw - FAR <= 32u ? INF : g * g;
         }
-        if (x < pitch) {
+        if (x < pitch && RK_CHECK(x < W + PAD + 2, CK_ROW)) {
             q[x] = v;
             if (SITE && x < W) gs[x] = (uint16_t)raw;
         }
@@ -275,6 +279,7 @@ __global__ void row_kernel(const uint16_t *G, int H, int W, int pitch, unsigned 
                 if ((j - 1) * (j - 1) >= max((int)b0, (int)b1)) break;   // (at once for EMPTY: both are negative)
 #pragma unroll
                 for (int k = 0; k < 4; k += 2) {
+                    if (!RK_CHECK(x - j - k >= -PAD && x + j + k + 1 < W + PAD + 2, CK_ROW)) continue;
                     const uint2 l = *(const uint2 *)&q[x - j - k], r = *(const uint2 *)&q[x + j + k];
                     const uint32_t s0 = (uint32_t)((j + k - 1) * (j + k - 1)), s1 = (uint32_t)((j + k) * (j + k)),
                                    s2 = (uint32_t)((j + k + 1) * (j + k + 1));
@@ -285,9 +290,9 @@ __global__ void row_kernel(const uint16_t *G, int H, int W, int pitch, unsigned 
                 }
             }
             if (j > PAD) {
-                search_far(x, W, low, [&](int c, uint32_t d) { b0 = min(b0, q[c] + d); }, [&](uint32_t d) { return d >= b0; });
+                search_far(x, W, low, [&](int c, uint32_t d) { if (RK_CHECK(c >= 0 && c < W, CK_ROW)) b0 = min(b0, q[c] + d); }, [&](uint32_t d) { return d >= b0; });
                 if (x + 1 < W)
-                    search_far(x + 1, W, low, [&](int c, uint32_t d) { b1 = min(b1, q[c] + d); },
+                    search_far(x + 1, W, low, [&](int c, uint32_t d) { if (RK_CHECK(c >= 0 && c < W, CK_ROW)) b1 = min(b1, q[c] + d); },
                                [&](uint32_t d) { return d >= b1; });
             }
             unsigned *o = d2 + (size_t)y * W + x;
@@ -317,6 +322,7 @@ __global__ void row_site_kernel(const uint16_t *G, int H, int W, int pitch, unsi
         load_row<true>(G + (size_t)y * pitch, W, pitch, y, q, low, gs);
         __syncthreads();
         auto site_of = [&](int c) {
+            if (!RK_CHECK(c >= 0 && c < W, CK_ROW)) return 0;
             const int g = gs[c];
             return (y + (g & 0x8000 ? -(g & 0x7FFF) : g)) * W + c;
         };
@@ -324,6 +330,7 @@ __global__ void row_site_kernel(const uint16_t *G, int H, int W, int pitch, unsi
             uint32_t best = q[x];
             int bs = best >= INF ? 0x7FFFFFFF : site_of(x);
             auto take = [&](int c, uint32_t d) {
+                if (!RK_CHECK(c >= -PAD && c < W + PAD + 2, CK_ROW)) return;
                 const uint32_t v = q[c] + d;
                 if (v > best || v >= INF) return;
                 const int s = site_of(c);
@@ -347,6 +354,8 @@ __global__ void row_site_kernel(const uint16_t *G, int H, int W, int pitch, unsi
 }
 
 }  // namespace dt
+
+RK_CHECK_READER(dt_read_checks)
 
 static size_t mask_bytes(int H, int W) { return (((size_t)((H + 31) / 32) * W * sizeof(uint32_t)) + 255) / 256 * 256; }
 static int g_pitch(int W) { return (W + 1) / 2 * 2; }

@@ -43,6 +43,7 @@
 // dense made the difference.
 #include <climits>
 #include <cstddef>
+#include "recon_check.h"
 #include "recon_forest.h"
 
 namespace rf {
@@ -310,8 +311,11 @@ struct SharedLinks {
     static constexpr unsigned SOURCE = RES;
     uint32_t *link;
     unsigned base;
-    __device__ uint32_t load(unsigned n) const { return *(volatile uint32_t *)&link[n]; }
-    __device__ bool cas(unsigned n, uint32_t o, uint32_t v) const { return atomicCAS(&link[n], o, v) == o; }
+    __device__ uint32_t load(unsigned n) const { return RK_CHECK(n < RES, CK_SLOT) ? *(volatile uint32_t *)&link[n] : (uint32_t)RES; }
+    __device__ bool cas(unsigned n, uint32_t o, uint32_t v) const
+    {
+        return RK_CHECK(n < RES, CK_SLOT) ? atomicCAS(&link[n], o, v) == o : true;
+    }
     __device__ unsigned weight(uint32_t l) const { return l >> 8; }
     __device__ unsigned parent(uint32_t l) const { return l & 255u; }
     __device__ uint32_t word(unsigned w, unsigned p) const { return w << 8 | p; }
@@ -322,10 +326,14 @@ struct GlobalLinks {
     typedef unsigned long long Word;
     static constexpr unsigned SOURCE = SRC;
     unsigned long long *link;
-    __device__ unsigned long long load(unsigned n) const { return *(volatile unsigned long long *)&link[n]; }
+    unsigned nodes;   // node numbers are below this
+    __device__ unsigned long long load(unsigned n) const
+    {
+        return RK_CHECK(n < nodes, CK_NODE) ? *(volatile unsigned long long *)&link[n] : (unsigned long long)SRC;
+    }
     __device__ bool cas(unsigned n, unsigned long long o, unsigned long long v) const
     {
-        return atomicCAS(&link[n], o, v) == o;
+        return RK_CHECK(n < nodes, CK_NODE) ? atomicCAS(&link[n], o, v) == o : true;
     }
     __device__ unsigned weight(unsigned long long l) const { return (unsigned)(l >> 32); }
     __device__ unsigned parent(unsigned long long l) const { return (unsigned)l; }
@@ -526,6 +534,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
         for (; tops; ++id) {
             const unsigned k = 31 - __clz(tops), b = k >> 3, h = ~k & 7u;
             tops ^= 1u << k;
+            if (!RK_CHECK(id < (unsigned)Smem<CONN>::NB && cell + (int)(h * ST + b) < NCELL, CK_BASIN)) continue;
             S.L[cell + (int)(h * ST + b)] = (uint16_t)(ROOT | id);
             S.sv[id] = j0[h * BS + b];                       // the top's own source edge
         }
@@ -537,7 +546,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
             for (uint32_t bits = fits ? rest[h] : 0u; bits; ++slot) {
                 const unsigned k = 31 - __clz(bits);
                 bits ^= 1u << k;
-                S.tab[slot] = 8u * (unsigned)(cell + h * ST) + k;
+                if (RK_CHECK(slot < (unsigned)TAB, CK_PASS)) S.tab[slot] = 8u * (unsigned)(cell + h * ST) + k;
             }
         }
     }
@@ -555,6 +564,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     {
         const unsigned L = (unsigned)__cvta_generic_to_shared(S.L);
         auto label = [&](unsigned at) {
+            if (!RK_CHECK(at < 2u * NCELL && !(at & 1u), CK_LABEL)) return ROOT;
             unsigned short v;
             asm volatile("ld.volatile.shared.u16 %0, [%1];" : "=h"(v) : "r"(L + at) : "memory");
             return (unsigned)v;
@@ -594,7 +604,8 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
             if (jw == 0u) continue;
 #pragma unroll
             for (int b = 0; b < 4; ++b)
-                over |= (((jw >> (8 * b)) & 255u) > S.sv[l[4 * i + b] - ROOT] ? 1u : 0u) << (4 * i + b);
+                if (RK_CHECK(l[4 * i + b] - ROOT < nb, CK_BASIN))
+                    over |= (((jw >> (8 * b)) & 255u) > S.sv[l[4 * i + b] - ROOT] ? 1u : 0u) << (4 * i + b);
         }
 #pragma unroll 1
         for (; over; over &= over - 1) {
@@ -608,7 +619,9 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     // Maxima are taken without a look at the present one first: on the 910 Mpx
     // batch the load and the compare cost more than the reductions they saved
     // (9.39 -> 8.84 ms of kernel time).
-    auto offer = [&](unsigned a, uint32_t key) { atomicMax(&S.best[a], key); };
+    auto offer = [&](unsigned a, uint32_t key) {
+        if (RK_CHECK(a < nb, CK_BASIN)) atomicMax(&S.best[a], key);
+    };
     // Passes join a saddle's own basin to the one the arc starts in. A pass no
     // heavier than the source edges of both ends is never taken. The first
     // round's maxima are taken here too.
@@ -620,7 +633,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     unsigned mine = listed ? (ne * (warp + 1)) / (NT / 32) - seg0 : 0u;   // the warp's passes
     auto close_up = [&](unsigned &to, uint32_t e) {   // keeps nonzero e; returns its place (warp-wide)
         const unsigned keep = __ballot_sync(FULL, e != 0u), at = to + __popc(keep & ((1u << lane) - 1u));
-        if (e) S.tab[at] = e;
+        if (e && RK_CHECK(at < (unsigned)TAB, CK_PASS)) S.tab[at] = e;
         to += __popc(keep);
         return at;
     };
@@ -629,10 +642,11 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
 #pragma unroll 1
         for (unsigned k = 0; k < mine; k += 32) {
             uint32_t n = 0u;
-            if (k + lane < mine) {
+            if (k + lane < mine &&
+                RK_CHECK(seg0 + k + lane < (unsigned)TAB && S.tab[seg0 + k + lane] >> 3 < (unsigned)NCELL, CK_PASS)) {
                 const uint32_t e = S.tab[seg0 + k + lane], p = e >> 3, w = ((const uint8_t *)bi)[p];
                 const unsigned a = S.L[p] & 0x7FFFu, b = S.L[(int)p + ring_off(e & 7u)] & 0x7FFFu;
-                if (a != b && (w > S.sv[a] || w > S.sv[b])) n = a << 20 | b << 8 | w;
+                if (RK_CHECK(a < nb && b < nb, CK_BASIN) && a != b && (w > S.sv[a] || w > S.sv[b])) n = a << 20 | b << 8 | w;
             }
             const unsigned at = close_up(to, n);
             if (n) {
@@ -690,7 +704,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
 #pragma unroll 1
                 for (unsigned k = 0; k < mine; k += 32) {
                     uint32_t n = 0u;
-                    if (k + lane < mine) {
+                    if (k + lane < mine && RK_CHECK(seg0 + k + lane < (unsigned)TAB, CK_PASS)) {
                         const uint32_t e = S.tab[seg0 + k + lane];
                         const unsigned a = S.comp[e >> 20], b = S.comp[(e >> 8) & 0xFFFu];
                         if (a != b) n = a << 20 | b << 8 | (e & 255u);
@@ -724,6 +738,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
 #pragma unroll 1
         for (unsigned k = tid; k < nlive; k += NT) {
             const unsigned b = rounds ? now[k] : k + 1;
+            if (!RK_CHECK(b < nb, CK_BASIN)) continue;
             const uint32_t key = S.best[b], src = S.sv[b] << 24 | K_SOURCE;
             if (src > key) {
                 S.capw[b] = (uint8_t)(src >> 24);
@@ -732,12 +747,14 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
             }
             if (!(key & K_EDGE)) {
                 S.capw[b] = (uint8_t)atomicAdd(&S.nt, 1u);
+                (void)RK_CHECK(S.capw[b] < RES, CK_SLOT);
                 *(volatile uint32_t *)&S.best[b] = NODE;
                 continue;
             }
             const unsigned i = key & 0x3FFFFFu;
             unsigned t, t2;
             if (listed) {
+                if (!RK_CHECK(i < (unsigned)TAB, CK_PASS)) continue;
                 const uint32_t e = S.tab[i];
                 t = e >> 20;
                 t2 = (e >> 8) & 0xFFFu;
@@ -747,6 +764,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
                 t2 = S.comp[S.L[p + dir_off(4u + (i & 3u))] & 0x7FFFu];
             }
             if (t == b) t = t2;
+            if (!RK_CHECK(t < nb, CK_BASIN)) continue;
             // both ends chose this edge: the lower number stays
             if (b < t && *(volatile uint32_t *)&S.best[t] == key && (S.sv[t] << 24 | K_SOURCE) < key) continue;
             S.up[b] = (uint16_t)t;
@@ -765,7 +783,8 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
                 atomicMax(&S.sv[t], S.sv[b]);
             } else if (S.best[b] < FINAL) {
                 S.best[b] = 0u;
-                next[atomicAdd(&S.nlive[rounds & 1], 1u)] = (uint16_t)b;
+                const unsigned at = atomicAdd(&S.nlive[rounds & 1], 1u);
+                if (RK_CHECK(at < (unsigned)Smem<CONN>::NB / (rounds & 1 ? 4 : 2), CK_LIVE)) next[at] = (uint16_t)b;
             }
         }
         __syncthreads();
@@ -794,7 +813,7 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
             w = min(w, min(fa >> 8, fb >> 8));
             if (na == nb2 || w == 0) return 0u;
             if (na != RES && nb2 != RES) return na << 16 | nb2 << 8 | w;   // between two nodes
-            atomicMax(&S.link[na == RES ? nb2 : na], w << 8 | RES);
+            if (RK_CHECK((na == RES ? nb2 : na) < nt, CK_SLOT)) atomicMax(&S.link[na == RES ? nb2 : na], w << 8 | RES);
             return 0u;
         };
         // (best and sv, next to each other, are no longer needed: room for every pass)
@@ -804,7 +823,9 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
 #pragma unroll 1
             for (unsigned k = lane; k < mine; k += 32) {
                 const uint32_t e = S.tab[seg0 + k], z = ends(e >> 20, (e >> 8) & 0xFFFu, e & 255u);
-                if (z) joins[atomicAdd(&S.nj, 1u)] = z;   // gathered, so that whole warps join
+                if (!z) continue;
+                const unsigned at = atomicAdd(&S.nj, 1u);   // gathered, so that whole warps join
+                if (RK_CHECK(at < (unsigned)TAB, CK_PASS)) joins[at] = z;
             }
         } else {
             each_pair(S, [&](unsigned a, unsigned b, unsigned w, unsigned) { ends(a, b, w); });
@@ -854,6 +875,8 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
 #pragma unroll
             for (int j = 0; j < 4; ++j) {   // pixels 8h + 2j, 8h + 2j + 1
                 const uint32_t i2 = iw[2 * h + (j >> 1)] >> (16 * (j & 1));
+                o[4 * h + j] = RES | RES << 16;
+                if (!RK_CHECK((w[j] & 0x7FFFu) < nb && (w[j] >> 16 & 0x7FFFu) < nb, CK_BASIN)) continue;
                 const uint32_t e0 = S.comp[w[j] & 0x7FFFu], e1 = S.comp[(w[j] >> 16) & 0x7FFFu];
                 o[4 * h + j] = (min(e0 >> 8, i2 & 255u) << 8 | (e0 & 255u)) |
                                (min(e1 >> 8, (i2 >> 8) & 255u) << 8 | (e1 & 255u)) << 16;
@@ -932,6 +955,7 @@ __global__ void __launch_bounds__(128) rim_kernel(const __grid_constant__ Params
             nb = blk + 1 + B.nbx;
             at = 0;
         }
+        there = there && RK_CHECK(nb < P.nblocks, CK_NODE);
         const unsigned qv = there ? P.rim[(size_t)nb * 4 * BS + at] : RES;
         qn[d] = (qv & 255u) == RES ? SRC : nb * MAX_TERM + (qv & 255u);
         w[d] = min(pv >> 8, qv >> 8);
@@ -948,7 +972,7 @@ __global__ void __launch_bounds__(128) rim_kernel(const __grid_constant__ Params
                 w[d] = 0;
             }
     }
-    GlobalLinks F{P.link};
+    GlobalLinks F{P.link, P.nblocks * MAX_TERM};
     bool ok = true;
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
@@ -985,7 +1009,7 @@ __global__ void __launch_bounds__(NT) value_kernel(const __grid_constant__ Param
     if (threadIdx.x < nt) {
         unsigned n = blk * MAX_TERM + threadIdx.x, v = 255;
         int it = 0;
-        for (; it < MAX_STEPS; ++it) {
+        for (; it < MAX_STEPS && RK_CHECK(n < P.nblocks * MAX_TERM, CK_NODE); ++it) {
             const unsigned long long l = __ldcg(&P.link[n]);
             v = min(v, (unsigned)(l >> 32));
             n = (unsigned)l;
@@ -1016,6 +1040,8 @@ __global__ void __launch_bounds__(NT) value_kernel(const __grid_constant__ Param
 }
 
 }  // namespace rf
+
+RK_CHECK_READER(rf_read_checks)
 
 extern "C" cudaError_t rf_configure()
 {

@@ -29,30 +29,12 @@
 // halo before it lets go. Every device-side wait is bounded.
 #include <climits>
 #include <cuda_runtime.h>
+#include "recon_check.h"
 #include "recon_internal.h"
 
 namespace rk {
 
 constexpr unsigned FULL = 0xFFFFFFFFu;
-
-// Bounds-checked build (-DRECON_CHECKS, librecon_checks.so): the stand-in for
-// a memory checker. Every queue slot and every wavefront pixel offset is
-// checked before it is used; a failed check is counted, its where-code kept
-// (1: queue slot, 2: wavefront pixel offset, 3: pushed pixel offset), and the
-// access is skipped instead of made. Read back with recon_checks().
-#ifdef RECON_CHECKS
-__device__ unsigned g_check_violations;
-__device__ unsigned g_check_first;
-__device__ __noinline__ bool check_fail(unsigned where)
-{
-    atomicAdd(&g_check_violations, 1u);
-    atomicCAS(&g_check_first, 0u, where);
-    return false;
-}
-#define RK_CHECK(cond, where) ((cond) ? true : check_fail(where))
-#else
-#define RK_CHECK(cond, where) true
-#endif
 
 __device__ __forceinline__ unsigned long long gtimer()
 {
@@ -652,7 +634,7 @@ template <int BH>
 __device__ __forceinline__ void put_entry(Smem<BH> &S, uint16_t *gsp, int lvl, unsigned slot, uint16_t v)
 {
     if (!RK_CHECK(v >= (unsigned)(PW * 4) && v < (unsigned)((BH + 1) * PW * 4) &&
-                  (unsigned)(v % (PW * 4) - XOFF) < (unsigned)BW, 3))
+                  (unsigned)(v % (PW * 4) - XOFF) < (unsigned)BW, CK_PUSHED_PIXEL))
         return;
     if (slot < (unsigned)QCAP) S.q[lvl][slot] = v;
     else if (slot - QCAP < (unsigned)GCAP) gsp[lvl * GCAP + (slot - QCAP)] = v;
@@ -662,7 +644,7 @@ __device__ __forceinline__ void put_entry(Smem<BH> &S, uint16_t *gsp, int lvl, u
 template <int BH>
 __device__ __forceinline__ uint16_t get_entry(const Smem<BH> &S, const uint16_t *gsp, int lvl, unsigned i)
 {
-    if (!RK_CHECK(i < (unsigned)(QCAP + GCAP), 1)) return (uint16_t)(PW * 4 + XOFF);
+    if (!RK_CHECK(i < (unsigned)(QCAP + GCAP), CK_QUEUE_SLOT)) return (uint16_t)(PW * 4 + XOFF);
     return i < (unsigned)QCAP ? S.q[lvl][i] : gsp[lvl * GCAP + (i - QCAP)];
 }
 
@@ -858,7 +840,7 @@ __device__ __forceinline__ unsigned expand(Smem<BH> &S, unsigned *claim, unsigne
 #ifdef RECON_CHECKS
     // an interior pixel of the block: rows 1 .. BH of J, columns XOFF .. XOFF + BW - 1
     if (act && !RK_CHECK(p >= (unsigned)RB && p < (unsigned)((BH + 1) * RB) && (unsigned)(p % RB - XOFF) < (unsigned)BW,
-                         2)) {
+                         CK_WAVEFRONT_PIXEL)) {
         act = false;
         p = RB + XOFF;
     }
@@ -1499,6 +1481,8 @@ extern "C" cudaError_t rk_launch_init(int grid, const rk::Params *P, cudaStream_
     return cudaGetLastError();
 }
 
+RK_CHECK_READER(rk_read_checks)
+
 // Bounds-checked build only: *enabled = 1, the number of failed checks since
 // the last reset and the where-code of the first. Other builds: *enabled = 0.
 extern "C" int recon_checks(int *enabled, unsigned *violations, unsigned *first, int reset)
@@ -1506,14 +1490,12 @@ extern "C" int recon_checks(int *enabled, unsigned *violations, unsigned *first,
     if (!enabled || !violations || !first) return 1;
 #ifdef RECON_CHECKS
     *enabled = 1;
-    if (cudaMemcpyFromSymbol(violations, rk::g_check_violations, sizeof(unsigned)) != cudaSuccess ||
-        cudaMemcpyFromSymbol(first, rk::g_check_first, sizeof(unsigned)) != cudaSuccess)
-        return 4;
-    if (reset) {
-        const unsigned z = 0;
-        if (cudaMemcpyToSymbol(rk::g_check_violations, &z, sizeof(z)) != cudaSuccess ||
-            cudaMemcpyToSymbol(rk::g_check_first, &z, sizeof(z)) != cudaSuccess)
-            return 4;
+    *violations = *first = 0;
+    for (check_reader read : {rk_read_checks, rf_read_checks, dt_read_checks}) {
+        unsigned v = 0, f = 0;
+        if (read(&v, &f, reset) != cudaSuccess) return 4;
+        if (v && !*violations) *first = f;
+        *violations += v;
     }
 #else
     *enabled = 0;
