@@ -233,3 +233,25 @@ def test_the_autotuner_tunes_the_wavefront_engine_and_moves_no_call(rc):
     rc.recon_free(c)
     rc.recon_free(c2)
     assert rc.lib().ht_faults() == 0
+
+
+def test_the_learned_schedule_is_planned_where_the_wavefront_engine_runs(rc):
+    """Once a batch in recon_batch, once a segment in a host batch; never for the
+    merging engine, which has no schedule."""
+    c = rc.recon_init(0, 0, rc.RECON_FLAG_SYNC | rc.RECON_FLAG_LEARNED)
+    assert rc.recon_sched_set_model(c, [0.0] * rc.RECON_MLP_NPARAMS, [0, 1, 0, 1], 1, 2) == rc.RECON_OK
+    small = [tile(40, 50) for _ in range(3)]
+    large = [tile(8192, 8256) for _ in range(4)]   # 271 Mpx: four segments on either engine
+    plans = []
+    for setting in (0, 1):
+        assert rc.recon_set_param(c, rc.RECON_P_REVISIT_SCANS, setting) == rc.RECON_OK
+        for run, tiles in ((rc.recon_batch, small), (rc.recon_batch_host, large)):
+            for t in tiles:
+                t[1][:] = 0
+            before = host_runtime.counts(rc)
+            assert run(c, [t[2] for t in tiles]) == rc.RECON_OK and done(tiles)
+            now = host_runtime.counts(rc)
+            plans.append(tuple(now[k] - before[k] for k in ("merging", "wavefront", "plan")))
+    assert plans == [(1, 0, 0), (4, 0, 0), (0, 1, 1), (0, 4, 4)]
+    rc.recon_free(c)
+    assert rc.lib().ht_faults() == 0
