@@ -1159,7 +1159,8 @@ static int ensure_orders(recon_ctx *c, size_t n)
     return RECON_OK;
 }
 
-// Epochs epoch0 .. epoch0 + epochs - 1 of mini-batch Adam, one launch each. The
+// Epochs epoch0 .. epoch0 + epochs - 1 of mini-batch Adam, one launch each, or two a
+// step where the device cannot place that launch's cluster. The
 // host shuffles the next epoch while one runs: two orders take turns, each refilled
 // once the copy out of it, queued behind the epoch before, is done.
 // adam_mv NULL: moments in the context's scratch, starting at zero.
@@ -1169,15 +1170,18 @@ static int train_epochs(recon_ctx *c, float *theta, float *adam_mv, int *step, i
     CK(cudaSetDevice(c->device));
     CK(cudaStreamSynchronize(c->stream));
     const size_t off_loss = align_up(sizeof(float) * 2 * MLP_NPARAMS, 16);
-    const size_t off_idx = align_up(off_loss + sizeof(float) * (size_t)epochs, 16);
+    const size_t off_grad = align_up(off_loss + sizeof(float) * (size_t)epochs, 16);
+    const size_t off_idx = align_up(off_grad + sizeof(float) * MLP_NPARAMS, 16);
     int rc = grow(&c->d_train, &c->cap_train, off_idx + sizeof(int) * 2 * (size_t)n);
     if (rc == RECON_OK) rc = ensure_orders(c, (size_t)n);
     if (rc) return rc;
     float *mv = adam_mv ? adam_mv : (float *)c->d_train, *dl = (float *)(c->d_train + off_loss);
+    float *grad = (float *)(c->d_train + off_grad);
     int *didx = (int *)(c->d_train + off_idx);
-    // the scratch moments and the epoch losses lie next to each other
-    cudaError_t e = adam_mv ? cudaMemsetAsync(dl, 0, sizeof(float) * (size_t)epochs, c->stream)
-                            : cudaMemsetAsync(c->d_train, 0, off_idx, c->stream);
+    // the scratch moments, the epoch losses and the gradient lie next to each other
+    const size_t zero_from = adam_mv ? off_loss : 0;
+    cudaError_t e = cudaMemsetAsync(c->d_train + zero_from, 0, off_idx - zero_from, c->stream);
+    const bool fits = rl_train_fits();
     batch = std::min(batch, n);
     int t = *step;
     const int nbatches = (n - 1) / batch + 1;
@@ -1195,9 +1199,14 @@ static int train_epochs(recon_ctx *c, float *theta, float *adam_mv, int *step, i
             std::swap(perm[i], perm[j]);
         }
         e = cudaMemcpyAsync(buf, perm, sizeof(int) * n, cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaEventRecord(c->order_free[k & 1], c->stream);
-        if (e == cudaSuccess)
+        if (e == cudaSuccess && k + 2 < epochs) e = cudaEventRecord(c->order_free[k & 1], c->stream);
+        if (e == cudaSuccess && fits)
             e = rl_train_epoch(theta, mv, mv + MLP_NPARAMS, X, T, buf, n, batch, t, lr, dl + k, c->stream);
+        for (int s = 0; !fits && s < nbatches && e == cudaSuccess; ++s) {
+            const size_t at = (size_t)s * batch;
+            e = rl_grad(theta, X, T, buf + at, (int)std::min<size_t>(batch, n - at), grad, dl + k, c->stream);
+            if (e == cudaSuccess) e = rl_adam(theta, grad, mv, mv + MLP_NPARAMS, t + s + 1, lr, c->stream);
+        }
         t += nbatches;
     }
     if (e == cudaSuccess && epoch_loss) {

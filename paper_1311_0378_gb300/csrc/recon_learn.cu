@@ -284,17 +284,16 @@ __global__ void adam_kernel(float *theta, float *grad, float *m, float *v, int t
 // sample at a time, with 32-way bank conflicts in the 64 x 64 layer (a thread per
 // row of stride 64); here the rows are 65 apart, a thread works on one unit of
 // four samples, and the next samples are on their way while these are worked on.
-// An epoch of 16 steps takes 216 us a call, 2473 with those launches.
-// Sixteen CTAs of 256 threads where the device can place them (a cluster that
-// large is not portable), otherwise eight of 512 (262 us; 32 samples a chunk).
+// An epoch of 16 steps takes 216 us a call, 2473 with those launches (which remain
+// for a device that cannot place sixteen CTAs together: rl_train_fits).
 namespace cg = cooperative_groups;
 constexpr int S1 = D0 + 1, S2 = D1 + 1;           // weight row strides: odd, so that a column has no bank conflicts
 constexpr int PW1 = 0, PB1 = PW1 + D1 * S1, PW2 = PB1 + D1, PB2 = PW2 + D2 * S2, PW3 = PB2 + D2,
               PB3 = PW3 + D3 * D2, PPAD = (PB3 + D3 + 3) / 4 * 4;
 
-template <int CL>
+constexpr int CL = 16;                             // CTAs (a cluster of more than eight is not portable)
+constexpr int TT = 256, TS = 16;                   // threads; samples at a time: four a unit and thread group
 struct TrainSmem {
-    static constexpr int TT = 4096 / CL, TS = 256 / CL;   // threads; samples at a time: four a unit and thread group
     float P[PPAD];                                 // weights, padded rows
     float G[(NP + 3) / 4 * 4];                     // this CTA's gradient, flat layout
     alignas(16) float a1[TS][D1], a2[TS][D2], dz1[TS][D1], dz2[TS][D2];
@@ -312,20 +311,17 @@ __device__ __forceinline__ int padded(int i)       // flat parameter index -> pl
 }
 static_assert(PW3 - PB2 == OW3 - OB2 && PB3 - PB2 == OB3 - OB2, "layout");
 
-template <int CL>
-__global__ void __launch_bounds__(TrainSmem<CL>::TT) train_kernel(float *theta, float *m, float *v, const float *X,
-                                                                  const float *T, const int *idx, int n, int batch,
-                                                                  int step0, float lr, float b1, float b2, float eps,
-                                                                  float *loss)
+__global__ void __launch_bounds__(TT) train_kernel(float *theta, float *m, float *v, const float *X, const float *T,
+                                                   const int *idx, int n, int batch, int step0, float lr, float b1,
+                                                   float b2, float eps, float *loss)
 {
-    typedef TrainSmem<CL> Sm;
-    constexpr int TT = Sm::TT, TS = Sm::TS, NG = TT / 64;   // NG thread groups, 4 samples each
+    constexpr int NG = TT / 64;                             // thread groups, 4 samples each
     constexpr int OWN = (NP + CL - 1) / CL, OPT = (OWN + TT - 1) / TT;   // parameters a CTA (a thread) updates
-    constexpr int RW = D2 / NG, IW = (D0 + NG - 1) / NG;    // W2 rows, inputs of W1 whose gradients a thread adds up
+    constexpr int RW = D2 / NG, IW = D0 / NG;               // W2 rows, inputs of W1 whose gradients a thread adds up
     constexpr int NF = (TS * (D0 + D3) + TT - 1) / TT;      // inputs and targets a thread fetches
-    static_assert(TS == 4 * NG, "four samples a group");
+    static_assert(TS == 4 * NG && D0 % NG == 0 && D2 % NG == 0, "four samples a group, whole rows and columns");
     extern __shared__ __align__(16) unsigned char train_smem[];
-    Sm &S = *reinterpret_cast<Sm *>(train_smem);
+    TrainSmem &S = *reinterpret_cast<TrainSmem *>(train_smem);
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank(), tid = threadIdx.x;
     const int j = tid & 63, g = tid >> 6;
@@ -465,8 +461,7 @@ __global__ void __launch_bounds__(TrainSmem<CL>::TT) train_kernel(float *theta, 
                     gw2[q + 3] = fmaf(d.w, a, gw2[q + 3]);
                 }
 #pragma unroll
-                for (int q = 0; q < IW; ++q)
-                    if (g + q * NG < D0) gw1[q] = fmaf(d1, S.x[s][g + q * NG], gw1[q]);
+                for (int q = 0; q < IW; ++q) gw1[q] = fmaf(d1, S.x[s][g + q * NG], gw1[q]);
                 if (g == 0) gb1 += d1;
                 else if (g == 1) gb2 += S.dz2[s][j];
                 if (g >= NG - 2) gw3 = fmaf(S.dy[s][g - (NG - 2)], S.a2[s][j], gw3);
@@ -477,8 +472,7 @@ __global__ void __launch_bounds__(TrainSmem<CL>::TT) train_kernel(float *theta, 
 #pragma unroll
         for (int q = 0; q < RW; ++q) S.G[OW2 + (RW * g + q) * D1 + j] = gw2[q];
 #pragma unroll
-        for (int q = 0; q < IW; ++q)
-            if (g + q * NG < D0) S.G[OW1 + j * D0 + g + q * NG] = gw1[q];
+        for (int q = 0; q < IW; ++q) S.G[OW1 + j * D0 + g + q * NG] = gw1[q];
         if (g == 0) S.G[OB1 + j] = gb1;
         else if (g == 1) S.G[OB2 + j] = gb2;
         if (g >= NG - 2) S.G[OW3 + (g - (NG - 2)) * D2 + j] = gw3;
@@ -600,41 +594,40 @@ cudaError_t rl_adam(float *theta, float *grad, float *m, float *v, int t, float 
     return cudaGetLastError();
 }
 
-template <int CL>
-static cudaError_t train_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr, cudaStream_t st)
+static cudaLaunchConfig_t train_config(cudaLaunchAttribute *attr, cudaStream_t st)
 {
-    typedef rl::TrainSmem<CL> Sm;
-    cudaError_t e = cudaFuncSetAttribute(rl::train_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sm));
-    if (e == cudaSuccess && CL > 8)
-        e = cudaFuncSetAttribute(rl::train_kernel<CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    *cfg = cudaLaunchConfig_t{};
     attr->id = cudaLaunchAttributeClusterDimension;
-    attr->val.clusterDim.x = CL;
+    attr->val.clusterDim.x = rl::CL;
     attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
-    cfg->gridDim = dim3(CL);
-    cfg->blockDim = dim3(Sm::TT);
-    cfg->dynamicSmemBytes = sizeof(Sm);
-    cfg->stream = st;
-    cfg->attrs = attr;
-    cfg->numAttrs = 1;
-    return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(rl::CL);
+    cfg.blockDim = dim3(rl::TT);
+    cfg.dynamicSmemBytes = sizeof(rl::TrainSmem);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+bool rl_train_fits()
+{
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = train_config(&attr, nullptr);
+    int clusters = 0;
+    cudaError_t e = cudaFuncSetAttribute(rl::train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(rl::TrainSmem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(rl::train_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, rl::train_kernel, &cfg);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && clusters > 0;
 }
 
 cudaError_t rl_train_epoch(float *theta, float *m, float *v, const float *X, const float *T, const int *idx, int n,
                            int batch, int step0, float lr, float *loss, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
-    int clusters = 0;
-    cudaError_t e = train_config<16>(&cfg, &attr, st);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, rl::train_kernel<16>, &cfg);
-    if (e == cudaSuccess && clusters > 0)
-        return cudaLaunchKernelEx(&cfg, rl::train_kernel<16>, theta, m, v, X, T, idx, n, batch, step0, lr, 0.9f, 0.999f,
-                                  1e-8f, loss);
-    cudaGetLastError();   // this device cannot place sixteen CTAs together
-    e = train_config<8>(&cfg, &attr, st);
-    if (e != cudaSuccess) return e;
-    return cudaLaunchKernelEx(&cfg, rl::train_kernel<8>, theta, m, v, X, T, idx, n, batch, step0, lr, 0.9f, 0.999f, 1e-8f,
+    const cudaLaunchConfig_t cfg = train_config(&attr, st);
+    return cudaLaunchKernelEx(&cfg, rl::train_kernel, theta, m, v, X, T, idx, n, batch, step0, lr, 0.9f, 0.999f, 1e-8f,
                               loss);
 }

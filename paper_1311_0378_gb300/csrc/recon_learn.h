@@ -21,6 +21,9 @@ cudaError_t rl_forward(const float *theta, const float *X, int n, float *Y, cuda
 cudaError_t rl_grad(const float *theta, const float *X, const float *T, const int *idx, int nb, float *grad,
                     float *loss, cudaStream_t st);
 cudaError_t rl_adam(float *theta, float *grad, float *m, float *v, int t, float lr, cudaStream_t st);
+// Whether the current device can place rl_train_epoch's cluster of sixteen CTAs (and
+// prepares it for that: asked before the first epoch).
+bool rl_train_fits();
 // Adam over the mini-batches idx[0 .. batch), idx[batch .. 2 batch), ... of one
 // epoch (n samples), steps step0 + 1, ...; *loss gets the sum of the batch losses.
 cudaError_t rl_train_epoch(float *theta, float *m, float *v, const float *X, const float *T, const int *idx, int n,

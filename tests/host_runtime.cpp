@@ -42,7 +42,8 @@ int faults = 0;
 int broken = 0;                          // waits for a stream under capture
 double now_ms = 0.0;                     // device clock: a kernel takes a nanosecond a pixel
 int n_merging = 0, n_wavefront = 0, n_graph = 0, n_plan = 0;
-std::vector<int> orders;                 // sample orders of the epochs trained
+std::vector<int> orders, steps;          // sample orders of the epochs trained; numbers of the single steps
+bool fits = true;                        // the training cluster can be placed
 
 void run_to(size_t n)
 {
@@ -140,7 +141,12 @@ extern "C" int ht_orders(int *out, int max)
     memcpy(out, orders.data(), sizeof(int) * std::min<size_t>(max, orders.size()));
     return (int)orders.size();
 }
-extern "C" void *ht_pinned(size_t bytes) { return alloc(bytes); }
+extern "C" int ht_steps(int *out, int max)
+{
+    memcpy(out, steps.data(), sizeof(int) * std::min<size_t>(max, steps.size()));
+    return (int)steps.size();
+}
+extern "C" void ht_train_fits(int yes) { fits = yes; }
 
 // ---- runtime
 extern "C" {
@@ -329,11 +335,27 @@ cudaError_t rl_forward(const float *, const float *, int n, float *Y, cudaStream
     put(st, [=] { memset(Y, 0, sizeof(float) * 2 * n); });
     return cudaSuccess;
 }
-cudaError_t rl_grad(const float *, const float *, const float *, const int *, int, float *, float *, cudaStream_t)
+cudaError_t rl_grad(const float *, const float *, const float *, const int *idx, int n, float *grad, float *loss,
+                    cudaStream_t st)
 {
+    put(st, [=] {
+        touch(idx, sizeof(int) * n);
+        orders.insert(orders.end(), idx, idx + n);
+        grad[0] += 1.0f;
+        *loss += 1.0f;
+    });
     return cudaSuccess;
 }
-cudaError_t rl_adam(float *, float *, float *, float *, int, float, cudaStream_t) { return cudaSuccess; }
+cudaError_t rl_adam(float *, float *grad, float *, float *, int t, float, cudaStream_t st)
+{
+    put(st, [=] {
+        faults += grad[0] != 1.0f;
+        grad[0] = 0.0f;
+        steps.push_back(t);
+    });
+    return cudaSuccess;
+}
+bool rl_train_fits() { return fits; }
 cudaError_t rl_train_epoch(float *, float *, float *, const float *, const float *, const int *idx, int n, int, int,
                            float, float *loss, cudaStream_t st)
 {

@@ -255,3 +255,25 @@ def test_the_learned_schedule_is_planned_where_the_wavefront_engine_runs(rc):
     assert plans == [(1, 0, 0), (4, 0, 0), (0, 1, 1), (0, 4, 4)]
     rc.recon_free(c)
     assert rc.lib().ht_faults() == 0
+
+
+@pytest.mark.parametrize("n,batch", [(5, 2), (64, 64), (10, 100)])
+def test_training_without_the_cluster_takes_the_same_steps(rc, n, batch):
+    """A device that cannot place sixteen CTAs together: gradient and Adam launches, the
+    same samples in the same order, the steps numbered on."""
+    rc.lib().ht_train_fits(0)
+    c = rc.recon_init(0, 0, rc.RECON_FLAG_SYNC)
+    a = np.zeros(3 * rc.RECON_MLP_NPARAMS, np.float32)
+    X = np.zeros((n, 22), np.float32)
+    per = -(-n // batch)
+    st, losses = rc.recon_mlp_train(c, a.ctypes.data, X.ctypes.data, X.ctypes.data, n, 3, batch, 1e-3, 5)
+    assert st == rc.RECON_OK and losses == [1.0] * 3
+    st, step, _ = rc.recon_mlp_train_resume(c, a.ctypes.data, a.ctypes.data, 3 * per, 3, X.ctypes.data, X.ctypes.data,
+                                            n, 1, batch, 1e-3, 5)
+    assert st == rc.RECON_OK and step == 4 * per
+    got, steps = (ctypes.c_int * (4 * n))(), (ctypes.c_int * (4 * per))()
+    assert rc.lib().ht_orders(got, 4 * n) == 4 * n and rc.lib().ht_steps(steps, 4 * per) == 4 * per
+    assert list(got) == [i for e in range(4) for i in order(n, 5, e)]
+    assert list(steps) == list(range(1, 4 * per + 1))
+    rc.recon_free(c)
+    assert rc.lib().ht_faults() == 0
