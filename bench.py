@@ -21,8 +21,9 @@ the workload's masks: objects I >= 100 and the space between them).
 The line's "compare" block (skip it with --no-compare) times the wavefront
 engine on the same batch: its plain schedule, the per-tile launch loop, the
 learned schedule with and without its planning pass, and the sweep-only and
-queue-first halves of the method with their own rooflines. "cpu_baseline" is the CPU oracle on a bounded sample of
-the workload, on all host cores and on one core. --microbench runs the
+queue-first halves of the method with their own rooflines. "cpu_baseline" is
+the CPU oracle on a bounded sample of the workload, on all host cores and on
+one core. --microbench runs the
 random-access and atomic micro-benchmarks instead; --tile T reconstructs one
 tile alone (a small fixed case for profilers); --subset n keeps every n-th
 tile; --impl reference times the CPU oracle on the same workload (the
@@ -98,15 +99,16 @@ def measured_traffic(workload):
     return w.get("dram_bytes_per_launch") if w else None
 
 
-def merging_launches(rc, ctx, tiles):
-    """Kernel launches of a batch on the region-merging engine, or None when the
-    context's settings ask for the wavefront engine. Tiles of one connectivity
-    form groups of up to 65536 blocks of 64 x 64; a group takes three launches
-    (one when every tile of it is a single block)."""
-    want = ((rc.RECON_P_BLOCK_H, 128), (rc.RECON_P_BANDS, 4), (rc.RECON_P_SWEEPS, 1),
-            (rc.RECON_P_TMA, 1), (rc.RECON_P_REVISIT_SCANS, 0), (rc.RECON_P_SCAN_GAIN, 2048))
-    if os.environ.get("RECON_GRID") or any(rc.recon_get_param(ctx, p) != v for p, v in want):
-        return None
+def ran_merging(work):
+    """Whether the call with these work counters (recon_get_work) ran on the
+    region-merging engine: only the wavefront engine fetches blocks from a work list."""
+    return all(w["phase_ns"]["fetch"] == 0 for w in work)
+
+
+def merging_launches(tiles):
+    """Kernel launches of a batch on the region-merging engine: tiles of one
+    connectivity form groups of up to 65536 blocks of 64 x 64; a group takes three
+    launches (one when every tile of it is a single block)."""
     n = 0
     for conn in (8, 4):
         left, flat = 0, True
@@ -122,6 +124,17 @@ def merging_launches(rc, ctx, tiles):
         if left:
             n += 1 if flat else 3
     return n
+
+
+def schedule_config(merging, settings, schedule, model_meta, tuned):
+    """The line's description of what ran: the region-merging engine has no schedule,
+    and no wavefront setting or cost model touches it."""
+    if merging:
+        return {"engine": "region merging", "schedule": None, "cost_model": None, "autotuned": False,
+                **dict.fromkeys(settings)}
+    return {"engine": "wavefront", "schedule": schedule, **settings, "autotuned": tuned is not None,
+            "cost_model": ({"tiles": model_meta.get("tiles"), "variants": model_meta.get("variants")}
+                           if model_meta else None)}
 
 
 def peaks():
@@ -742,15 +755,12 @@ def main():
     if args.autotune:
         st, tuned = rc.recon_autotune(ctx, desc, 2)
         rc.check(st, "recon_autotune")
-    params = {"block_h": rc.recon_get_param(ctx, rc.RECON_P_BLOCK_H),
-              "bands": rc.recon_get_param(ctx, rc.RECON_P_BANDS),
-              "scan_pairs": rc.recon_get_param(ctx, rc.RECON_P_SWEEPS),
-              "grid": rc.recon_get_param(ctx, rc.RECON_P_GRID), "autotuned": tuned is not None,
-              "schedule": args.schedule,
-              "cost_model": ({"tiles": model_meta.get("tiles"), "variants": model_meta.get("variants")}
-                             if model_meta else None)}
-    merging = merging_launches(rc, ctx, tiles)
-    params["engine"] = "wavefront" if merging is None else "region merging"
+        for key, val in zip((rc.RECON_P_BLOCK_H, rc.RECON_P_BANDS, rc.RECON_P_SWEEPS, rc.RECON_P_SCAN_GAIN), tuned):
+            rc.check(rc.recon_set_param(ctx, key, val))   # asks for the wavefront engine, unless they are the defaults
+    settings = {"block_h": rc.recon_get_param(ctx, rc.RECON_P_BLOCK_H),
+                "bands": rc.recon_get_param(ctx, rc.RECON_P_BANDS),
+                "scan_pairs": rc.recon_get_param(ctx, rc.RECON_P_SWEEPS),
+                "grid": rc.recon_get_param(ctx, rc.RECON_P_GRID)}
     px = sum(t.H * t.W for t in tiles)          # this rank's pixels per step
     job_px = sum(t.H * t.W for t in job)        # every rank's pixels per step
     flush = torch.empty(512 << 20, dtype=torch.uint8, device=dev)
@@ -767,6 +777,8 @@ def main():
     for _ in range(max(args.warmup, 3)):
         step()
     rc.check(rc.recon_sync(ctx), "warmup")
+    merging = ran_merging(rc.recon_get_work(ctx, len(desc)))
+    params = schedule_config(merging, settings, args.schedule, model_meta, tuned)
 
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
     kern_ms = []
@@ -836,14 +848,14 @@ def main():
     alg = ALG_BYTES_PER_PX[args.op]
     achieved = alg * px / (kms / 1e3) / 1e9
     traffic_key = w.name if args.op == "dilate" else "%s:%s" % (w.name, args.op)
-    traffic = measured_traffic(traffic_key) if args.subset == 1 and world == 1 and merging is not None else None
+    traffic = measured_traffic(traffic_key) if args.subset == 1 and world == 1 and merging else None
     roof = {"bound": "hbm", "achieved": round(achieved, 2), "peak": pk["hbm_gbs"], "unit": "GB/s",
             "frac": round(achieved / pk["hbm_gbs"], 5), "traffic": traffic,
-            "kernel": "recon_persistent" if merging is None else "block_kernel, rim_kernel, value_kernel",
+            "kernel": "block_kernel, rim_kernel, value_kernel" if merging else "recon_persistent",
             "kernel_ms": round(kms, 4),
             "alg_bytes_per_px": alg, "alg_bytes_per_launch": alg * px, "peak_source": src,
-            "limiter": ("propagation depth and shared-memory latency of thin wavefronts (not DRAM)" if merging is None
-                        else "instruction issue and shared-memory latency of block_kernel (not DRAM)")}
+            "limiter": ("instruction issue and shared-memory latency of block_kernel (not DRAM)" if merging
+                        else "propagation depth and shared-memory latency of thin wavefronts (not DRAM)")}
     if traffic:
         roof["dram_GBps"] = round(traffic / (kms / 1e3) / 1e9, 2)
         roof["dram_frac"] = round(traffic / (kms / 1e3) / 1e9 / pk["hbm_gbs"], 5)
@@ -863,7 +875,7 @@ def main():
         "e2e": {"value": round(e2e, 2), "unit": "Mpix/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
         # per step: the groups' launches, or init + persistent kernel, plus features, finalize
         # and MLP forward when learned, plus the marker kernel for FillHoles
-        "gpu_launches": (((5 if learned else 2) + (0 if reset_j else 1)) if merging is None else merging) * args.steps,
+        "gpu_launches": (merging_launches(tiles) if merging else (5 if learned else 2) + (0 if reset_j else 1)) * args.steps,
         "compare": compare,
         "clocks": clk.summary(),
     }
