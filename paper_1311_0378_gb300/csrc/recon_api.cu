@@ -72,16 +72,17 @@ struct recon_ctx {
     uint8_t *d_img = nullptr; size_t cap_img = 0;
     cudaStream_t s_h2d = nullptr, s_d2h = nullptr, s_plan = nullptr;
     cudaEvent_t ev_in[HOST_SEGMENTS] = {}, ev_out[HOST_SEGMENTS] = {};
-    rk::Ctl *h_seg_ctl = nullptr;   // pinned: each segment's control word, copied right after its kernel
-    cudaEvent_t ev_seg[HOST_SEGMENTS][2] = {};                // a segment's kernels start and end
-    rk::Work *h_work = nullptr; size_t cap_hwork = 0;         // pinned: all segments' counters
+    unsigned char *h_seg = nullptr; size_t cap_hseg = 0;   // pinned: each segment's control word (and counters), copied
+                                                           // right after its kernels
+    cudaEvent_t ev_seg[HOST_SEGMENTS][2] = {};             // a segment's kernels start and end
     // last call
     int last_n = 0;
     int launched = 0;
     int last_err_tile = -1;
     int last_abort = 0;
     int host_status = 0;     // 1: last_err_tile / last_abort hold the last call's status
-    int host_whole = 0;      // 1: h_work / host_ms hold the counters and the time of all its segments
+    int host_whole = 0;      // 1: host_work / host_ms hold the counters and the time of all its segments
+    std::vector<rk::Work> host_work;
     float host_ms = 0.0f;
     // diagnostics: per-warp progress words in mapped host memory
     unsigned *h_trace = nullptr; unsigned *d_trace = nullptr; size_t cap_trace = 0; int trace_on = 0;
@@ -260,8 +261,7 @@ extern "C" int recon_free(recon_ctx *c)
     for (auto &pair : c->ev_seg)
         for (cudaEvent_t e : pair)
             if (e) cudaEventDestroy(e);
-    if (c->h_seg_ctl) cudaFreeHost(c->h_seg_ctl);
-    if (c->h_work) cudaFreeHost(c->h_work);
+    if (c->h_seg) cudaFreeHost(c->h_seg);
     if (c->own_stream) cudaStreamDestroy(c->stream);
     recon_sched_destroy(c->sched);
     delete c;
@@ -507,10 +507,13 @@ static int stage_meta(recon_ctx *c, const recon_tile *tiles, int n, const int *v
 // engine: when the caller left the context's wavefront settings at their defaults.
 // Setting any of them (recon_set_param, RECON_*) or passing variants or an order
 // asks for the wavefront engine. recon_autotune does not: its trials run on that
-// engine and what it installs applies there, but a call stays where it was. The merging engine was
-// faster at every size, marker, connectivity and operation measured, by 2
-// (4096^2, h-dome: 403 -> 204 us) to 26 times (holes filled: 2.67 -> 0.104 ms),
-// so there is no size below or above which the other is chosen.
+// engine and what it installs applies there, but a call stays where it was.
+// No size decides: on noise with blobs the merging engine was faster at every size,
+// marker, connectivity and operation measured, by 2 (4096^2, h-dome: 403 -> 203 us)
+// to 26 times (holes filled: 2.67 -> 0.104 ms). The contents, which the host does not
+// know, can favour the wavefront: an empty marker, which leaves it nothing to
+// propagate (4096^2: 137 us there, 319 here), or a dithered mask, whose blocks
+// overflow their pass lists, under an h-dome marker (275 and 615).
 static bool use_forest(const recon_ctx *c)
 {
     return c->ask_bh == 128 && c->ask_k == 1 && c->grid == 0 && c->ask_bands == 4 && c->use_tma == 1 &&
@@ -870,7 +873,7 @@ extern "C" int recon_get_work(recon_ctx *c, recon_work *out, int n)
     CK(cudaStreamSynchronize(c->stream));
     if (n == 0) return RECON_OK;
     std::vector<rk::Work> w(n);
-    if (c->host_whole) std::copy(c->h_work, c->h_work + n, w.begin());
+    if (c->host_whole) std::copy(c->host_work.begin(), c->host_work.begin() + n, w.begin());
     else CK(cudaMemcpy(w.data(), c->last_work, sizeof(rk::Work) * n, cudaMemcpyDeviceToHost));
     for (int i = 0; i < n; ++i) {
         out[i].visits = w[i].visits;
@@ -919,7 +922,6 @@ static int ensure_pipeline(recon_ctx *c)
         for (cudaEvent_t &e : c->ev_seg[s])
             if (!e) CK(cudaEventCreate(&e));
     }
-    if (!c->h_seg_ctl) CK(cudaMallocHost((void **)&c->h_seg_ctl, sizeof(rk::Ctl) * HOST_SEGMENTS));
     return RECON_OK;
 }
 
@@ -974,13 +976,20 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
     // A batch this small would be one launch on the wavefront engine; cut up, it still reports as one: the counters
     // of all tiles, the kernel time of all segments, and a violation does not keep the other tiles from running.
     const bool whole = nseg > 1 && total < HOST_SEGMENT_MIN_WAVEFRONT;
-    if (whole && c->cap_hwork < (size_t)n) {
-        if (c->h_work) cudaFreeHost(c->h_work);
-        c->h_work = nullptr;
-        c->cap_hwork = 0;
-        c->host_whole = c->last_n = 0;   // the call before may have its counters there
-        CK(cudaMallocHost((void **)&c->h_work, sizeof(rk::Work) * (size_t)n));
-        c->cap_hwork = (size_t)n;
+    // a segment's place in h_seg: control word, room for the tiles' statuses that follow it on the device, counters
+    size_t seg_off[HOST_SEGMENTS], work_off[HOST_SEGMENTS], seg_bytes = 0;
+    for (int s = 0; s < nseg; ++s) {
+        const size_t ns = seg_end[s] - (s ? seg_end[s - 1] : 0);
+        seg_off[s] = seg_bytes;
+        work_off[s] = align_up(sizeof(rk::Ctl), 16) + align_up(sizeof(int) * ns, 16);
+        seg_bytes += work_off[s] + (whole ? align_up(sizeof(rk::Work) * ns, 16) : 0);
+    }
+    if (c->cap_hseg < seg_bytes) {
+        if (c->h_seg) cudaFreeHost(c->h_seg);
+        c->h_seg = nullptr;
+        c->cap_hseg = 0;
+        CK(cudaMallocHost((void **)&c->h_seg, seg_bytes));
+        c->cap_hseg = seg_bytes;
     }
     auto first = [&](int s) { return s ? seg_end[s - 1] : 0; };
     auto queue_inputs = [&](int s) -> int {
@@ -1027,9 +1036,15 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
         if (whole) own_events();
         if (brc != RECON_OK) return brc;
         ++ran;
-        if (whole)
-            CK(cudaMemcpyAsync(c->h_work + t0, c->last_work, sizeof(rk::Work) * (size_t)ns, cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaMemcpyAsync(&c->h_seg_ctl[s], c->last_ctl, sizeof(rk::Ctl), cudaMemcpyDeviceToHost, c->stream));
+        // (the merging engine's counters lie behind the control word in the same buffer: one copy)
+        const bool together = whole && c->last_ctl != c->d_ctl;
+        const size_t wb = whole ? sizeof(rk::Work) * (size_t)ns : 0;
+        const size_t gap = together ? (size_t)((unsigned char *)c->last_work - (unsigned char *)c->last_ctl) : 0;
+        CK(cudaMemcpyAsync(c->h_seg + seg_off[s], c->last_ctl, together ? gap + wb : sizeof(rk::Ctl),
+                           cudaMemcpyDeviceToHost, c->stream));
+        if (together) work_off[s] = gap;   // (at most what was set aside)
+        else if (whole)
+            CK(cudaMemcpyAsync(c->h_seg + seg_off[s] + work_off[s], c->last_work, wb, cudaMemcpyDeviceToHost, c->stream));
         CK(cudaEventRecord(c->ev_out[s], c->stream));
         return RECON_OK;
     };
@@ -1044,7 +1059,7 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
         if (rc != RECON_OK) break;
         cudaError_t e = cudaEventSynchronize(c->ev_out[s]);
         if (e != cudaSuccess) { rc = cuda_status(e); break; }
-        const rk::Ctl &h = c->h_seg_ctl[s];
+        const rk::Ctl &h = *(const rk::Ctl *)(c->h_seg + seg_off[s]);
         // a segment failed: its results and those of the segments behind it stay on the device
         if ((h.abort || h.err_tile != INT_MAX) && failed == RECON_OK) {
             abort_code = h.abort;
@@ -1064,7 +1079,10 @@ extern "C" int recon_batch_host(recon_ctx *c, const recon_tile *tiles, int n)
     if (whole) {
         c->last_n = ran == nseg ? n : 0;
         c->host_ms = 0.0f;
+        c->host_work.resize(n);
         for (int s = 0; s < ran; ++s) {
+            memcpy(c->host_work.data() + first(s), c->h_seg + seg_off[s] + work_off[s],
+                   sizeof(rk::Work) * (size_t)(seg_end[s] - first(s)));
             float ms = 0.0f;
             if (cudaEventElapsedTime(&ms, c->ev_seg[s][0], c->ev_seg[s][1]) == cudaSuccess) c->host_ms += ms;
         }

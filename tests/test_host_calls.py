@@ -277,3 +277,18 @@ def test_training_without_the_cluster_takes_the_same_steps(rc, n, batch):
     assert list(steps) == list(range(1, 4 * per + 1))
     rc.recon_free(c)
     assert rc.lib().ht_faults() == 0
+
+
+def test_a_host_batch_in_segments_without_scratch_for_the_merging_engine(rc):
+    """The wavefront engine takes over segment by segment; its control word and its
+    counters lie in buffers of their own."""
+    c = rc.recon_init(0, 0, 0)
+    tiles = [tile(64 * (20 + k), 1700) for k in range(5)]
+    px = sum(I.size for I, _, _ in tiles)
+    rc.lib().ht_device_limit(rc.lib().ht_device_bytes() + 2 * px + (3 << 20))
+    assert rc.recon_batch_host(c, [t[2] for t in tiles]) == rc.RECON_OK and done(tiles)
+    assert host_runtime.counts(rc)["wavefront"] == 4 and host_runtime.counts(rc)["merging"] == 0
+    assert [w["scan_rows"] for w in rc.recon_get_work(c, 5)] == [64 * (20 + k) for k in range(5)]
+    assert rc.recon_last_kernel_ms(c) == pytest.approx(1e-6 * px, rel=1e-5)
+    rc.recon_free(c)
+    assert rc.lib().ht_faults() == 0
