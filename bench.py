@@ -755,8 +755,8 @@ def main():
     if args.autotune:
         st, tuned = rc.recon_autotune(ctx, desc, 2)
         rc.check(st, "recon_autotune")
-        for key, val in zip((rc.RECON_P_BLOCK_H, rc.RECON_P_BANDS, rc.RECON_P_SWEEPS, rc.RECON_P_SCAN_GAIN), tuned):
-            rc.check(rc.recon_set_param(ctx, key, val))   # asks for the wavefront engine, unless they are the defaults
+        # the grid as it is, but asked for: the tuned settings are the wavefront engine's
+        rc.check(rc.recon_set_param(ctx, rc.RECON_P_GRID, rc.recon_get_param(ctx, rc.RECON_P_GRID)))
     settings = {"block_h": rc.recon_get_param(ctx, rc.RECON_P_BLOCK_H),
                 "bands": rc.recon_get_param(ctx, rc.RECON_P_BANDS),
                 "scan_pairs": rc.recon_get_param(ctx, rc.RECON_P_SWEEPS),
