@@ -109,8 +109,8 @@ typedef struct {
  * Returns RECON_OK and *ctx, or an error code with *ctx = NULL. */
 int recon_init(recon_ctx **ctx, int device, void *cuda_stream, unsigned flags);
 
-/* Reconstructs one tile (Table II; Algorithm 1 with the hybrid scan + queue
- * schedule of Sec. V-C). I, J: device pointers, pitch = W. J <- R in place. */
+/* Reconstructs one tile (Table II; on the wavefront engine by Algorithm 1 with
+ * the hybrid scan + queue schedule of Sec. V-C). I, J: device pointers, pitch = W. J <- R in place. */
 int recon_run(recon_ctx *ctx, const uint8_t *I, uint8_t *J, int H, int W, int conn);
 
 /* recon_run for any operation: op = RECON_OP_DILATE, RECON_OP_ERODE (J >= I,
@@ -118,8 +118,9 @@ int recon_run(recon_ctx *ctx, const uint8_t *I, uint8_t *J, int H, int W, int co
  * J need not be initialised). Device pointers, pitch = W. */
 int recon_run_op(recon_ctx *ctx, const uint8_t *I, uint8_t *J, int H, int W, int conn, int op);
 
-/* Reconstructs n independent tiles of any sizes in one persistent launch
- * (tiles are processed concurrently, as the 4K x 4K tiles of Sec. V are).
+/* Reconstructs n independent tiles of any sizes in one call (tiles are processed
+ * concurrently, as the 4K x 4K tiles of Sec. V are: in one persistent launch on
+ * the wavefront engine, in groups of up to 268 Mpx on the merging engine).
  * `tiles` is a HOST array of n descriptors with device image pointers.
  * Tiles must not overlap in memory. With RECON_FLAG_LEARNED the cost model
  * chooses each tile's variant and the packing order when the wavefront engine
@@ -210,9 +211,10 @@ int64_t recon_get_param(recon_ctx *ctx, int key);
 
 /* Work counters of one tile in the last call (propagation work measured by
  * the method itself: what the cost model learns from). The merging engine
- * reports visits (blocks of 64 x 64 pixels), seeds (basins of the mask), levels
- * (merging rounds, summed over the blocks), busy_ns and, in phase_ns: load,
- * basins, passes, rounds, results, 0. */
+ * reports visits (blocks of 64 x 64 pixels), seeds (basins of the mask), pops
+ * (passes between basins), levels (merging rounds, summed over the blocks),
+ * busy_ns and, in phase_ns: load, basins, passes, rounds, results, 0; scan_rows
+ * is 0. */
 typedef struct {
     uint64_t visits;      /* block visits (first visits + revisits after a halo change) */
     uint64_t scan_rows;   /* rows processed by raster / anti-raster scans */
@@ -236,8 +238,8 @@ int recon_trace(recon_ctx *ctx, unsigned *out, int n);
 /* Copies the counters of the last call's first n tiles into out[] (syncs). */
 int recon_get_work(recon_ctx *ctx, recon_work *out, int n);
 
-/* Device time of the last call's persistent kernel in ms (CUDA events on the
- * context's stream; syncs). */
+/* Device time of the last call's persistent kernel, or of the merging engine's
+ * kernels, in ms (CUDA events on the context's stream; syncs). */
 int recon_last_kernel_ms(recon_ctx *ctx, float *ms);
 
 

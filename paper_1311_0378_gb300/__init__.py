@@ -194,6 +194,10 @@ def recon_get_param(ctx, key: int) -> int:
 
 
 def recon_get_work(ctx, n: int):
+    """Work counters of the last call's first n tiles, one dict a tile. The names of
+    phase_ns are the wavefront engine's phases; the merging engine, which runs with
+    default settings, fills them, in this order, with the time it takes to load, to
+    find basins, to list passes, for its rounds and to write results, and 0."""
     out = (recon_work * max(n, 1))()
     rc = lib().recon_get_work(ctx, out, n)
     if rc != RECON_OK:
@@ -365,8 +369,8 @@ def context_for(device, stream=None, flags: int = RECON_FLAG_SYNC):
 
 
 def run(I, J, conn: int = 8, op: int = RECON_OP_DILATE, ctx=None):
-    """Reconstructs J in place under I (Table II; Algorithm 1 with the hybrid
-    scan + queue schedule of Sec. V-C) and returns J. I, J: contiguous uint8
+    """Reconstructs J in place under I (Table II; the fixed point of Algorithm 1)
+    and returns J. I, J: contiguous uint8
     CUDA tensors of shape (H, W); op: RECON_OP_DILATE (J <= I), RECON_OP_ERODE
     (J >= I) or RECON_OP_FILL_HOLES (J receives FillHoles(I)). Runs on torch's
     current stream unless `ctx` is given; raises ReconError on failure."""

@@ -17,7 +17,10 @@ Pipeline (every step on the GPU goes through the C ABI):
   4. training: recon_mlp_train (the library's forward / backward / Adam
      kernels) on standardised targets;
   5. the weights, target normalisation and variant ids go to a small file that
-     recon_sched_set_model installs for RECON_FLAG_LEARNED batches.
+     recon_sched_set_model installs for RECON_FLAG_LEARNED batches that run on
+     the wavefront engine (a context with one of its settings changed, or the
+     plan passed to recon_batch_ex). A call on default settings runs on the
+     merging engine, which has no schedule: there the model changes nothing.
 The model never touches pixel values: it only picks each tile's variant and
 the packing order (decreasing predicted cost).
 """

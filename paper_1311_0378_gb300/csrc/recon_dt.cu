@@ -12,7 +12,7 @@
 //   column_kernel  signed distance to the nearest background row of the column,
 //                  by bit scans of the column's words (16 bits a pixel)
 //   row_kernel     a row of squared column distances in shared memory; each
-//                  pixel searches outwards until dx^2 reaches its best, past 32
+//                  pixel searches outwards until dx^2 reaches its best, past 128
 //                  columns in runs of 32 that a run's minimum can rule out
 //
 // The work per pixel is a few bit operations plus about two instructions per
@@ -39,8 +39,8 @@ constexpr int WMAX = 32768;             // widest row
 constexpr int PAD = 128;                // columns of INF at both ends of a row in shared memory
 
 // A kernel may be launched when the last CTAs of the one before it run, and
-// waits for all of that one's results before it reads any: 145 -> 141 and 40 ->
-// 35 us a call on the two masks above.
+// waits for all of that one's results before it reads any: 4 and 5 us of a call on
+// the two masks above.
 __device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -260,7 +260,7 @@ __device__ __forceinline__ void search_far(int x, int W, const uint32_t *low, Ta
 // Distances only. Two neighbouring pixels a thread: a pair of columns (one
 // 64-bit load) gives each of them two candidates, one add-and-min instruction
 // each, so a column costs 1.5 instructions a pixel and side (one pixel a thread
-// with 32-bit loads: 314 us for the 4096^2 mask's call instead of 165).
+// with 32-bit loads nearly doubles the 4096^2 mask's call).
 __global__ void row_kernel(const uint16_t *G, int H, int W, int pitch, unsigned *d2)
 {
     extern __shared__ __align__(16) uint32_t dt_smem[];

@@ -37,10 +37,9 @@
 // block_kernel takes most of it (0.195 of 0.235 ms of kernel time on the
 // border-seeded tile) and is bound by instruction issue and the shared-memory
 // pipe (about 65% and 55%; DRAM below 4%), so what counts is warp instructions
-// a block: 25 200 (h-dome) to 35 000 (border), 76 500 and 94 900 at first.
-// Saddles instead of all pixel pairs, arcs and targets of four pixels at once in
-// byte lanes, loops rolled to fit the instruction cache, and lists that stay
-// dense made the difference.
+// a block, 25 200 (h-dome) to 35 000 (border): hence saddles instead of all pixel
+// pairs, arcs and targets of four pixels at once in byte lanes, loops rolled to
+// fit the instruction cache, and lists that stay dense.
 #include <climits>
 #include <cstddef>
 #include "recon_check.h"
@@ -98,8 +97,8 @@ __device__ __forceinline__ unsigned long long now_ns()
 
 // The next kernel of a group may be launched while this one still runs (its
 // CTAs fill the places that the last CTAs leave free); it waits for all of this
-// one's results before it reads any. 512^2: 78 -> 74 us a call; the 910 Mpx batch
-// 10.95 -> 10.83 ms of kernel time.
+// one's results before it reads any: 4 us of a call on 512^2, 1% of the 910 Mpx
+// batch's kernel time.
 __device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -360,10 +359,9 @@ __device__ __noinline__ void each_pair(Smem<CONN> &S, F f)
 }
 
 // Five CTAs an SM where shared memory allows it (8-connectivity: 43 KB; 4: 56 KB
-// for twice the basins), in 48 registers without spills: with the timers and the tile's
-// record in registers instead of shared memory there were spills, 10.95 instead of
-// 10.40 ms of kernel time on the 910 Mpx batch when that was done, with four CTAs
-// 11.13.
+// for twice the basins), in 48 registers without spills, for which the timers and the
+// tile's record are in shared memory: 5% of the 910 Mpx batch's kernel time against
+// five CTAs with spills, 7% against four.
 template <int CONN>
 __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __grid_constant__ Params P)
 {
@@ -477,9 +475,8 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     // Basins: every pixel points to the first upper neighbour of its first arc
     // (its heaviest edges all weigh its own height); pixels without one are tops.
     // A lane takes a word of four pixels in each of four rows: 4.5 loads and a
-    // quarter of a warp's scan a word instead of 9 and one (10 500 instructions
-    // a block with a row each and the labels pixel by pixel; on the 910 Mpx
-    // batch 10.40 -> 9.54 ms of kernel time).
+    // quarter of a warp's scan a word instead of the 9 and one that a row each
+    // takes (8% of the 910 Mpx batch's kernel time).
     {
         constexpr int RL = BS / (NT / 16);
         const int row = RL * (2 * warp + (lane >> 4)), cw = lane & 15;
@@ -616,9 +613,9 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
     }
     __syncthreads();
     if (tid == 0) S.tick[2] = now_ns();
-    // Maxima are taken without a look at the present one first: on the 910 Mpx
-    // batch the load and the compare cost more than the reductions they saved
-    // (9.39 -> 8.84 ms of kernel time).
+    // Maxima are taken without a look at the present one first: the load and the
+    // compare cost more than the reductions they save (6% of the 910 Mpx batch's
+    // kernel time).
     auto offer = [&](unsigned a, uint32_t key) {
         if (RK_CHECK(a < nb, CK_BASIN)) atomicMax(&S.best[a], key);
     };
@@ -919,12 +916,12 @@ __global__ void __launch_bounds__(NT, CONN == 8 ? 5 : 4) block_kernel(const __gr
 
 // Joins across block borders: a CTA of 128 threads handles the edges from its
 // block's right column (warps 0, 1) and bottom row (warps 2, 3) to the blocks
-// E, NE, SE and S, SW of it (the other diagonals belong to those blocks). Bound
-// by the latency of dependent loads (walks are 1 to 6 links long on average, L2
-// accesses each), so everything before the walks takes two, and a lane whose
-// neighbour holds the same two nodes with a heavier edge leaves it to that lane.
-// 20 us on a 4096^2 h-dome tile, 27 us seeded from the border (34 and 40 us with a
-// search for the tile first and a warp-wide match and maximum before each join).
+// E, NE, SE and S of it (the edges of its corners to NW and SW are the SE and NE
+// edges of the blocks there). Bound by the latency of dependent loads (walks are 1
+// to 6 links long on average, L2 accesses each), so everything before the walks
+// takes two, and a lane whose neighbour holds the same two nodes with a heavier
+// edge leaves it to that lane.
+// 20 us on a 4096^2 h-dome tile, 27 us seeded from the border.
 template <int CONN>
 __global__ void __launch_bounds__(128) rim_kernel(const __grid_constant__ Params P)
 {
