@@ -106,6 +106,7 @@ struct recon_ctx {
 static int cuda_status(cudaError_t e)
 {
     if (e == cudaSuccess) return RECON_OK;
+    cudaGetLastError();   // reported here: the check after the next launch is not to find it again
     if (e == cudaErrorMemoryAllocation) return RECON_ENOMEM;
     return RECON_ECUDA;
 }
@@ -122,7 +123,6 @@ static int grow(T **p, size_t *cap, size_t need)
     size_t n = std::max(need, (size_t)1);
     const cudaError_t e = cudaMalloc((void **)p, n * sizeof(T));
     if (e != cudaSuccess) {
-        cudaGetLastError();   // an allocation failure leaves the context usable: clear it
         *p = nullptr;
         return cuda_status(e);
     }

@@ -36,7 +36,8 @@ namespace {
 std::deque<std::function<void()>> queue;
 size_t queued = 0, done = 0;             // operations so far; the queue holds done + 1 .. queued
 std::map<unsigned char *, size_t> live, dead;
-size_t dev_bytes = 0, dev_limit = SIZE_MAX;
+size_t dev_bytes = 0, dev_limit = SIZE_MAX, pinned_limit = SIZE_MAX;
+cudaError_t last_error = cudaSuccess;
 std::map<unsigned char *, size_t> dev;   // sizes of device allocations
 int faults = 0;
 int broken = 0;                          // waits for a stream under capture
@@ -130,6 +131,7 @@ extern "C" int ht_faults() { return faults; }
 extern "C" int ht_broken_captures() { return broken; }
 extern "C" int ht_graph_nodes(cudaGraph_t g) { return (int)g->ops.size(); }
 extern "C" void ht_device_limit(size_t bytes) { dev_limit = bytes; }
+extern "C" void ht_pinned_limit(size_t bytes) { pinned_limit = bytes; }   // of one allocation
 extern "C" size_t ht_device_bytes() { return dev_bytes; }
 extern "C" void ht_counts(int *out)
 {
@@ -152,7 +154,12 @@ extern "C" void ht_train_fits(int yes) { fits = yes; }
 extern "C" {
 cudaError_t cudaGetDeviceCount(int *n) { *n = 1; return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError()
+{
+    const cudaError_t e = last_error;
+    last_error = cudaSuccess;
+    return e;
+}
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { *v = 4; return cudaSuccess; }
 cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **, unsigned, unsigned long long,
                                              cudaDriverEntryPointQueryResult *)
@@ -161,7 +168,7 @@ cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **, unsigned, un
 }
 cudaError_t cudaMalloc(void **p, size_t n)
 {
-    if (dev_bytes + n > dev_limit) return cudaErrorMemoryAllocation;
+    if (dev_bytes + n > dev_limit) return last_error = cudaErrorMemoryAllocation;
     *p = alloc(n);
     dev[(unsigned char *)*p] = n;
     dev_bytes += n;
@@ -178,7 +185,12 @@ cudaError_t cudaFree(void *p)
     release(p);
     return cudaSuccess;
 }
-cudaError_t cudaMallocHost(void **p, size_t n) { *p = alloc(n); return cudaSuccess; }
+cudaError_t cudaMallocHost(void **p, size_t n)
+{
+    if (n > pinned_limit) return last_error = cudaErrorMemoryAllocation;
+    *p = alloc(n);
+    return cudaSuccess;
+}
 cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { *p = alloc(n); return cudaSuccess; }
 cudaError_t cudaFreeHost(void *p) { release(p); return cudaSuccess; }
 cudaError_t cudaHostGetDevicePointer(void **d, void *h, unsigned) { *d = h; return cudaSuccess; }
@@ -317,7 +329,7 @@ cudaError_t rf_launch(int, const rf::Params *Pp, cudaStream_t st)
             P.work[d.index].visits += (unsigned long long)d.nbx * d.nby;
         }
     });
-    return cudaSuccess;
+    return cudaGetLastError();   // as after a launch
 }
 }
 
@@ -364,7 +376,7 @@ cudaError_t rl_train_epoch(float *, float *, float *, const float *, const float
         orders.insert(orders.end(), idx, idx + n);
         *loss += 1.0f;
     });
-    return cudaSuccess;
+    return cudaGetLastError();
 }
 size_t dt_scratch_bytes(int H, int W) { return (size_t)H * W; }
 int dt_run(const uint8_t *, int, int, int *, unsigned *, void *, unsigned, int, cudaStream_t) { return DT_OK; }

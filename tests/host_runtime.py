@@ -38,7 +38,7 @@ def load(tmp_path):
     spec.loader.exec_module(m)
     m.LIB_PATH = lib
     L = m.lib()
-    L.ht_device_limit.argtypes = [ctypes.c_size_t]
+    L.ht_device_limit.argtypes = L.ht_pinned_limit.argtypes = [ctypes.c_size_t]
     L.ht_device_bytes.restype = ctypes.c_size_t
     return m
 

@@ -292,3 +292,22 @@ def test_a_host_batch_in_segments_without_scratch_for_the_merging_engine(rc):
     assert rc.recon_last_kernel_ms(c) == pytest.approx(1e-6 * px, rel=1e-5)
     rc.recon_free(c)
     assert rc.lib().ht_faults() == 0
+
+
+def test_a_failed_pinned_allocation_is_reported_once(rc):
+    """Its error must not show again in the check after the next launch."""
+    c = rc.recon_init(0, 0, rc.RECON_FLAG_SYNC)
+    few, many = [tile(5, 5) for _ in range(2)], [tile(2, 2) for _ in range(2000)]
+    a, X = np.zeros(3 * rc.RECON_MLP_NPARAMS, np.float32), np.zeros((5000, 22), np.float32)
+
+    def train(n):
+        return rc.recon_mlp_train(c, a.ctypes.data, X.ctypes.data, X.ctypes.data, n, 2, 10, 1e-3)[0]
+    rc.lib().ht_pinned_limit(1 << 12)
+    assert rc.recon_batch(c, [t[2] for t in many]) == rc.RECON_ENOMEM
+    assert rc.recon_batch(c, [t[2] for t in few]) == rc.RECON_OK and done(few)
+    assert train(5000) == rc.RECON_ENOMEM and train(20) == rc.RECON_OK
+    rc.lib().ht_pinned_limit(1 << 40)
+    assert rc.recon_batch(c, [t[2] for t in many]) == rc.RECON_OK and done(many)
+    assert train(5000) == rc.RECON_OK
+    rc.recon_free(c)
+    assert rc.lib().ht_faults() == 0
